@@ -184,7 +184,11 @@ struct lbvh_tree_s {
     DevBuf keys[2], vals[2];
     DevBuf nodes, store, lookback, hist, partials, bounds, ctl;
     DevBuf pend;  // climbs handed from the construct to its second kernel (zeroed, kept zero)
-    DevBuf counts, tile_sums, overflow, slots, spill_head, spill;
+    DevBuf counts, tile_sums, overflow, slots, spill_head, spill, sparse;
+    DevBuf packed;             // boxes of the leaf blocks (packet.cu), made by the first query that walks them
+    bool packed_ok = false;    // `packed` belongs to the present leaves
+    bool few_seen = false;     // few queries have come since the leaves changed (see query_count)
+    bool loaded = false;       // a checkpoint's tree: walked by Algorithm 1, which checks its links
     DevBuf qkeys[2], qvals[2], qlookback;  // Morton order of the queries
     DevBuf vscratch;                       // scratch of the Karras / Apetrei builds
     // lbvh_query_into_host: device staging of two chunks' CSR, the stream
@@ -330,19 +334,26 @@ constexpr int64_t kOrderMinQueries = 2048;  // below this, walk in input order
 // walk time than the pass saves; order changes speed only. Batches use 30.
 constexpr int order_bits() { return 30; }
 
+// The queries are the primitives of the last build (same pointer and count):
+// the build's permutation is their order.
+bool own_order(lbvh_tree_t t, const lbvh::QueryArgs &qa) {
+    const bool same_points = qa.qkind == LBVH_Q_SPHERE && t->kind == LBVH_PRIM_POINTS;
+    const bool same_boxes = qa.qkind == LBVH_Q_BOX && t->kind == LBVH_PRIM_BOXES;
+    return t->n > 0 && qa.queries == t->prims_ptr && qa.nq == t->n && (same_points || same_boxes);
+}
+
 // The order in which threads take the queries: the Morton order of the query
 // centres inside the tree's bounds (encode + radix sort of `bits`-bit codes,
 // the build's own kernels). Queries that are the primitives of the last build
 // (same pointer and count) reuse the build's permutation. Order only changes
 // speed, never results.
-lbvh_status query_order(lbvh_tree_t t, lbvh::QueryArgs &qa, cudaStream_t s, int bits = order_bits()) {
+lbvh_status query_order(lbvh_tree_t t, lbvh::QueryArgs &qa, cudaStream_t s, int bits = order_bits(),
+                        lbvh::CodeLayout curve = lbvh::kCodeLow) {
     using namespace lbvh;
     qa.order = nullptr;
     // rays are walked in the caller's order (a camera's rays are coherent as given)
     if (qa.nq < kOrderMinQueries || t->n == 0 || qa.qkind == LBVH_Q_RAY) return LBVH_OK;
-    const bool same_points = qa.qkind == LBVH_Q_SPHERE && t->kind == LBVH_PRIM_POINTS;
-    const bool same_boxes = qa.qkind == LBVH_Q_BOX && t->kind == LBVH_PRIM_BOXES;
-    if (qa.queries == t->prims_ptr && qa.nq == t->n && (same_points || same_boxes)) {
+    if (own_order(t, qa)) {
         qa.order = t->perm();
         return LBVH_OK;
     }
@@ -354,10 +365,12 @@ lbvh_status query_order(lbvh_tree_t t, lbvh::QueryArgs &qa, cudaStream_t s, int 
         LBVH_CUDA(t->qvals[k].ensure(unq * 4, s));
     }
     LBVH_CUDA(t->qlookback.ensure((size_t)sort_tiles_max(qa.nq) * kRadix * 4 * 2, s));
+    // a Hilbert order of 30 bits takes the whole four bytes: 11 levels of the curve but for the last bit
+    const bool whole = curve == kCodeHilbert && bits == 30;
     LBVH_CUDA(cudaMemsetAsync(t->hist.p, 0, (size_t)sort_passes(bits) * kRadix * 4, s));
     const int as_prims = qa.qkind == LBVH_Q_SPHERE ? LBVH_PRIM_POINTS : LBVH_PRIM_BOXES;
-    launch_encode(qa.queries, qa.nq, as_prims, bits, t->bounds.as<float>(), t->qkeys[0].as<uint64_t>(),
-                  t->hist.as<uint32_t>(), 1, kCodeLow, 0, s);
+    launch_encode(qa.queries, qa.nq, as_prims, whole ? 33 : bits, t->bounds.as<float>(), t->qkeys[0].as<uint64_t>(),
+                  t->hist.as<uint32_t>(), 1, curve, whole ? 1 : 0, s);
     LBVH_LAUNCHED();
     SortScratch scratch{t->hist.as<uint32_t>(), t->qlookback.as<uint32_t>(), sort_tiles_max(qa.nq) * kRadix};
     qa.order = run_index_sort(t->qkeys[0].as<uint64_t>(), t->qkeys[1].as<uint64_t>(), t->qvals[0].as<uint32_t>(),
@@ -369,7 +382,7 @@ lbvh_status query_order(lbvh_tree_t t, lbvh::QueryArgs &qa, cudaStream_t s, int 
 lbvh::QueryScratch query_scratch(lbvh_tree_t t) {
     return lbvh::QueryScratch{t->counts.as<uint32_t>(), t->slots.as<uint32_t>(), t->overflow.as<uint32_t>(),
                               t->spill_head.as<uint32_t>(), t->spill.as<uint32_t>(),
-                              lbvh::spill_chunks_for(t->spill_nq)};
+                              lbvh::spill_chunks_for(t->spill_nq), t->sparse.as<uint2>()};
 }
 
 // The query up to the hit count: order, collecting walk, scan; synchronises `s`.
@@ -392,13 +405,36 @@ lbvh_status query_count(lbvh_tree_t t, lbvh::QueryArgs &qa, int64_t *d_offsets,
     t->prof.clear(LBVH_STAGE_QCOUNT, LBVH_STAGE_QORDER + 1);
     const int choice = t->walk_choice >= 0 ? t->walk_choice : tune_walk_choice(t->n, t->bits, t->kind, qa.qkind, 1);
     qa.walk = walk_choice_kind(choice);
+    // spheres and boxes walk the leaf blocks unless the tuner chose a walk of the nodes
+    RangeWalk how = kRangeNodes;
+    if (qa.walk == kWalkThread && qa.qkind != LBVH_Q_RAY && t->n > 0 && !t->loaded)
+        how = range_walk(qa.nq, t->n, own_order(t, qa));
+    // few queries on a large tree whose blocks nobody has packed: the second such call packs them
+    // (0.2 ms at 2^25 leaves, about what a call saves), so a tree that is queried once never pays
+    if (how == kRangeSparse && !t->packed_ok && t->n > kPackForFew && !t->few_seen) {
+        t->few_seen = true;
+        how = kRangeNodes;
+    }
     t->prof.begin(LBVH_STAGE_QORDER, s);
-    lbvh_status ost = query_order(t, qa, s, walk_choice_order_bits(choice));
+    lbvh_status ost = LBVH_OK;
+    if (how != kRangeSparse || own_order(t, qa))
+        ost = query_order(t, qa, s, walk_choice_order_bits(choice), how == kRangePackets ? kCodeHilbert : kCodeLow);
     t->prof.end(LBVH_STAGE_QORDER, s);
     if (ost != LBVH_OK) return ost;
+    bool pack = false;
+    if (how != kRangeNodes) {
+        LBVH_CUDA(t->sparse.ensure((unq / 32 + 1) * sizeof(uint2), s));
+        pack = !t->packed_ok;
+        if (pack) LBVH_CUDA(t->packed.ensure((size_t)pack_records(t->n) * 32, s));
+    }
     const QueryScratch qs = query_scratch(t);
     t->prof.begin(LBVH_STAGE_QCOUNT, s);
-    launch_query_collect(t->view(), qa, qs, c, s);
+    if (how != kRangeNodes) {
+        if (pack) launch_pack(t->view(), t->packed.as<float4>(), c, s);
+        launch_query_packets(t->view(), t->packed.as<float4>(), qa, qs, how, c, s);
+    } else {
+        launch_query_collect(t->view(), qa, qs, c, s);
+    }
     t->prof.end(LBVH_STAGE_QCOUNT, s);
     LBVH_LAUNCHED();
     t->prof.begin(LBVH_STAGE_QSCAN, s);
@@ -407,6 +443,7 @@ lbvh_status query_count(lbvh_tree_t t, lbvh::QueryArgs &qa, int64_t *d_offsets,
     LBVH_LAUNCHED();
     lbvh_status st = read_control(t, s);
     if (st != LBVH_OK) return st;
+    if (pack) t->packed_ok = true;  // complete: the stream has been synchronised
     st = flags_status(t->h_ctl->build_flags);
     if (st == LBVH_OK) st = flags_status(t->h_ctl->query_flags);
     *total = t->h_ctl->total;
@@ -478,15 +515,15 @@ struct lbvh_batch_s {
     int64_t count = 0, N = 0, NQ = 0, nchunks = 0, nqchunks = 0;
     int passes = 0, qpasses = 0, sort_variant = -1;
     bool self_query = false, sorted_in_b = false;
-    DevBuf prim_off, query_off, node_start, store_start, chunks, chunk_first, qchunks;
+    DevBuf prim_off, query_off, node_start, store_start, pack_start, chunks, chunk_first, qchunks;
     DevBuf keys[2], vals[2], nodes, store, lookback, hist, partials, bounds, ctl;
-    DevBuf counts, slots, overflow, tile_sums, qkeys[2], qvals[2], qlookback, spill_head, spill;
+    DevBuf counts, slots, overflow, tile_sums, qkeys[2], qvals[2], qlookback, spill_head, spill, sparse, packed;
     // Segmented-sort tile tables: row r (r < sort_variant_count(): that
     // variant; the last row: the default variant) holds count + 1 entries.
     DevBuf tile_first, qtile_first;
     std::vector<int64_t> h_tiles, h_qtiles;  // tiles per row
     int64_t max_tiles = 0, max_qtiles = 0;
-    std::vector<int64_t> h_node_start;
+    std::vector<int64_t> h_node_start, h_pack_start;
     lbvh::Control *h_ctl = nullptr;
     cudaGraphExec_t exec = nullptr;
     int graph_kernels = 0;
@@ -496,12 +533,15 @@ struct lbvh_batch_s {
 
     lbvh::BatchTables tables() const {
         return lbvh::BatchTables{prim_off.as<int64_t>(), query_off.as<int64_t>(), node_start.as<int64_t>(),
-                                 store_start.as<int64_t>(), chunks.as<lbvh::BatchChunk>(),
+                                 store_start.as<int64_t>(), pack_start.as<int64_t>(), chunks.as<lbvh::BatchChunk>(),
                                  chunk_first.as<int64_t>(), qchunks.as<lbvh::BatchChunk>(), (int)count,
                                  N, NQ, nchunks, nqchunks};
     }
     const uint64_t *sorted_codes() const { return keys[sorted_in_b ? 1 : 0].as<uint64_t>(); }
     const uint32_t *perm() const { return vals[sorted_in_b ? 1 : 0].as<uint32_t>(); }
+    // The queries walk in packets (as range_walk; few queries stay with
+    // Algorithm 1); the leaf blocks are packed then.
+    bool packets() const { return NQ > 0 && N > 0 && N <= 4 * NQ; }
     lbvh::Control *dctl() const { return ctl.as<lbvh::Control>(); }
     // Segments of the primitive (or query) sort for tile shape `variant`.
     lbvh::SortSegments segments(bool queries, int variant) const {
@@ -554,12 +594,14 @@ lbvh_status batch_setup(lbvh_batch_t b, cudaStream_t s) {
     const std::vector<BatchChunk> qchunks = make_chunks(g.query_off, nullptr);
     b->nchunks = (int64_t)chunks.size();
     b->nqchunks = (int64_t)qchunks.size();
-    std::vector<int64_t> node_start(b->count), store_start(b->count);
-    int64_t units = 0, words = 0;
+    std::vector<int64_t> node_start(b->count), store_start(b->count), pack_start(b->count);
+    int64_t units = 0, words = 0, records = 0;
     for (int64_t k = 0; k < b->count; ++k) {
         const int64_t n = g.prim_off[k + 1] - g.prim_off[k];
         node_start[k] = units;
         store_start[k] = words;
+        pack_start[k] = records;
+        records += pack_records(n);
         if (n > 0) {
             units += 2 * (n - 1) + (g.kind == LBVH_PRIM_POINTS ? n : 2 * n);
             units += units & 1;  // every tree starts on a 32-byte boundary (the walk loads 32-byte records)
@@ -567,6 +609,7 @@ lbvh_status batch_setup(lbvh_batch_t b, cudaStream_t s) {
         }
     }
     b->h_node_start = node_start;
+    b->h_pack_start = pack_start;
     // Tile tables of the segmented sorts, one row per tile shape.
     const int rows = sort_variant_count() + 1;
     std::vector<int64_t> tf((size_t)rows * (b->count + 1)), qtf((size_t)rows * (b->count + 1));
@@ -595,6 +638,7 @@ lbvh_status batch_setup(lbvh_batch_t b, cudaStream_t s) {
     if ((st = upload(b->query_off, g.query_off.data(), g.query_off.size() * 8, s)) != LBVH_OK) return st;
     if ((st = upload(b->node_start, node_start.data(), node_start.size() * 8, s)) != LBVH_OK) return st;
     if ((st = upload(b->store_start, store_start.data(), store_start.size() * 8, s)) != LBVH_OK) return st;
+    if ((st = upload(b->pack_start, pack_start.data(), pack_start.size() * 8, s)) != LBVH_OK) return st;
     if ((st = upload(b->chunks, chunks.data(), chunks.size() * sizeof(BatchChunk), s)) != LBVH_OK) return st;
     if ((st = upload(b->chunk_first, first.data(), first.size() * 8, s)) != LBVH_OK) return st;
     if ((st = upload(b->qchunks, qchunks.data(), qchunks.size() * sizeof(BatchChunk), s)) != LBVH_OK) return st;
@@ -607,6 +651,8 @@ lbvh_status batch_setup(lbvh_batch_t b, cudaStream_t s) {
         LBVH_CUDA(b->qvals[k].ensure(unq * 4 + 4, s));
     }
     LBVH_CUDA(b->nodes.ensure((size_t)units * 16 + 16, s));
+    LBVH_CUDA(b->packed.ensure((size_t)records * 32 + 32, s));
+    LBVH_CUDA(b->sparse.ensure(((size_t)b->NQ / 32 + 1) * sizeof(uint2), s));
     LBVH_CUDA(b->store.ensure((size_t)words * 8 + 8, s, true));
     LBVH_CUDA(b->lookback.ensure((size_t)b->max_tiles * kRadix * 8 + 8, s));
     LBVH_CUDA(b->qlookback.ensure((size_t)b->max_qtiles * kRadix * 8 + 8, s));
@@ -655,13 +701,14 @@ lbvh_status batch_enqueue(lbvh_batch_t b, cudaStream_t s) {
         return LBVH_OK;
     }
     QueryArgs qa{g.queries, b->NQ, g.qkind, g.radii, g.radius, nullptr};
+    const bool packets = b->packets();
     if (b->self_query) {
         qa.order = b->perm();
     } else {
         LBVH_CUDA(cudaMemsetAsync(b->hist.p, 0, (size_t)b->qpasses * b->count * kRadix * 4, s));
         const int as_prims = g.qkind == LBVH_Q_SPHERE ? LBVH_PRIM_POINTS : LBVH_PRIM_BOXES;
         launch_batch_encode(g.queries, as_prims, true, bt, order_bits(), b->bounds.as<float>(), b->qkeys[0].as<uint64_t>(),
-                            b->hist.as<uint32_t>(), s);
+                            b->hist.as<uint32_t>(), s, packets);
         SortScratch scratch{b->hist.as<uint32_t>(), b->qlookback.as<uint32_t>(), b->max_qtiles * kRadix};
         const SortSegments seg = b->segments(true, b->sort_variant);
         const bool in_b = run_onesweep(b->qkeys[0].as<uint64_t>(), b->qvals[0].as<uint32_t>(), true,
@@ -670,8 +717,13 @@ lbvh_status batch_enqueue(lbvh_batch_t b, cudaStream_t s) {
         qa.order = b->qvals[in_b ? 1 : 0].as<uint32_t>();
     }
     const QueryScratch qs{b->counts.as<uint32_t>(), b->slots.as<uint32_t>(), b->overflow.as<uint32_t>(),
-                          b->spill_head.as<uint32_t>(), b->spill.as<uint32_t>(), spill_chunks_for(b->NQ)};
-    launch_batch_collect(b->nodes.as<float4>(), g.kind, bt, qa, qs, c, s);
+                          b->spill_head.as<uint32_t>(), b->spill.as<uint32_t>(), spill_chunks_for(b->NQ), b->sparse.as<uint2>()};
+    if (packets) {
+        launch_batch_pack(b->nodes.as<float4>(), g.kind, bt, b->packed.as<float4>(), s);
+        launch_batch_packets(b->nodes.as<float4>(), g.kind, b->packed.as<float4>(), bt, qa, qs, c, s);
+    } else {
+        launch_batch_collect(b->nodes.as<float4>(), g.kind, bt, qa, qs, c, s);
+    }
     launch_exclusive_scan(qs.counts, b->NQ, g.offsets, b->tile_sums.as<int64_t>(), c, s);
     launch_query_copy_checked(qa, qs, g.offsets, g.hits, g.capacity, c, s);
     launch_batch_overflow(b->nodes.as<float4>(), g.kind, bt, qa, qs, c, g.offsets, g.hits, g.capacity, s);
@@ -754,7 +806,7 @@ void lbvh_tree_destroy(lbvh_tree_t t) {
                       &t->store, &t->pend, &t->lookback, &t->hist, &t->partials, &t->bounds, &t->ctl,
                       &t->counts, &t->tile_sums, &t->overflow, &t->qkeys[0], &t->qkeys[1],
                       &t->qvals[0], &t->qvals[1], &t->qlookback, &t->slots, &t->vscratch, &t->spill_head,
-                      &t->spill, &t->stage_off[0], &t->stage_off[1], &t->stage_hits[0], &t->stage_hits[1]})
+                      &t->spill, &t->sparse, &t->packed, &t->stage_off[0], &t->stage_off[1], &t->stage_hits[0], &t->stage_hits[1]})
         b->release(cudaStreamPerThread);
     pinned_controls().put(t->h_ctl);
     if (t->built) cudaEventDestroy(t->built);
@@ -787,6 +839,7 @@ lbvh_status build_impl(lbvh_tree_t t, const float *d_prims, int64_t n, int kind,
     t->kind = kind;
     t->bits = morton_bits;
     t->prims_ptr = d_prims;
+    t->packed_ok = t->few_seen = t->loaded = false;
     Control *c = t->dctl();
     LBVH_CUDA(cudaMemsetAsync(&c->build_flags, 0, sizeof(uint32_t), s));
     if (t->store_dirty && t->store.bytes) {
@@ -894,6 +947,7 @@ lbvh_status lbvh_build_from_sorted(lbvh_tree_t t, const uint64_t *d_sorted_codes
     t->kind = kind;
     t->bits = 0;
     t->prims_ptr = d_prims;
+    t->packed_ok = t->few_seen = t->loaded = false;
     t->codes_in = t->perm_in = 0;
     Control *c = t->dctl();
     LBVH_CUDA(cudaMemsetAsync(&c->build_flags, 0, sizeof(uint32_t), s));
@@ -923,6 +977,7 @@ lbvh_status lbvh_refit(lbvh_tree_t t, const float *d_prims, lbvh_stream_t stream
     LBVH_CUDA(cudaStreamWaitEvent(s, t->built, 0));
     if (t->queried) LBVH_CUDA(cudaStreamWaitEvent(s, t->used, 0));
     t->prims_ptr = d_prims;
+    t->packed_ok = t->few_seen = false;
     Control *c = t->dctl();
     LBVH_CUDA(cudaMemsetAsync(&c->build_flags, 0, sizeof(uint32_t), s));
     if (t->store_dirty && t->store.bytes) {
@@ -1019,6 +1074,8 @@ lbvh_status lbvh_tree_load(lbvh_tree_t t, const void *h_buf, uint64_t bytes, lbv
     t->bits = (int)h.bits;
     t->codes_in = t->perm_in = 0;
     t->prims_ptr = nullptr;
+    t->packed_ok = t->few_seen = false;
+    t->loaded = true;
     LBVH_CUDA(cudaMemsetAsync(&t->dctl()->build_flags, 0, sizeof(uint32_t), s));
     LBVH_CUDA(cudaMemcpyAsync(t->bounds.p, h.bounds, 24, cudaMemcpyHostToDevice, s));
     const char *in = static_cast<const char *>(h_buf) + sizeof h;
@@ -1054,7 +1111,7 @@ lbvh_status lbvh_tree_bytes(lbvh_tree_t t, uint64_t *bytes) {
                             &t->store, &t->pend, &t->lookback, &t->hist, &t->partials, &t->bounds, &t->ctl,
                             &t->counts, &t->tile_sums, &t->overflow, &t->qkeys[0], &t->qkeys[1],
                             &t->qvals[0], &t->qvals[1], &t->qlookback, &t->slots, &t->vscratch,
-                            &t->spill_head, &t->spill})
+                            &t->spill_head, &t->spill, &t->sparse, &t->packed})
         b += d->bytes;
     *bytes = b;
     return LBVH_OK;
@@ -1422,7 +1479,7 @@ void lbvh_batch_destroy(lbvh_batch_t b) {
                       &b->qchunks, &b->keys[0], &b->keys[1], &b->vals[0], &b->vals[1], &b->nodes, &b->store,
                       &b->lookback, &b->hist, &b->partials, &b->bounds, &b->ctl, &b->counts, &b->slots,
                       &b->overflow, &b->tile_sums, &b->qkeys[0], &b->qkeys[1], &b->qvals[0], &b->qvals[1],
-                      &b->qlookback, &b->tile_first, &b->qtile_first, &b->spill_head, &b->spill})
+                      &b->qlookback, &b->tile_first, &b->qtile_first, &b->spill_head, &b->spill, &b->sparse, &b->packed, &b->pack_start})
         d->release(s);
     if (s) cudaStreamSynchronize(s);
     pinned_controls().put(b->h_ctl);
@@ -1617,7 +1674,10 @@ lbvh_status tree_from_batch(lbvh_batch_t b, int64_t instance, lbvh_tree_t t, cud
     LBVH_CUDA(t->nodes.ensure((size_t)units * 16 + 16, s));
     LBVH_CUDA(t->hist.ensure((size_t)kMaxPasses * kRadix * 4, s));
     LBVH_CUDA(t->bounds.ensure(6 * 4, s));
+    const size_t pack_bytes = (size_t)pack_records(n) * 32;
+    LBVH_CUDA(t->packed.ensure(pack_bytes, s));
     t->lean = true;
+    t->loaded = false;
     t->n = n;
     t->kind = kind;
     t->bits = b->sig.bits;
@@ -1628,12 +1688,16 @@ lbvh_status tree_from_batch(lbvh_batch_t b, int64_t instance, lbvh_tree_t t, cud
     if (units > 0)
         LBVH_CUDA(cudaMemcpyAsync(t->nodes.p, b->nodes.as<float4>() + b->h_node_start[instance], units * 16,
                                   cudaMemcpyDeviceToDevice, s));
+    t->packed_ok = b->packets();  // else the first query packs them
+    if (t->packed_ok && pack_bytes > 0)
+        LBVH_CUDA(cudaMemcpyAsync(t->packed.p, b->packed.as<float4>() + 2 * b->h_pack_start[instance], pack_bytes,
+                                  cudaMemcpyDeviceToDevice, s));
     return finish_build(t, s);
 }
 
 void tree_release_query_scratch(lbvh_tree_t t, cudaStream_t s) {
     for (DevBuf *b : {&t->counts, &t->tile_sums, &t->overflow, &t->slots, &t->qkeys[0], &t->qkeys[1],
-                      &t->qvals[0], &t->qvals[1], &t->qlookback, &t->spill_head, &t->spill,
+                      &t->qvals[0], &t->qvals[1], &t->qlookback, &t->spill_head, &t->spill, &t->sparse,
                       &t->stage_off[0], &t->stage_off[1], &t->stage_hits[0], &t->stage_hits[1]})
         b->release(s);
     t->spill_nq = 0;

@@ -11,6 +11,8 @@
 
 namespace lbvh {
 
+int device_sm_count();
+
 // ---------------------------------------------------------------- status bits
 // Latched on the device during a build or query; read back with the control
 // block and mapped to an lbvh_status on the host.
@@ -30,6 +32,8 @@ struct Control {
     uint32_t build_flags;          // kFlag* latched by the last build
     uint32_t bounds_ticket;        // last-block detection of the bounds reduction
     uint32_t sort_ticket[16];      // tile tickets of each sort pass
+    uint32_t pack_ticket;          // last-block detection of launch_pack
+    uint32_t reserved;
     uint32_t query_flags;          // kFlag* latched by the last query
     uint32_t overflow_filled;      // entries of the overflow list
     unsigned long long total;      // total hits of the last query
@@ -39,7 +43,8 @@ struct Control {
     uint32_t run_fallback;         //   a run too long for one CTA was met,
     uint32_t run_sort_count;       //   elements of the fallback sort,
     uint32_t run_heads;            //   runs listed for short_runs_kernel (in this order)
-    uint32_t pad[2];
+    uint32_t sparse_filled;        // packets left to Algorithm 1
+    uint32_t pad[3];
 };
 constexpr int kQueryBufferHits = 64;  // hits kept per query by the walk
 
@@ -209,7 +214,9 @@ void launch_bounds(const float *prims, int64_t n, int kind, float *partials, flo
 // of at most 32 bits, run_index_sort's packed mode); or the top bits
 // (code >> (ib - 1)) << ib | i for run_top_sort, ib = index_bits with
 // n <= 2^ib (index_bits is read for kCodeTop only).
-enum CodeLayout : int { kCodePlain = 0, kCodeLow = 1, kCodeTop = 2 };
+// kCodeHilbert is kCodeLow with the cell's Hilbert index, without its low
+// index_bits bits, as the code.
+enum CodeLayout : int { kCodePlain = 0, kCodeLow = 1, kCodeTop = 2, kCodeHilbert = 3 };
 // Index bits of the top layout for n primitives: ceil(log2 n), at least 1.
 inline int top_index_bits(int64_t n) {
     int ib = 1;
@@ -306,7 +313,11 @@ inline int walk_choice_order_bits(int c) { return c >= kWalkKinds ? 24 : 30; }
 constexpr int kSpillChunkWords = 64;
 constexpr uint32_t kSpilledTag = 1u << 31;  // overflow-list entry whose hits are all in slot + chunks
 inline uint32_t spill_chunks_for(int64_t nq) {
-    const int64_t c = nq / 16;
+    // few queries may all have long lists: 16 chunks each, as long as that is
+    // no more than 16 MB (30,011 queries of 20 hits on average, one in 20 past
+    // its slot: nq / 16 chunks ran out, and the second walk took 0.42 ms)
+    int64_t c = 16 * nq < 65536 ? 16 * nq : 65536;
+    if (c < nq / 16) c = nq / 16;
     return (uint32_t)(c < 1024 ? 1024 : (c > (1 << 26) ? (1 << 26) : c));
 }
 
@@ -317,6 +328,7 @@ struct QueryScratch {
     uint32_t *spill_head;     // nq: first spill chunk of query q
     uint32_t *spill;          // spill_chunks * kSpillChunkWords
     uint32_t spill_chunks;
+    uint2 *sparse_list;       // nq / 32 + 1: packets left to Algorithm 1 (32 walk positions from 32 x, lanes y)
 };
 // The collecting walk (counts, short sorted lists, overflow list).
 void launch_query_collect(const TreeView &t, const QueryArgs &q, const QueryScratch &qs, Control *ctl,
@@ -347,6 +359,45 @@ void launch_query_overflow(const TreeView &t, const QueryArgs &q, const QueryScr
                            uint32_t count, const int64_t *offsets, uint32_t *hits, Control *ctl,
                            cudaStream_t s);
 
+// ---- packets over leaf blocks (packet.cu)
+// The sorted leaves cut into blocks of 8, those into blocks of 8 and so on,
+// until one block is left; block i of a height covers blocks (at height 0:
+// leaves) 8i .. 8i + 7 of the one below. A block's record is its box, two
+// float4, in heap order: the root is record 0 and the children of record g
+// are 8g + 1 .. 8g + 8; the leaf blocks, at the end, start at
+// pack_leaf_start(n).
+// Heights above the leaf blocks.
+__host__ __device__ inline int pack_depth(int64_t n) {
+    int depth = 0;
+    while ((int64_t(8) << (3 * depth)) < n) ++depth;
+    return depth;
+}
+__host__ __device__ inline uint32_t pack_leaf_start(int64_t n) {
+    return (uint32_t)(((int64_t(1) << (3 * pack_depth(n))) - 1) / 7);
+}
+// Records (32 bytes each) of a tree of n leaves; every height but the root's
+// is padded to a multiple of 8.
+inline int64_t pack_records(int64_t n) { return n > 0 ? (int64_t)pack_leaf_start(n) + (n + 63) / 64 * 8 : 0; }
+// The boxes of all blocks, from the tree's leaves.
+void launch_pack(const TreeView &t, float4 *rec, Control *ctl, cudaStream_t s);
+// How nq sphere or box queries on a tree of n leaves walk (`sorted`: an order
+// is at hand):
+enum RangeWalk : int {
+    kRangePackets,  // packets of 32 neighbours, which want a query order
+    kRangeSparse,   // 8 lanes per query through the blocks, in any order
+    kRangeNodes     // Algorithm 1, a thread per query
+};
+RangeWalk range_walk(int64_t nq, int64_t n, bool sorted);
+// Leaves up to which packing them for one call of few queries pays.
+constexpr int64_t kPackForFew = int64_t(1) << 23;
+// The queries of qs.sparse_list.
+void launch_query_collect_left(const TreeView &t, const float4 *rec, const QueryArgs &q, const QueryScratch &qs,
+                               Control *ctl, cudaStream_t s);
+// The collecting walk of sphere and box queries through the blocks (counts,
+// slots, spill chunks and overflow list as launch_query_collect's). t.n > 0.
+void launch_query_packets(const TreeView &t, const float4 *rec, const QueryArgs &q, const QueryScratch &qs,
+                          RangeWalk how, Control *ctl, cudaStream_t s);
+
 // ---------------------------------------------------------------- batches
 // Many independent trees in one pass. Instance b owns primitives
 // [prim_off[b], prim_off[b+1]) of one concatenated array and queries
@@ -364,6 +415,7 @@ struct BatchTables {
     const int64_t *query_off;    // count + 1
     const int64_t *node_start;   // count
     const int64_t *store_start;  // count
+    const int64_t *pack_start;   // count: instance b's first leaf-block record
     const BatchChunk *chunks;    // nchunks (primitives)
     const int64_t *chunk_first;  // count + 1: instance b's chunks are [chunk_first[b], chunk_first[b+1])
     const BatchChunk *qchunks;   // nqchunks (queries, for their Morton order)
@@ -382,14 +434,17 @@ __device__ __forceinline__ int instance_of(const int64_t *__restrict__ off, int 
     return lo;
 }
 
+// Every instance's leaf blocks, from its leaves.
+void launch_batch_pack(const float4 *nodes, int kind, const BatchTables &bt, float4 *rec, cudaStream_t s);
 // Per-instance bounds: partials (nchunks * 8 floats), then bounds (count * 6).
 void launch_batch_bounds(const float *prims, int kind, const BatchTables &bt, float *partials,
                          float *bounds, Control *ctl, cudaStream_t s);
 // Morton codes of primitives (or of query centres, with `queries` = true:
 // qchunks and qkind decide the layout), each in its own instance's grid, plus
-// pass 0's digit histogram of every instance (hist row inst * kRadix).
+// pass 0's digit histogram of every instance (hist row inst * kRadix). With
+// `hilbert`, the first 32 bits of the Hilbert index of 11 levels instead.
 void launch_batch_encode(const float *data, int kind, bool queries, const BatchTables &bt, int bits,
-                         const float *bounds, uint64_t *keys, uint32_t *hist, cudaStream_t s);
+                         const float *bounds, uint64_t *keys, uint32_t *hist, cudaStream_t s, bool hilbert = false);
 void launch_batch_construct(const uint64_t *sorted_codes, const uint32_t *perm, const float *prims,
                             const BatchTables &bt, int kind, float4 *nodes, unsigned long long *store,
                             uint32_t *flags, cudaStream_t s);
@@ -400,6 +455,12 @@ void launch_batch_collect(const float4 *nodes, int kind, const BatchTables &bt, 
 void launch_batch_overflow(const float4 *nodes, int kind, const BatchTables &bt, const QueryArgs &q,
                            const QueryScratch &qs, Control *ctl, const int64_t *offsets, uint32_t *hits,
                            unsigned long long capacity, cudaStream_t s);
+// The collecting walk in packets (rec: launch_batch_pack's records), and
+// Algorithm 1 for the queries it leaves.
+void launch_batch_packets(const float4 *nodes, int kind, const float4 *rec, const BatchTables &bt, const QueryArgs &q,
+                          const QueryScratch &qs, Control *ctl, cudaStream_t s);
+void launch_batch_collect_left(const float4 *nodes, int kind, const BatchTables &bt, const QueryArgs &q,
+                               const QueryScratch &qs, Control *ctl, cudaStream_t s);
 // Copy with the capacity check on the device (no host round trip): lists are
 // written only if ctl->total <= capacity; otherwise kFlagCapacity is latched.
 void launch_query_copy_checked(const QueryArgs &q, const QueryScratch &qs, const int64_t *offsets,
@@ -412,8 +473,6 @@ void launch_query_copy_checked(const QueryArgs &q, const QueryScratch &qs, const
 void batch_set_graphs(lbvh_batch_t b, bool on);
 lbvh_status tree_from_batch(lbvh_batch_t b, int64_t instance, lbvh_tree_t t, cudaStream_t s);
 void tree_release_query_scratch(lbvh_tree_t t, cudaStream_t s);
-
-int device_sm_count();
 
 // ---------------------------------------------------------------- autotuner (tune.cu)
 // A configuration: GPU, ceil(log2 n), Morton bits, primitive kind, query kind

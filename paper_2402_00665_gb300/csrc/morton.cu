@@ -173,6 +173,11 @@ __global__ void __launch_bounds__(kThreads)
 // histograms count the bytes of the code (plain, low) or of the word from
 // byte top_first_byte(ib, skip) on (top): the bytes the sort's passes take
 // in turn.
+// kCodeHilbert: as kCodeLow with the Hilbert index of the cell, without its
+// low ib bits, in place of the Morton code (the order of queries that are
+// walked in packets).
+__device__ const HilbertTable kHilbert = hilbert_table();
+
 template <int kKind, int kLayout>
 __global__ void __launch_bounds__(kThreads)
     encode_kernel(const float *__restrict__ prims, int64_t n, int b, const float *__restrict__ bounds,
@@ -181,12 +186,14 @@ __global__ void __launch_bounds__(kThreads)
     for (int k = threadIdx.x; k < passes * kRadix; k += kThreads) s_hist[k] = 0;
     const Grid3 g = make_grid(bounds, b);
     const int hist_shift = kLayout == kCodeTop ? kRadixBits * top_first_byte(ib, skip) : 0;
+    __shared__ uint32_t s_hilbert[kLayout == kCodeHilbert ? kHilbertStates * 8 : 1];
+    if (kLayout == kCodeHilbert && threadIdx.x < kHilbertStates * 8) s_hilbert[threadIdx.x] = kHilbert.next[threadIdx.x];
     __syncthreads();
     for_each_centroid<kKind>(prims, n, [&](int64_t i, float x, float y, float z) {
-        const uint64_t c = morton(x, y, z, g);
+        const uint64_t c = kLayout == kCodeHilbert ? hilbert(x, y, z, g, b, s_hilbert) >> ib : morton(x, y, z, g);
         const uint64_t w = kLayout == kCodeTop   ? ((c >> (ib - 1)) << ib) | (uint64_t)(uint32_t)i
-                           : kLayout == kCodeLow ? (c << 32) | (uint64_t)(uint32_t)i
-                                                 : c;
+                           : kLayout != kCodePlain ? (c << 32) | (uint64_t)(uint32_t)i
+                                                   : c;
         codes[i] = w;
         const uint64_t h = kLayout == kCodeTop ? w >> hist_shift : c;
         for (int p = 0; p < passes; ++p)
@@ -300,7 +307,7 @@ __global__ void __launch_bounds__(kThreads)
     if (!all) atomicOr(&ctl->build_flags, kFlagNonfinite);
 }
 
-template <int kKind>
+template <int kKind, bool kCurve>
 __global__ void __launch_bounds__(kThreads)
     batch_encode_kernel(const float *__restrict__ data, const BatchChunk *__restrict__ chunks, int b,
                         const float *__restrict__ bounds, uint64_t *__restrict__ keys,
@@ -309,11 +316,13 @@ __global__ void __launch_bounds__(kThreads)
     s_hist[threadIdx.x] = 0;  // kThreads == kRadix
     const BatchChunk c = chunks[blockIdx.x];
     const Grid3 g = make_grid(bounds + 6 * (int64_t)c.inst, b);
+    __shared__ uint32_t s_hilbert[kCurve ? kHilbertStates * 8 : 1];
+    if (kCurve && threadIdx.x < kHilbertStates * 8) s_hilbert[threadIdx.x] = kHilbert.next[threadIdx.x];
     __syncthreads();
     for (int64_t i = c.begin + threadIdx.x; i < c.end; i += kThreads) {
         float x, y, z;
         centroid_at<kKind>(data, i, x, y, z);
-        const uint64_t key = morton(x, y, z, g);
+        const uint64_t key = kCurve ? hilbert(x, y, z, g, b, s_hilbert) >> 1 : morton(x, y, z, g);
         keys[i] = key;
         atomicAdd(&s_hist[(uint32_t)key & (kRadix - 1)], 1u);
     }
@@ -337,17 +346,16 @@ void launch_batch_bounds(const float *prims, int kind, const BatchTables &bt, fl
 }
 
 void launch_batch_encode(const float *data, int kind, bool queries, const BatchTables &bt, int bits,
-                         const float *bounds, uint64_t *keys, uint32_t *hist, cudaStream_t s) {
+                         const float *bounds, uint64_t *keys, uint32_t *hist, cudaStream_t s, bool hilbert) {
     const int64_t nchunks = queries ? bt.nqchunks : bt.nchunks;
     const BatchChunk *chunks = queries ? bt.qchunks : bt.chunks;
     if (nchunks <= 0) return;
-    const int b = bits / 3;
-    if (kind == LBVH_PRIM_POINTS)
-        batch_encode_kernel<LBVH_PRIM_POINTS><<<(unsigned)nchunks, kThreads, 0, s>>>(data, chunks, b, bounds,
-                                                                                     keys, hist);
-    else
-        batch_encode_kernel<LBVH_PRIM_BOXES><<<(unsigned)nchunks, kThreads, 0, s>>>(data, chunks, b, bounds,
-                                                                                    keys, hist);
+    const int b = hilbert ? 11 : bits / 3;
+    const bool points = kind == LBVH_PRIM_POINTS;
+    auto k = hilbert ? (points ? batch_encode_kernel<LBVH_PRIM_POINTS, true> : batch_encode_kernel<LBVH_PRIM_BOXES, true>)
+                     : (points ? batch_encode_kernel<LBVH_PRIM_POINTS, false>
+                               : batch_encode_kernel<LBVH_PRIM_BOXES, false>);
+    k<<<(unsigned)nchunks, kThreads, 0, s>>>(data, chunks, b, bounds, keys, hist);
     count_launches(1);
 }
 
@@ -373,11 +381,11 @@ void launch_encode(const float *prims, int64_t n, int kind, int bits, const floa
     const int blocks = bounds_blocks(n);
     const int b = bits / 3;
     using Kernel = void (*)(const float *, int64_t, int, const float *, uint64_t *, uint32_t *, int, int, int);
-    static const Kernel table[2][3] = {
+    static const Kernel table[2][4] = {
         {encode_kernel<LBVH_PRIM_POINTS, kCodePlain>, encode_kernel<LBVH_PRIM_POINTS, kCodeLow>,
-         encode_kernel<LBVH_PRIM_POINTS, kCodeTop>},
+         encode_kernel<LBVH_PRIM_POINTS, kCodeTop>, encode_kernel<LBVH_PRIM_POINTS, kCodeHilbert>},
         {encode_kernel<LBVH_PRIM_BOXES, kCodePlain>, encode_kernel<LBVH_PRIM_BOXES, kCodeLow>,
-         encode_kernel<LBVH_PRIM_BOXES, kCodeTop>}};
+         encode_kernel<LBVH_PRIM_BOXES, kCodeTop>, encode_kernel<LBVH_PRIM_BOXES, kCodeHilbert>}};
     table[kind == LBVH_PRIM_POINTS ? 0 : 1][layout]<<<blocks, kThreads, 0, s>>>(prims, n, b, bounds, codes, hist,
                                                                                hist_passes, index_bits, skip);
     count_launches(1);

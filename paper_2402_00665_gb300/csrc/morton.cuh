@@ -76,6 +76,59 @@ __device__ __forceinline__ uint64_t morton(float x, float y, float z, const Grid
     return (spread3(qx) << 2) | (spread3(qy) << 1) | spread3(qz);
 }
 
+// ---- Hilbert order (queries only: neighbours on the curve are neighbours in
+// space, without the Morton curve's jumps; the order of the queries changes
+// no result). One level at a time with the entry point e and direction d of
+// the cell (C. Hamilton, "Compact Hilbert Indices", 2006): the octant l
+// becomes t = rotr(l ^ e, d + 1), its rank on the curve is the inverse Gray
+// code w of t, and the child's e ^= rotl(entry(w), d + 1), d += dir(w) + 1.
+// The table holds, for state e * 3 + d and octant l, w | next state << 3.
+constexpr int kHilbertStates = 24;
+struct HilbertTable {
+    uint8_t next[kHilbertStates * 8];
+};
+constexpr uint32_t rot3(uint32_t v, uint32_t left) {
+    left %= 3u;
+    return ((v << left) | (v >> (3u - left))) & 7u;
+}
+constexpr HilbertTable hilbert_table() {
+    HilbertTable t{};
+    for (uint32_t e = 0; e < 8; ++e)
+        for (uint32_t d = 0; d < 3; ++d)
+            for (uint32_t l = 0; l < 8; ++l) {
+                const uint32_t g = rot3(l ^ e, 3u - (d + 1u) % 3u);
+                const uint32_t w = g ^ (g >> 1) ^ (g >> 2);
+                const uint32_t before = w == 0 ? 0u : 2u * ((w - 1u) / 2u);  // entry(w) = gray(before)
+                const uint32_t ne = e ^ rot3(before ^ (before >> 1), d + 1u);
+                // dir(w): trailing ones of w (odd w) or of w - 1 (even w > 0), mod 3
+                uint32_t v = w == 0 ? 0u : (w & 1u ? w : w - 1u), dir = 0;
+                while (v & 1u) {
+                    ++dir;
+                    v >>= 1;
+                }
+                const uint32_t nd = (d + dir + 1u) % 3u;
+                t.next[(e * 3u + d) * 8u + l] = (uint8_t)(w | (ne * 3u + nd) << 3);
+            }
+    return t;
+}
+
+// The Hilbert index of a cell of the grid (b bits per axis, 3b at most 63);
+// `table`: hilbert_table().next, one word per entry.
+__device__ __forceinline__ uint64_t hilbert(float x, float y, float z, const Grid3 &g, int b, const uint32_t *table) {
+    const uint32_t qx = cell_of(x, g.lo[0], g.extent[0], g);
+    const uint32_t qy = cell_of(y, g.lo[1], g.extent[1], g);
+    const uint32_t qz = cell_of(z, g.lo[2], g.extent[2], g);
+    uint64_t code = 0;
+    uint32_t state = 0;
+    for (int k = b - 1; k >= 0; --k) {
+        const uint32_t l = ((qx >> k) & 1u) << 2 | ((qy >> k) & 1u) << 1 | ((qz >> k) & 1u);
+        const uint32_t e = table[state * 8u + l];
+        code = code << 3 | (e & 7u);
+        state = e >> 3;
+    }
+    return code;
+}
+
 __device__ __forceinline__ bool finite3(float x, float y, float z) {
     return fabsf(x) <= FLT_MAX && fabsf(y) <= FLT_MAX && fabsf(z) <= FLT_MAX;
 }

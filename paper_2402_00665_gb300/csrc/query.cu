@@ -50,147 +50,13 @@
 
 #include "lbvh_internal.cuh"
 #include "morton.cuh"
+#include "walk.cuh"
 
 namespace lbvh {
 
 namespace {
 
 constexpr int kThreads = 256;
-
-struct Sphere {
-    float3 c;
-    float r2;
-};
-struct Box {
-    float3 lo, hi;
-};
-// A ray segment: origin, 1/direction per axis (IEEE division), which axes
-// are parallel (direction 0, or a reciprocal that overflows), and [tmin, tmax].
-struct Ray {
-    float3 o, inv;
-    float tmin, tmax;
-    uint32_t parallel;  // bit a: axis a
-};
-
-// |gap| between c and [lo, hi]: c - clamp(c, lo, hi) (sign irrelevant: squared)
-__device__ __forceinline__ float gap(float lo, float c, float hi) {
-    return __fsub_rn(c, fminf(fmaxf(c, lo), hi));
-}
-
-// Squared distance from c to the box: ex*ex, then + ey*ey and + ez*ez each
-// as one fused multiply-add.
-__device__ __forceinline__ float box_d2(float3 c, float3 lo, float3 hi) {
-    const float ex = gap(lo.x, c.x, hi.x);
-    const float ey = gap(lo.y, c.y, hi.y);
-    const float ez = gap(lo.z, c.z, hi.z);
-    return __fmaf_rn(ez, ez, __fmaf_rn(ey, ey, __fmul_rn(ex, ex)));
-}
-
-__device__ __forceinline__ bool hits(const Sphere &s, float3 lo, float3 hi) { return box_d2(s.c, lo, hi) <= s.r2; }
-
-// Slab test, each operation rounded once: per axis t1 = (lo - o) * inv and
-// t2 = (hi - o) * inv; tnear = max(tmin, min(t1, t2)), tfar = min(tmax,
-// max(t1, t2)); a parallel axis instead requires lo <= o <= hi. Hit iff
-// tnear <= tfar. Monotone in the box, like the other predicates.
-__device__ __forceinline__ bool slab(float lo, float hi, float o, float inv, bool parallel, float &tn,
-                                     float &tf) {
-    if (parallel) return lo <= o && o <= hi;
-    const float t1 = __fmul_rn(__fsub_rn(lo, o), inv), t2 = __fmul_rn(__fsub_rn(hi, o), inv);
-    tn = fmaxf(tn, fminf(t1, t2));
-    tf = fminf(tf, fmaxf(t1, t2));
-    return true;
-}
-
-__device__ __forceinline__ bool hits(const Ray &r, float3 lo, float3 hi) {
-    float tn = r.tmin, tf = r.tmax;
-    if (!slab(lo.x, hi.x, r.o.x, r.inv.x, r.parallel & 1u, tn, tf)) return false;
-    if (!slab(lo.y, hi.y, r.o.y, r.inv.y, r.parallel & 2u, tn, tf)) return false;
-    if (!slab(lo.z, hi.z, r.o.z, r.inv.z, r.parallel & 4u, tn, tf)) return false;
-    return tn <= tf;
-}
-
-__device__ __forceinline__ bool hits(const Box &q, float3 lo, float3 hi) {
-    return q.lo.x <= hi.x && lo.x <= q.hi.x && q.lo.y <= hi.y && lo.y <= q.hi.y &&
-           q.lo.z <= hi.z && lo.z <= q.hi.z;
-}
-
-template <int kQ>
-struct QueryOf;
-template <>
-struct QueryOf<LBVH_Q_SPHERE> {
-    using type = Sphere;
-    static __device__ __forceinline__ Sphere load(const QueryArgs &a, int64_t q) {
-        const float *p = a.queries + 3 * q;
-        const float r = a.radii ? __ldcs(a.radii + q) : a.radius;
-        return Sphere{make_float3(__ldcs(p), __ldcs(p + 1), __ldcs(p + 2)), __fmul_rn(r, r)};
-    }
-};
-template <>
-struct QueryOf<LBVH_Q_RAY> {
-    using type = Ray;
-    static __device__ __forceinline__ float axis_inv(float d, uint32_t bit, uint32_t &parallel) {
-        const float inv = __fdiv_rn(1.0f, d);
-        if (d == 0.0f || isinf(inv)) parallel |= bit;
-        return inv;
-    }
-    static __device__ __forceinline__ Ray load(const QueryArgs &a, int64_t q) {
-        const float4 *p = reinterpret_cast<const float4 *>(a.queries) + 2 * q;
-        const float4 u = __ldcs(p), v = __ldcs(p + 1);
-        Ray r;
-        r.parallel = 0;
-        r.o = make_float3(u.x, u.y, u.z);
-        r.inv = make_float3(axis_inv(v.x, 1u, r.parallel), axis_inv(v.y, 2u, r.parallel),
-                            axis_inv(v.z, 4u, r.parallel));
-        r.tmin = u.w;
-        r.tmax = v.w;
-        const bool finite = isfinite(u.x) && isfinite(u.y) && isfinite(u.z) && isfinite(v.x) && isfinite(v.y) &&
-                            isfinite(v.z) && !isnan(u.w) && !isnan(v.w);
-        if (!finite) {  // hits nothing: an empty parameter interval on every axis
-            r.tmin = 1.0f;
-            r.tmax = 0.0f;
-            r.parallel = 0;
-            r.o = make_float3(0.0f, 0.0f, 0.0f);
-            r.inv = make_float3(1.0f, 1.0f, 1.0f);
-        }
-        return r;
-    }
-};
-template <>
-struct QueryOf<LBVH_Q_BOX> {
-    using type = Box;
-    static __device__ __forceinline__ Box load(const QueryArgs &a, int64_t q) {
-        const float *p = a.queries + 6 * q;
-        return Box{make_float3(__ldcs(p), __ldcs(p + 1), __ldcs(p + 2)),
-                   make_float3(__ldcs(p + 3), __ldcs(p + 4), __ldcs(p + 5))};
-    }
-};
-
-__device__ __forceinline__ float3 xyz(float4 v) { return make_float3(v.x, v.y, v.z); }
-
-// A node record as one 32-byte load (two float4 halves), read-only path.
-// Records of two float4 start on 32-byte boundaries (internal nodes and box
-// leaves; batches pad every tree to an even float4 offset).
-__device__ __forceinline__ void ld_node32(const float4 *p, float4 &a, float4 &b) {
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
-        : "l"(p));
-}
-
-// The node at `unit` (float4 units). In a box tree every record is 32 bytes:
-// one 32-byte load per step (measured: D3's walk 10.14 -> 8.39 ms). In a
-// point tree a leaf is one float4 (its box is its point): a first 16-byte
-// load common to every lane and a second one for internal nodes measured
-// faster than splitting the warp between a 16- and a 32-byte load.
-template <int kP>
-__device__ __forceinline__ void load_node(const float4 *base, int unit, bool leaf, float4 &a, float4 &b) {
-    if (kP == LBVH_PRIM_BOXES) {
-        ld_node32(base + unit, a, b);
-    } else {
-        a = __ldg(base + unit);
-        b = a;
-        if (!leaf) b = __ldg(base + unit + 1);
-    }
-}
 
 // Algorithm 1. on_leaf(id) is called with the primitive index of every leaf
 // that satisfies the predicate, leaves in increasing sorted position. Returns
@@ -260,38 +126,6 @@ __device__ __forceinline__ bool walk_group(const TreeView &t, const Q &q, bool a
         }
     }
     return node == kSentinel || node == nodes;
-}
-
-constexpr int kSlot = kQueryBufferHits;  // ids kept per walk (slot size)
-constexpr int kRegSort = 32;             // lists up to this long are sorted in one thread's registers
-
-__device__ __forceinline__ int64_t thread_query(const QueryArgs &qa, int64_t i) {
-    return qa.order ? (int64_t)__ldcs(qa.order + i) : i;
-}
-
-// Hits past a walk's slot: appended to chunks from the shared pool, the first
-// chunk recorded in spill_head[q], each chunk's word 0 linking to the next.
-// `cur` is the walk's current chunk (kNoChunk before the first); it becomes
-// kSpillFailed when the pool is exhausted, and the query then takes the
-// second walk.
-constexpr uint32_t kNoChunk = 0xffffffffu, kSpillFailed = 0xfffffffeu;
-
-__device__ __forceinline__ void spill_put(const QueryScratch &qs, Control *ctl, int64_t i, uint32_t cnt,
-                                          uint32_t id, uint32_t &cur) {
-    if (cur == kSpillFailed) return;
-    const uint32_t sidx = cnt - (uint32_t)kSlot;                   // index among the spilled hits
-    const uint32_t off = sidx % (uint32_t)(kSpillChunkWords - 1);  // slot in the chunk (after the link)
-    if (off == 0) {
-        const uint32_t fresh = atomicAdd(&ctl->spill_used, 1u);
-        if (fresh >= qs.spill_chunks) {
-            cur = kSpillFailed;
-            return;
-        }
-        if (cur == kNoChunk) qs.spill_head[i] = fresh;
-        else qs.spill[(int64_t)cur * kSpillChunkWords] = fresh;
-        cur = fresh;
-    }
-    qs.spill[(int64_t)cur * kSpillChunkWords + 1 + off] = id;
 }
 
 // One query's collecting walk at walk position i (query qi): the first kSlot
@@ -377,6 +211,43 @@ __global__ void __launch_bounds__(kT, 2048 / kT)
     if (i >= qa.nq) return;
     const bool walk_ok = t.n > 0 && ctl->build_flags == 0;
     collect_walk<kQ, kP, kP == LBVH_PRIM_POINTS>(t, qa, qs, ctl, i, thread_query(qa, i), walk_ok);
+}
+
+// The queries that packet_kernel left (packets of queries too far apart; list
+// entries of 32 walk positions each). A few entries: 8 lanes per query
+// through the leaf blocks, 4 queries per warp (2^24 box queries on 2^25 boxes
+// leave about 200 entries: Algorithm 1 took 0.29 ms, one long walk after the
+// other). Many: Algorithm 1, a warp per entry, the faster one when the GPU is
+// full. A fixed grid strides over the list.
+constexpr int64_t kLeftFew = 2048;
+
+template <int kQ, int kP>
+__global__ void __launch_bounds__(kThreads)
+    collect_left_kernel(TreeView t, const float4 *__restrict__ rec, QueryArgs qa, QueryScratch qs, Control *ctl) {
+    __shared__ uint32_t s_stack[kThreads / 8][kSparseStack];
+    const int64_t count = ctl->sparse_filled;
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)gridDim.x * (kThreads / 32);
+    const int64_t first = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
+    if (count <= kLeftFew) {
+        const Blocks blocks{t.leaves, rec, (int)t.n, pack_leaf_start(t.n)};
+        for (int64_t j = first; j < 8 * count; j += stride) {
+            const uint2 e = qs.sparse_list[j >> 3];
+            const int at = (int)(j & 7) * 4 + (lane >> 3);
+            const bool has = (e.y >> at) & 1u;
+            const int64_t qi = has ? thread_query(qa, (int64_t)e.x * 32 + at) : 0;
+            typename QueryOf<kQ>::type q{};
+            if (has) q = QueryOf<kQ>::load(qa, qi);
+            sparse_walk<kQ, kP>(blocks, s_stack[threadIdx.x >> 3], q, has, qi, qs, ctl);
+        }
+        return;
+    }
+    for (int64_t j = first; j < count; j += stride) {
+        const uint2 e = qs.sparse_list[j];
+        const int64_t i = (int64_t)e.x * 32 + lane;
+        if ((e.y >> lane) & 1u)
+            collect_walk<kQ, kP, kP == LBVH_PRIM_POINTS>(t, qa, qs, ctl, i, thread_query(qa, i), true);
+    }
 }
 
 // Batcher's odd-even merge sort of v[0..kN) (kN a power of two), keeping only
@@ -813,6 +684,24 @@ __global__ void __launch_bounds__(kThreads, 8)  // at most 32 registers: full oc
     collect_walk<kQ, kP, false>(t, qa, qs, ctl, i, qi, n > 0 && ctl->build_flags == 0);
 }
 
+template <int kQ, int kP>
+__global__ void __launch_bounds__(kThreads, 8)
+    batch_collect_left_kernel(const float4 *__restrict__ nodes, BatchTables bt, QueryArgs qa, QueryScratch qs,
+                              Control *ctl) {
+    const int64_t count = ctl->sparse_filled;
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)gridDim.x * (kThreads / 32);
+    for (int64_t j = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5; j < count; j += stride) {
+        const uint2 e = qs.sparse_list[j];
+        if (!((e.y >> lane) & 1u)) continue;
+        const int64_t i = (int64_t)e.x * 32 + lane, qi = thread_query(qa, i);
+        const int b = instance_of(bt.query_off, bt.count, qi);
+        const int64_t n = bt.prim_off[b + 1] - bt.prim_off[b];
+        const TreeView t{nodes + bt.node_start[b], nullptr, n, kP};
+        collect_walk<kQ, kP, false>(t, qa, qs, ctl, i, qi, n > 0);
+    }
+}
+
 // Overflow lists whose number is known only on the device: a fixed grid
 // strides over them.
 template <int kQ, int kP>
@@ -1064,6 +953,16 @@ void launch_query_collect(const TreeView &t, const QueryArgs &q, const QueryScra
     count_launches(1);
 }
 
+void launch_query_collect_left(const TreeView &t, const float4 *rec, const QueryArgs &q, const QueryScratch &qs,
+                               Control *ctl, cudaStream_t s) {
+    const unsigned blocks =
+        (unsigned)std::min<int64_t>((q.nq + kThreads - 1) / kThreads, (int64_t)device_sm_count() * 8);
+    dispatch_kinds(q.qkind, t.kind, [&](auto qk, auto pk) {
+        collect_left_kernel<decltype(qk)::value, decltype(pk)::value><<<blocks, kThreads, 0, s>>>(t, rec, q, qs, ctl);
+    });
+    count_launches(1);
+}
+
 void launch_query_copy_checked(const QueryArgs &q, const QueryScratch &qs, const int64_t *offsets,
                                uint32_t *hits, unsigned long long capacity, Control *ctl, cudaStream_t s) {
     if (q.nq <= 0) return;
@@ -1113,6 +1012,17 @@ void launch_batch_collect(const float4 *nodes, int kind, const BatchTables &bt, 
     dispatch_kinds(q.qkind, kind, [&](auto qk, auto pk) {
         batch_collect_kernel<decltype(qk)::value, decltype(pk)::value><<<blocks, kThreads, 0, s>>>(nodes, bt, q, qs,
                                                                                                     ctl);
+    });
+    count_launches(1);
+}
+
+void launch_batch_collect_left(const float4 *nodes, int kind, const BatchTables &bt, const QueryArgs &q,
+                               const QueryScratch &qs, Control *ctl, cudaStream_t s) {
+    const unsigned blocks =
+        (unsigned)std::min<int64_t>((q.nq + kThreads - 1) / kThreads, (int64_t)device_sm_count() * 8);
+    dispatch_kinds(q.qkind, kind, [&](auto qk, auto pk) {
+        batch_collect_left_kernel<decltype(qk)::value, decltype(pk)::value><<<blocks, kThreads, 0, s>>>(nodes, bt, q, qs,
+                                                                                                        ctl);
     });
     count_launches(1);
 }

@@ -153,17 +153,18 @@ uint64_t estimate_bytes(const lbvh_request &r) {
     const uint64_t n = (uint64_t)r.n, nq = (uint64_t)r.nq;
     const uint64_t prim = r.kind == LBVH_PRIM_POINTS ? 12 : 24;
     const uint64_t qsz = r.qkind == LBVH_Q_SPHERE ? 12 : (r.qkind == LBVH_Q_BOX ? 24 : 32);
-    const uint64_t build = n * (prim + 24 + 24 + 48 + 8 + 16);
+    const uint64_t build = n * (prim + 24 + 24 + 48 + 8 + 16) + (uint64_t)lbvh::pack_records(r.n) * 32;
     const uint64_t query = nq * (qsz + 4 + 8 + lbvh::kQueryBufferHits * 4 + 4 + 8 + 24 + 8) + r.capacity * 4;
     return std::max<uint64_t>(build + query, 1);  // a running job always counts as in flight
 }
 
 // Device bytes of a resident tree: its nodes (2(n-1) internal records of
-// 32 bytes, leaves of 16 or 32 bytes) plus the control block, bounds and the
-// query-order histogram.
+// 32 bytes, leaves of 16 or 32 bytes) and leaf blocks plus the control block,
+// bounds and the query-order histogram.
 uint64_t resident_bytes_of(int64_t n, int kind) {
     const uint64_t un = (uint64_t)std::max<int64_t>(n, 1);
-    return (2 * (un - 1) + (kind == LBVH_PRIM_POINTS ? un : 2 * un)) * 16 + 16 + 8192 + 512;
+    return (2 * (un - 1) + (kind == LBVH_PRIM_POINTS ? un : 2 * un)) * 16 + 16 + 8192 + 512 +
+           (uint64_t)lbvh::pack_records(un) * 32;
 }
 
 bool same_batch_kind(const lbvh_request &a, const lbvh_request &b) {

@@ -1,0 +1,149 @@
+"""Range queries through the leaf blocks (packets of 32 queries, 8 lanes per
+query) against Algorithm 1 over the nodes, which walk variant 4 runs: the same
+CSR bit for bit at the edges of the blocks' levels, for every query and
+primitive kind, with special queries, queries too far apart for a packet, and
+after the leaves changed."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from paper_2402_00665_gb300 import _build, inputs
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+NODES = 4  # walk variant: Algorithm 1, one thread per query
+PACKETS = 100_003  # queries, enough for packets whatever the order
+
+
+@pytest.fixture(scope="module", autouse=True)
+def lib():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    _build.build()
+    from paper_2402_00665_gb300 import lbvh
+    return lbvh.load()
+
+
+def L():
+    from paper_2402_00665_gb300 import lbvh
+    return lbvh
+
+
+def csr(tree, q, qkind, **kw):
+    off, hits = tree.query(q, qkind, **kw)
+    return off.cpu().numpy(), hits.cpu().numpy()
+
+
+def both(tree, q, qkind, **kw):
+    tree.set_tuning(-1, -1)
+    got = csr(tree, q, qkind, **kw)
+    tree.set_tuning(-1, NODES)
+    want = csr(tree, q, qkind, **kw)
+    tree.set_tuning(-1, -1)
+    assert np.array_equal(got[0], want[0])
+    assert np.array_equal(got[1], want[1])
+    return want
+
+
+def boxes_at(points, half):
+    return np.concatenate([points - half, points + half], axis=1).astype(np.float32)
+
+
+@pytest.mark.parametrize("nq", [37, PACKETS])
+@pytest.mark.parametrize("kind", ["points", "boxes"])
+@pytest.mark.parametrize("n", [1, 2, 7, 8, 9, 63, 64, 65, 511, 512, 513, 4095, 4096, 4097, 32767, 32769, 262145])
+def test_block_levels(n, kind, nq):
+    lbvh = L()
+    pts = inputs.uniform_points(n, seed=n)
+    q = inputs.uniform_points(nq, seed=n + 1)
+    r = 0.6 * float(inputs.radius_for_neighbours(n))
+    t = lbvh.Tree()
+    t.build(pts if kind == "points" else boxes_at(pts, 0.2 * r), lbvh.POINTS if kind == "points" else lbvh.BOXES, 63)
+    total = both(t, q, lbvh.SPHERE, radius=r)[0][-1]
+    both(t, boxes_at(q, 0.7 * r), lbvh.BOX)
+    assert total > 0 or n * nq < 1000
+    t.close()
+
+
+@pytest.mark.parametrize("nq", [900, PACKETS])
+def test_special_queries(nq):
+    lbvh = L()
+    n = 5000
+    pts = inputs.uniform_points(n, seed=3)
+    q = inputs.uniform_points(nq, seed=4)
+    radii = np.full(nq, 0.03, np.float32)
+    inf, nan = np.float32(np.inf), np.float32(np.nan)
+    q[5::97, 1], q[6::97, 0], q[7::97, 2] = nan, inf, -inf
+    radii[8::97], radii[9::97], radii[10::97], radii[11::97] = nan, 0.0, -0.05, 3e38
+    radii[12::9973] = inf
+    q[11::194, 2], q[12::9973, 0] = inf, -inf  # an infinite distance within an infinite radius
+    t = lbvh.Tree().build(pts, lbvh.POINTS, 30)
+    both(t, q, lbvh.SPHERE, radii=radii)
+    b = boxes_at(q, 0.03)
+    b[13::97, :3], b[14::97, 3:] = b[13::97, 3:] + 0.01, nan  # the wrong way round, and NaN
+    both(t, b, lbvh.BOX)
+    t.close()
+
+
+@pytest.mark.parametrize("n,scale", [(300_000, 0.02), (300_000, 1.5), (20_000, 12.0)])
+def test_queries_far_apart_and_long_lists(n, scale):
+    """Regions that are not tight (small radii), lists past a slot (large ones), and jumps between clusters."""
+    lbvh = L()
+    pts = inputs.gaussian_mixture_points(n, seed=7, components=5, sigma=0.02)
+    q = np.concatenate([inputs.gaussian_mixture_points(PACKETS - 2000, seed=7, components=5, sigma=0.05),
+                        inputs.uniform_points(2000, seed=8)])
+    r = scale * float(inputs.radius_for_neighbours(n)) * 0.1
+    t = lbvh.Tree().build(pts, lbvh.POINTS, 63)
+    off, _ = both(t, q, lbvh.SPHERE, radius=r)
+    if scale > 10:
+        assert np.diff(off).max() > 64
+    t.close()
+
+
+def test_own_points_and_changed_leaves():
+    lbvh = L()
+    n = 120_001
+    pts = torch.from_numpy(inputs.uniform_points(n, seed=11)).cuda()
+    r = float(inputs.radius_for_neighbours(n))
+    t = lbvh.Tree().build(pts, lbvh.POINTS, 30)
+    first = both(t, pts, lbvh.SPHERE, radius=r)
+    moved = pts + 0.5 * r * torch.randn_like(pts)
+    t.refit(moved)
+    second = both(t, moved, lbvh.SPHERE, radius=r)
+    assert first[0][-1] != second[0][-1]
+    image = t.save()
+    loaded = lbvh.Tree().load(image)
+    off, hits = csr(loaded, moved, lbvh.SPHERE, radius=r)
+    assert np.array_equal(off, second[0]) and np.array_equal(hits, second[1])
+    t.build(pts[:5000].contiguous(), lbvh.POINTS, 30, algorithm=lbvh.BUILD_KARRAS)
+    both(t, pts, lbvh.SPHERE, radius=4 * r)
+    t.close()
+    loaded.close()
+
+
+def test_batch_of_small_and_empty_instances():
+    """Warps whose queries belong to several instances."""
+    lbvh = L()
+    sizes = np.array([0, 1, 5, 31, 32, 33, 0, 64, 65, 300, 1, 1, 4097, 9000, 2], np.int64)
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    pts = inputs.uniform_points(int(off[-1]), seed=31)
+    q = inputs.uniform_points(int(off[-1]), seed=32)
+    batch = lbvh.Batch()
+    boff, bhits, total, st = batch.build_query(torch.from_numpy(pts).cuda(), off, lbvh.POINTS, 30,
+                                               torch.from_numpy(q).cuda(), off, radius=0.08, capacity=4_000_000)
+    assert st == lbvh.OK
+    boff, bhits = boff.cpu().numpy(), bhits.cpu().numpy()
+    for k, n in enumerate(sizes):
+        a, e = off[k], off[k + 1]
+        if n == 0:
+            continue
+        t = lbvh.Tree().build(pts[a:e], lbvh.POINTS, 30)
+        t.set_tuning(-1, NODES)
+        o, h = csr(t, q[a:e], lbvh.SPHERE, radius=0.08)
+        assert np.array_equal(boff[a:e + 1] - boff[a], o)
+        assert np.array_equal(bhits[boff[a]:boff[e]], h)
+        t.close()
+    batch.close()
