@@ -1322,20 +1322,45 @@ lbvh_status lbvh_knn(lbvh_tree_t t, const float *d_queries, int64_t nq, int k, u
     QueryArgs qa{d_queries, nq, LBVH_Q_SPHERE, nullptr, 0.0f, nullptr};
     t->prof.clear(LBVH_STAGE_QCOUNT, LBVH_STAGE_QORDER + 1);
     t->prof.begin(LBVH_STAGE_QORDER, s);
-    lbvh_status st = query_order(t, qa, s);  // the Morton order of the query points
-    t->prof.end(LBVH_STAGE_QORDER, s);
-    if (st != LBVH_OK) return st;
     // a lean (server-resident) tree keeps no sorted codes: its walks start
     // without seeds, which is exact but slower
     const uint64_t *codes = t->lean ? nullptr : t->sorted_codes();
+    const bool packets = codes && t->bits > 0 && !t->loaded && knn_in_packets(nq, t->n, k);
+    // the order of the query points
+    lbvh_status st = query_order(t, qa, s, order_bits(), packets ? kCodeHilbert : kCodeLow);
+    t->prof.end(LBVH_STAGE_QORDER, s);
+    if (st != LBVH_OK) return st;
+    const bool own = qa.order && own_order(t, qa);
+    KnnScratch sc{};
+    bool pack = false;
+    if (packets) {
+        sc.chunk = knn_chunk(nq);
+        LBVH_CUDA(t->slots.ensure((size_t)sc.chunk * knn_slot_bytes(k), s));
+        const int64_t chunks = (nq + sc.chunk - 1) / sc.chunk;
+        LBVH_CUDA(t->counts.ensure((size_t)(3 * sc.chunk + chunks) * 4, s));
+        pack = !t->packed_ok;
+        if (pack) LBVH_CUDA(t->packed.ensure((size_t)pack_records(t->n) * 32, s));
+        sc.slots = t->slots.as<uint2>();
+        sc.counts = t->counts.as<uint32_t>();
+        sc.radii2 = t->counts.as<float>() + sc.chunk;
+        sc.redo = sc.counts + 2 * sc.chunk;
+        sc.redo_counts = sc.counts + 3 * sc.chunk;
+    }
     t->prof.begin(LBVH_STAGE_QCOUNT, s);  // the kNN walk is timed as the query walk
-    launch_knn(t->view(), codes, t->bounds.as<float>(), t->bits, qa, k, d_idx, d_dist2, c, s);
+    if (packets) {
+        if (pack) launch_pack(t->view(), t->packed.as<float4>(), c, s);
+        launch_knn_packets(t->view(), t->packed.as<float4>(), codes, t->bounds.as<float>(), t->bits, qa, own, k, sc, d_idx,
+                           d_dist2, c, s);
+    } else {
+        launch_knn(t->view(), codes, t->bounds.as<float>(), t->bits, qa, k, d_idx, d_dist2, c, s);
+    }
     t->prof.end(LBVH_STAGE_QCOUNT, s);
     LBVH_LAUNCHED();
     if (!t->used) LBVH_CUDA(cudaEventCreateWithFlags(&t->used, cudaEventDisableTiming));
     LBVH_CUDA(cudaEventRecord(t->used, s));
     t->queried = true;
     if ((st = read_control(t, s)) != LBVH_OK) return st;
+    if (pack) t->packed_ok = true;
     st = flags_status(t->h_ctl->build_flags);
     return st != LBVH_OK ? st : flags_status(t->h_ctl->query_flags);
 }

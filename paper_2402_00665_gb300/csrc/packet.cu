@@ -33,6 +33,7 @@
 #include <type_traits>
 
 #include "lbvh_internal.cuh"
+#include "packet.cuh"
 #include "walk.cuh"
 
 namespace lbvh {
@@ -77,20 +78,6 @@ __device__ __forceinline__ void put_block(float4 *rec, int64_t at, const Bounds 
 __device__ __forceinline__ Bounds get_block(const float4 *rec, int64_t at) {
     const float4 a = __ldcg(rec + 2 * at), b = __ldcg(rec + 2 * at + 1);
     return Bounds{make_float3(a.x, a.y, a.z), make_float3(b.x, b.y, b.z)};
-}
-
-// A primitive's box with its bounds in order: the exact test of a box given
-// the wrong way round (lo > hi) looks at either bound, so a region has to
-// meet both.
-template <int kP>
-__device__ __forceinline__ float3 leaf_lo(float4 a, float4 b) {
-    if (kP == LBVH_PRIM_POINTS) return xyz(a);
-    return make_float3(fminf(a.x, b.x), fminf(a.y, b.y), fminf(a.z, b.z));
-}
-template <int kP>
-__device__ __forceinline__ float3 leaf_hi(float4 a, float4 b) {
-    if (kP == LBVH_PRIM_POINTS) return xyz(b);
-    return make_float3(fmaxf(a.x, b.x), fmaxf(a.y, b.y), fmaxf(a.z, b.z));
 }
 
 // Blocks of height h (0: leaf blocks) of a tree of n leaves, and the same
@@ -242,209 +229,7 @@ __global__ void __launch_bounds__(kPackThreads) batch_pack_top_kernel(BatchTable
     if (n > 0) pack_top(n, pack_depth(n), 3, rec + 2 * bt.pack_start[blockIdx.x]);
 }
 
-// f32x2: two FP32 operations of one instruction, each rounded as its scalar form
-__device__ __forceinline__ uint64_t pack2(float a, float b) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float &a, float &b) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
-// ---------------------------------------------------------------- regions
-
-// The region of a packet: meets() holds wherever hits() holds for one of the
-// packet's queries (every operation is monotone in the query's bounds under
-// round-to-nearest, so this needs no margin).
-template <typename Q>
-struct Region;
-
-__device__ __forceinline__ float warp_min(float v) {
-    float r;
-    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-    return r;
-}
-__device__ __forceinline__ float warp_max(float v) {
-    float r;
-    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-    return r;
-}
-
-__device__ __forceinline__ float max3(float a, float b, float c) {
-    float r;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
-
-template <>
-struct Region<Sphere> {
-    float3 lo, hi;  // the box of the centres
-    float r2;       // the largest squared radius
-    // `use`: this lane's query belongs to the packet (warp-wide call)
-    __device__ __forceinline__ void gather(const Sphere &s, bool use) {
-        const float inf = __int_as_float(0x7f800000);
-        lo = make_float3(warp_min(use ? s.c.x : inf), warp_min(use ? s.c.y : inf), warp_min(use ? s.c.z : inf));
-        hi = make_float3(warp_max(use ? s.c.x : -inf), warp_max(use ? s.c.y : -inf), warp_max(use ? s.c.z : -inf));
-        r2 = warp_max(use ? s.r2 : 0.0f);
-    }
-    // A query that can hit nothing (it would only blow the region up).
-    static __device__ __forceinline__ bool hopeless(const Sphere &s) {
-        return isnan(s.c.x) || isnan(s.c.y) || isnan(s.c.z) || isnan(s.r2);
-    }
-    // The queries overlap enough that the region is not much more than one
-    // query's own: the centres spread over at most 4 radii.
-    __device__ __forceinline__ bool tight() const {
-        const float e = fmaxf(hi.x - lo.x, fmaxf(hi.y - lo.y, hi.z - lo.z));
-        return e * e <= 16.0f * r2;
-    }
-    // The gap between the boxes per axis, max(blo - hi, lo - bhi, 0), then d2
-    // as hits() forms it.
-    __device__ __forceinline__ bool meets(float3 blo, float3 bhi) const {
-        float ax, ay, bx, by;
-        unpack2(add2(pack2(blo.x, blo.y), pack2(-hi.x, -hi.y)), ax, ay);
-        unpack2(fma2(pack2(bhi.x, bhi.y), pack2(-1.0f, -1.0f), pack2(lo.x, lo.y)), bx, by);
-        const float ex = max3(ax, bx, 0.0f), ey = max3(ay, by, 0.0f);
-        const float ez = max3(__fsub_rn(blo.z, hi.z), __fsub_rn(lo.z, bhi.z), 0.0f);
-        return __fmaf_rn(ez, ez, __fmaf_rn(ey, ey, __fmul_rn(ex, ex))) <= r2;
-    }
-};
-
-template <>
-struct Region<Box> {
-    Box u;          // the union of the query boxes
-    float3 size;    // the largest extent of one of them
-    __device__ __forceinline__ void gather(const Box &q, bool use) {
-        const float inf = __int_as_float(0x7f800000);
-        u.lo = make_float3(warp_min(use ? q.lo.x : inf), warp_min(use ? q.lo.y : inf), warp_min(use ? q.lo.z : inf));
-        u.hi = make_float3(warp_max(use ? q.hi.x : -inf), warp_max(use ? q.hi.y : -inf),
-                           warp_max(use ? q.hi.z : -inf));
-        size = make_float3(warp_max(use ? q.hi.x - q.lo.x : 0.0f), warp_max(use ? q.hi.y - q.lo.y : 0.0f),
-                           warp_max(use ? q.hi.z - q.lo.z : 0.0f));
-    }
-    static __device__ __forceinline__ bool hopeless(const Box &q) {
-        return isnan(q.lo.x) || isnan(q.lo.y) || isnan(q.lo.z) || isnan(q.hi.x) || isnan(q.hi.y) || isnan(q.hi.z);
-    }
-    __device__ __forceinline__ bool tight() const {
-        return u.hi.x - u.lo.x <= 3.0f * size.x && u.hi.y - u.lo.y <= 3.0f * size.y &&
-               u.hi.z - u.lo.z <= 3.0f * size.z;
-    }
-    __device__ __forceinline__ bool meets(float3 blo, float3 bhi) const { return hits(u, blo, bhi); }
-};
-
-// ---------------------------------------------------------------- packets
-
-constexpr int kPacketWarps = 4;
-// CTAs per SM: points at 32 registers and full occupancy (walk of 2^25 uniform
-// points 7.64 ms, 8.97 with 12 CTAs at 40 registers), boxes at 40 (2^25 boxes
-// 8.30 ms, 8.56 at 32).
-template <int kP>
-constexpr int kPacketCtas = kP == LBVH_PRIM_POINTS ? 16 : 12;
-// Stack of a packet: a step takes four blocks (at most 28 more entries than
-// before) up to kStackFour entries and one block beyond, which adds at most
-// 7 entries for each of the 8 heights below the root's children and 8 at the
-// end: 48 - 4 + 32 + 7 * 8 + 8 = 140 at most.
-constexpr int kStack = 144, kStackFour = 48;
-constexpr int kLeafList = 256;   // leaf blocks waiting to be read
-constexpr int kCand = 64;        // candidate ring: a full set of 32 and the one being filled
-
-// 16-byte alignment: the candidates are read four at a time, and a CTA holds one of these per warp.
-template <int kP>
-struct alignas(16) PacketSmem {
-    static constexpr int kDim = kP == LBVH_PRIM_POINTS ? 3 : 6;
-    float cand[kDim][kCand];
-    uint32_t id[kCand];
-    uint32_t list[kStack + kLeafList];  // the stack, then the leaf blocks
-};
-static_assert(sizeof(PacketSmem<LBVH_PRIM_POINTS>) % 16 == 0 && sizeof(PacketSmem<LBVH_PRIM_BOXES>) % 16 == 0 &&
-                  (kCand * sizeof(float)) % 16 == 0,
-              "rows of candidates start on 16-byte boundaries");
-
-// The lane's query against the 32 candidates at `base` of the ring: bit 31 - j
-// = hit of candidate j. For a sphere and points, the gap c - clamp(c, p, p) is
-// c - p, taken as p - c (the same magnitude, squared), two candidates per
-// instruction; the sign of r2 - d2 says d2 > r2 exactly, and it is shifted
-// into the mask (an infinite d2 against an infinite r2 gives the canonical
-// NaN, whose sign is clear: a hit, as d2 <= r2).
-template <int kP>
-__device__ __forceinline__ uint32_t test32(const PacketSmem<kP> &sm, int base, const Sphere &q) {
-    if constexpr (kP == LBVH_PRIM_POINTS) {
-        uint32_t miss = 0;
-        const uint64_t nx = pack2(-q.c.x, -q.c.x), ny = pack2(-q.c.y, -q.c.y), nz = pack2(-q.c.z, -q.c.z);
-        const uint64_t r2 = pack2(q.r2, q.r2), neg = pack2(-1.0f, -1.0f);
-#pragma unroll
-        for (int j = 0; j < 32; j += 4) {
-            const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(&sm.cand[0][base + j]);
-            const ulonglong2 y = *reinterpret_cast<const ulonglong2 *>(&sm.cand[1][base + j]);
-            const ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(&sm.cand[2][base + j]);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const uint64_t ex = add2(h ? x.y : x.x, nx), ey = add2(h ? y.y : y.x, ny), ez = add2(h ? z.y : z.x, nz);
-                float a, b;
-                unpack2(fma2(fma2(ez, ez, fma2(ey, ey, mul2(ex, ex))), neg, r2), a, b);
-                miss = __funnelshift_l(__float_as_uint(a), miss, 1);
-                miss = __funnelshift_l(__float_as_uint(b), miss, 1);
-            }
-        }
-        return ~miss;
-    } else {
-        uint32_t mask = 0;
-#pragma unroll 8
-        for (int j = 0; j < 32; ++j) {
-            const float3 lo = make_float3(sm.cand[0][base + j], sm.cand[1][base + j], sm.cand[2][base + j]);
-            const float3 hi = make_float3(sm.cand[3][base + j], sm.cand[4][base + j], sm.cand[5][base + j]);
-            if (hits(q, lo, hi)) mask |= 0x80000000u >> j;
-        }
-        return mask;
-    }
-}
-
-// A box: q.lo <= hi and lo <= q.hi on every axis, as the signs of hi - q.lo
-// and q.hi - lo (exact under rounding), two candidates per instruction; one
-// sign bit set is a miss.
-template <int kP>
-__device__ __forceinline__ uint32_t test32(const PacketSmem<kP> &sm, int base, const Box &q) {
-    constexpr int kHi = kP == LBVH_PRIM_POINTS ? 0 : 3;
-    const float ql[3] = {q.lo.x, q.lo.y, q.lo.z}, qh[3] = {q.hi.x, q.hi.y, q.hi.z};
-    const uint64_t neg = pack2(-1.0f, -1.0f);
-    uint32_t miss = 0;
-#pragma unroll
-    for (int j = 0; j < 32; j += 4) {
-        uint32_t s[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const ulonglong2 lo = *reinterpret_cast<const ulonglong2 *>(&sm.cand[d][base + j]);
-            const ulonglong2 hi = kHi ? *reinterpret_cast<const ulonglong2 *>(&sm.cand[kHi + d][base + j]) : lo;
-            const uint64_t nl = pack2(-ql[d], -ql[d]), h = pack2(qh[d], qh[d]);
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                float a, b, c, e;
-                unpack2(add2(k ? hi.y : hi.x, nl), a, b);
-                unpack2(fma2(k ? lo.y : lo.x, neg, h), c, e);
-                s[2 * k] |= __float_as_uint(a) | __float_as_uint(c);
-                s[2 * k + 1] |= __float_as_uint(b) | __float_as_uint(e);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) miss = __funnelshift_l(s[k], miss, 1);
-    }
-    return ~miss;
-}
+// ---------------------------------------------------------------- range queries
 
 // A lane's query in a packet: its hits so far and its spill chunk. Hits go to
 // the slot four at a time (one 16-byte store; words past the count are never
@@ -452,6 +237,9 @@ __device__ __forceinline__ uint32_t test32(const PacketSmem<kP> &sm, int base, c
 // sector of its own (walk of 2^25 uniform points: 11.96 ms with single
 // stores, 9.01 with pairs, 8.97 with fours, at 12 CTAs per SM each).
 struct Keeper {
+    static constexpr int kMaxBlocks = 0;  // every list is taken whole
+    const QueryScratch &qs;
+    Control *ctl;
     uint32_t *slot;
     int64_t qi;
     uint32_t cnt, cur, h0, h1, h2;  // h0, h1, h2: the last three hits
@@ -471,7 +259,30 @@ struct Keeper {
         if (r >= 2) __stcs(slot + cnt - 2, h1);
         if (r >= 3) __stcs(slot + cnt - 3, h0);
     }
-    __device__ __forceinline__ void finish(const QueryScratch &qs, Control *ctl) const {
+    template <int kP, typename Q>
+    __device__ __forceinline__ void take(uint32_t m, const PacketSmem<kP> &sm, int ring, const Q &) {
+        const uint32_t *ids = sm.id + ring + 31;
+        const bool room = !__any_sync(kFull, cnt + __popc(m) > (uint32_t)kSlot);
+        if (room) {
+            while (m) {
+                const int b = 31 - __clz(m);
+                m ^= 1u << b;
+                keep(ids[-b]);
+            }
+        } else {  // a lane's hits run past its slot
+            while (m) {
+                const int b = 31 - __clz(m);
+                m ^= 1u << b;
+                if (cnt < (uint32_t)kSlot) {
+                    keep(ids[-b]);
+                } else {
+                    spill_put(qs, ctl, qi, cnt, ids[-b], cur);
+                    ++cnt;
+                }
+            }
+        }
+    }
+    __device__ __forceinline__ void finish() const {
         drain();
         __stcs(qs.counts + qi, cnt);  // streamed: keep L2 for the tree
         if (cnt > (uint32_t)kSlot)
@@ -479,172 +290,6 @@ struct Keeper {
                 (uint32_t)qi | (cur != kSpillFailed ? kSpilledTag : 0u);
     }
 };
-
-// The packet of the lanes with `use` set walks one tree. False, with nothing
-// kept: its region is not tight and either more than kLeafList - 32 leaf
-// blocks meet it, or must_be_tight is set. Warp-wide.
-template <int kQ, int kP>
-__device__ __forceinline__ bool packet_walk(const Blocks &t, PacketSmem<kP> &sm, const typename QueryOf<kQ>::type &q,
-                                            bool use, bool must_be_tight, const QueryScratch &qs, Control *ctl,
-                                            Keeper &k) {
-    using Q = typename QueryOf<kQ>::type;
-    const int lane = threadIdx.x & 31, sub = lane >> 3;
-    const uint32_t below = (1u << lane) - 1u;
-    Region<Q> region;
-    use = use && !Region<Q>::hopeless(q);
-    if (!__any_sync(kFull, use)) return true;
-    region.gather(q, use);
-    const bool tight = region.tight();
-    if (must_be_tight && !tight) return false;
-    int ns = 0, nl = 0;      // entries of the stack and of the leaf list
-    int ring = 0, nc = 0;    // candidates: the set of 32 being filled starts at `ring`
-    bool fresh = true;       // no leaf block has been read yet
-    if (lane == 0) sm.list[t.start0 ? 0 : kStack] = 0u;
-    if (t.start0) ns = 1;
-    else nl = 1;
-    __syncwarp();
-    // tests the full (or, at the end, last) set of candidates
-    auto flush = [&](int count) {
-        uint32_t m = test32<kP>(sm, ring, q);
-        if (count < 32) m &= ~(kFull >> count);
-        if (!use) m = 0;
-        const uint32_t *ids = sm.id + ring + 31;
-        const bool room = !__any_sync(kFull, k.cnt + __popc(m) > (uint32_t)kSlot);
-        if (room) {
-            while (m) {
-                const int b = 31 - __clz(m);
-                m ^= 1u << b;
-                k.keep(ids[-b]);
-            }
-        } else {  // a lane's hits run past its slot
-            while (m) {
-                const int b = 31 - __clz(m);
-                m ^= 1u << b;
-                if (k.cnt < (uint32_t)kSlot) {
-                    k.keep(ids[-b]);
-                } else {
-                    spill_put(qs, ctl, k.qi, k.cnt, ids[-b], k.cur);
-                    ++k.cnt;
-                }
-            }
-        }
-    };
-    while (true) {
-        // ---- blocks: until the leaf list could overflow in the next step
-        while (ns > 0 && nl <= kLeafList - 32) {
-            const int take = ns > kStackFour ? 1 : min(4, ns);
-            ns -= take;
-            bool hit = false;
-            uint32_t child = 0;
-            if (sub < take) {
-                child = sm.list[ns + sub] * kFan + 1u + (lane & 7);
-                float4 a, b;
-                ld_node32(t.rec + 2 * (int64_t)child, a, b);
-                hit = region.meets(xyz(a), xyz(b)) && __float_as_uint(b.w) == kBlockExists;
-            }
-            const bool leaf = child >= t.start0;
-            const uint32_t inner = __ballot_sync(kFull, hit && !leaf), leafs = __ballot_sync(kFull, hit && leaf);
-            if (hit) sm.list[(leaf ? kStack + nl : ns) + __popc((leaf ? leafs : inner) & below)] = child;
-            ns += __popc(inner);
-            nl += __popc(leafs);
-            __syncwarp();
-        }
-        if (ns > 0 && fresh && !tight) return false;
-        fresh = false;
-        // ---- leaves
-        while (nl > 0) {
-            const int take = min(4, nl);
-            nl -= take;
-            bool in = false;
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-            if (sub < take) {
-                const int pos = (int)(sm.list[kStack + nl + sub] - t.start0) * kFan + (lane & 7);
-                if (pos < t.n) {
-                    if (kP == LBVH_PRIM_BOXES) {
-                        ld_node32(t.leaves + 2 * (int64_t)pos, a, b);
-                    } else {
-                        a = __ldg(t.leaves + pos);
-                        b = a;
-                    }
-                    in = region.meets(leaf_lo<kP>(a, b), leaf_hi<kP>(a, b));
-                }
-            }
-            const uint32_t got = __ballot_sync(kFull, in);
-            if (in) {
-                const int at = (ring + nc + __popc(got & below)) & (kCand - 1);
-                sm.cand[0][at] = a.x;
-                sm.cand[1][at] = a.y;
-                sm.cand[2][at] = a.z;
-                if constexpr (kP == LBVH_PRIM_BOXES) {
-                    sm.cand[3][at] = b.x;
-                    sm.cand[4][at] = b.y;
-                    sm.cand[5][at] = b.z;
-                }
-                sm.id[at] = __float_as_uint(a.w) & kLeafIndexMask;
-            }
-            nc += __popc(got);
-            __syncwarp();
-            if (nc >= 32) {
-                flush(32);
-                ring ^= 32;
-                nc -= 32;
-                __syncwarp();
-            }
-        }
-        if (ns == 0) break;
-    }
-    if (nc > 0) flush(nc);
-    __syncwarp();
-    return true;
-}
-
-__device__ __forceinline__ float3 middle(const Sphere &s) { return s.c; }
-__device__ __forceinline__ float3 middle(const Box &b) {
-    return make_float3(b.lo.x + b.hi.x, b.lo.y + b.hi.y, b.lo.z + b.hi.z);
-}
-
-// The lanes of `mine` before its widest step from one query to the next (the
-// order is a Morton curve: it jumps now and then, and a packet that holds a
-// jump is two packets far apart). `mine` is a run of lanes, two at least.
-template <typename Q>
-__device__ __forceinline__ uint32_t before_jump(const Q &q, uint32_t mine) {
-    const int lane = threadIdx.x & 31;
-    const float3 c = middle(q);
-    const float dx = c.x - __shfl_up_sync(kFull, c.x, 1), dy = c.y - __shfl_up_sync(kFull, c.y, 1),
-                dz = c.z - __shfl_up_sync(kFull, c.z, 1);
-    const float d = fmaxf(fabsf(dx), fmaxf(fabsf(dy), fabsf(dz)));
-    const bool step = ((mine >> lane) & 1u) && lane > __ffs(mine) - 1;
-    const float widest = warp_max(step && d >= 0.0f ? d : 0.0f);
-    const uint32_t at = __ballot_sync(kFull, step && d == widest);
-    const int cut = at ? __ffs(at) - 1 : __ffs(mine);
-    return mine & ((1u << cut) - 1u);
-}
-
-// The queries of `mine` (a run of lanes of one tree): as one packet, or as
-// two on either side of the widest jump. Returns the lanes left over, whose
-// queries lie too far apart.
-template <int kQ, int kP>
-__device__ __forceinline__ uint32_t packets(const Blocks &t, PacketSmem<kP> &sm, const typename QueryOf<kQ>::type &q,
-                                            uint32_t mine, const QueryScratch &qs, Control *ctl, Keeper &k) {
-    const int lane = threadIdx.x & 31;
-    uint32_t cur = mine, next = 0, left = 0;
-    bool whole = true;
-    while (cur) {
-        if (!packet_walk<kQ, kP>(t, sm, q, (cur >> lane) & 1u, false, qs, ctl, k)) {
-            if (whole && __popc(cur) > 1) {
-                const uint32_t first = before_jump(q, cur);
-                next = cur & ~first;
-                cur = first;
-                whole = false;
-                continue;
-            }
-            left |= cur;
-        }
-        cur = next;
-        next = 0;
-    }
-    return left;
-}
 
 template <int kQ, int kP>
 __global__ void __launch_bounds__(32 * kPacketWarps, kPacketCtas<kP>)
@@ -658,15 +303,15 @@ __global__ void __launch_bounds__(32 * kPacketWarps, kPacketCtas<kP>)
     if (w * 32 >= qa.nq) return;
     const bool has = i < qa.nq;
     const int64_t qi = has ? thread_query(qa, i) : 0;
-    Keeper k{qs.slots + qi * kSlot, qi, 0u, kNoChunk, 0u, 0u, 0u};
+    Keeper k{qs, ctl, qs.slots + qi * kSlot, qi, 0u, kNoChunk, 0u, 0u, 0u};
     uint32_t left = 0;
     if (ctl->build_flags == 0) {
         typename QueryOf<kQ>::type q{};
         if (has) q = QueryOf<kQ>::load(qa, qi);
-        left = packets<kQ, kP>(Blocks{leaves, rec, n, start0}, sm, q, __ballot_sync(kFull, has), qs, ctl, k);
+        left = packets<kQ, kP>(Blocks{leaves, rec, n, start0}, sm, q, __ballot_sync(kFull, has), k);
         if (left && lane == 0) qs.sparse_list[atomicAdd(&ctl->sparse_filled, 1u)] = make_uint2((uint32_t)w, left);
     }
-    if (has && !((left >> lane) & 1u)) k.finish(qs, ctl);
+    if (has && !((left >> lane) & 1u)) k.finish();
 }
 
 // Batches: the same, on the tree of the queries' instance; the instances of a
@@ -683,7 +328,7 @@ __global__ void __launch_bounds__(32 * kPacketWarps, kPacketCtas<kP>)
     if (w * 32 >= qa.nq) return;
     const bool has = i < qa.nq;
     const int64_t qi = has ? thread_query(qa, i) : 0;
-    Keeper k{qs.slots + qi * kSlot, qi, 0u, kNoChunk, 0u, 0u, 0u};
+    Keeper k{qs, ctl, qs.slots + qi * kSlot, qi, 0u, kNoChunk, 0u, 0u, 0u};
     uint32_t left = 0;
     if (ctl->build_flags == 0) {
         typename QueryOf<kQ>::type q{};
@@ -697,11 +342,11 @@ __global__ void __launch_bounds__(32 * kPacketWarps, kPacketCtas<kP>)
             const int64_t n = bt.prim_off[b + 1] - bt.prim_off[b];
             if (n <= 0) continue;
             const Blocks t{nodes + bt.node_start[b] + 2 * (n - 1), rec + 2 * bt.pack_start[b], (int)n, pack_leaf_start(n)};
-            left |= packets<kQ, kP>(t, sm, q, mine, qs, ctl, k);
+            left |= packets<kQ, kP>(t, sm, q, mine, k);
         }
         if (left && lane == 0) qs.sparse_list[atomicAdd(&ctl->sparse_filled, 1u)] = make_uint2((uint32_t)w, left);
     }
-    if (has && !((left >> lane) & 1u)) k.finish(qs, ctl);
+    if (has && !((left >> lane) & 1u)) k.finish();
 }
 
 // ---------------------------------------------------------------- 8 lanes per query

@@ -147,3 +147,52 @@ def test_batch_of_small_and_empty_instances():
         assert np.array_equal(bhits[boff[a]:boff[e]], h)
         t.close()
     batch.close()
+
+
+def knn_both(tree, q, k):
+    """k nearest in packets (all queries at once) and one thread per query (pieces too small for packets)."""
+    idx, d2 = tree.knn(q, k)
+    step = 5000
+    want = [tree.knn(q[a:a + step], k) for a in range(0, len(q), step)]
+    assert torch.equal(idx, torch.cat([w[0] for w in want]))
+    assert torch.equal(d2, torch.cat([w[1] for w in want]))
+
+
+@pytest.mark.parametrize("kind", ["points", "boxes"])
+@pytest.mark.parametrize("k", [1, 3, 4, 5, 8, 9, 16, 17, 32])
+def test_knn_packets_other_queries(k, kind):
+    lbvh = L()
+    nq = 40_001
+    for n in (1024, 4097, 60_001):
+        pts = inputs.gaussian_mixture_points(n, seed=n + k, components=6, sigma=0.05)
+        q = np.concatenate([inputs.gaussian_mixture_points(nq - 3000, seed=n + k, components=6, sigma=0.06),
+                            inputs.uniform_points(3000, seed=k)])
+        q[7::991, 0], q[8::991, 1], q[9::991, 2] = np.nan, np.inf, -np.inf
+        t = lbvh.Tree().build(pts if kind == "points" else boxes_at(pts, 0.002),
+                              lbvh.POINTS if kind == "points" else lbvh.BOXES, 63 if n > 5000 else 30)
+        knn_both(t, torch.from_numpy(q).cuda(), k)
+        t.close()
+
+
+@pytest.mark.parametrize("k", [2, 16, 31])
+def test_knn_packets_own_points_ties_and_duplicates(k):
+    lbvh = L()
+    for pts in (inputs.uniform_points(30_011, seed=1), inputs.duplicated_points(30_011, 700, seed=2),
+                np.round(inputs.uniform_points(30_011, seed=3) * 24).astype(np.float32),  # a lattice: equal distances
+                np.full((12_000, 3), 0.5, np.float32)):
+        p = torch.from_numpy(pts).cuda()
+        t = lbvh.Tree().build(p, lbvh.POINTS, 63)
+        knn_both(t, p, k)
+        t.close()
+
+
+def test_knn_packets_in_chunks_without_distances():
+    lbvh = L()
+    n = (1 << 20) + 77  # more than one chunk of queries
+    p = torch.from_numpy(inputs.uniform_points(n, seed=4)).cuda()
+    t = lbvh.Tree().build(p, lbvh.POINTS, 30)
+    idx, none = t.knn(p, 8, distances=False)
+    assert none is None
+    for a in (0, 524_288, n - 3000):
+        assert torch.equal(idx[a:a + 3000], t.knn(p[a:a + 3000].contiguous(), 8)[0])
+    t.close()
