@@ -1325,18 +1325,24 @@ lbvh_status lbvh_knn(lbvh_tree_t t, const float *d_queries, int64_t nq, int k, u
     // a lean (server-resident) tree keeps no sorted codes: its walks start
     // without seeds, which is exact but slower
     const uint64_t *codes = t->lean ? nullptr : t->sorted_codes();
-    const bool packets = codes && t->bits > 0 && !t->loaded && knn_in_packets(nq, t->n, k);
+    KnnWalk how = codes && t->bits > 0 && !t->loaded ? knn_walk(nq, t->n, k, own_order(t, qa)) : kKnnHeap;
+    if (how == kKnnSparse && !t->packed_ok && t->n > kPackForFew && !t->few_seen) {  // as in query_count
+        t->few_seen = true;
+        how = kKnnHeap;
+    }
     // the order of the query points
-    lbvh_status st = query_order(t, qa, s, order_bits(), packets ? kCodeHilbert : kCodeLow);
+    lbvh_status st = LBVH_OK;
+    if (how != kKnnSparse || own_order(t, qa))
+        st = query_order(t, qa, s, order_bits(), how == kKnnPackets ? kCodeHilbert : kCodeLow);
     t->prof.end(LBVH_STAGE_QORDER, s);
     if (st != LBVH_OK) return st;
     const bool own = qa.order && own_order(t, qa);
     KnnScratch sc{};
     bool pack = false;
-    if (packets) {
+    if (how != kKnnHeap) {
         sc.chunk = knn_chunk(nq);
-        LBVH_CUDA(t->slots.ensure((size_t)sc.chunk * knn_slot_bytes(k), s));
         const int64_t chunks = (nq + sc.chunk - 1) / sc.chunk;
+        if (how == kKnnPackets) LBVH_CUDA(t->slots.ensure((size_t)sc.chunk * knn_slot_bytes(k), s));
         LBVH_CUDA(t->counts.ensure((size_t)(3 * sc.chunk + chunks) * 4, s));
         pack = !t->packed_ok;
         if (pack) LBVH_CUDA(t->packed.ensure((size_t)pack_records(t->n) * 32, s));
@@ -1347,10 +1353,10 @@ lbvh_status lbvh_knn(lbvh_tree_t t, const float *d_queries, int64_t nq, int k, u
         sc.redo_counts = sc.counts + 3 * sc.chunk;
     }
     t->prof.begin(LBVH_STAGE_QCOUNT, s);  // the kNN walk is timed as the query walk
-    if (packets) {
+    if (how != kKnnHeap) {
         if (pack) launch_pack(t->view(), t->packed.as<float4>(), c, s);
-        launch_knn_packets(t->view(), t->packed.as<float4>(), codes, t->bounds.as<float>(), t->bits, qa, own, k, sc, d_idx,
-                           d_dist2, c, s);
+        launch_knn_packets(t->view(), t->packed.as<float4>(), codes, t->bounds.as<float>(), t->bits, qa, own, k, how, sc,
+                           d_idx, d_dist2, c, s);
     } else {
         launch_knn(t->view(), codes, t->bounds.as<float>(), t->bits, qa, k, d_idx, d_dist2, c, s);
     }

@@ -423,13 +423,13 @@ __device__ __forceinline__ int keep_smallest(uint64_t *keys, int cnt, int k, int
 // sparse_walk; they are too few and too far apart for packets), to the end:
 // the hits' keys are gathered in shared memory, cut back to the k smallest
 // whenever they could overrun, and the k-th of those is the new bound. A fixed
-// grid strides over the list.
+// grid strides over the list (redo null: over all queries).
 template <int kP, int kK>
 __global__ void __launch_bounds__(128)
     knn_redo_kernel(const float4 *__restrict__ leaves, const float4 *__restrict__ rec, int n, uint32_t start0,
                     QueryArgs qa, int k, int64_t first, int64_t count, const float *__restrict__ radii2,
                     const uint32_t *__restrict__ redo, const uint32_t *redo_count, uint32_t *__restrict__ out_idx,
-                    float *__restrict__ out_d2) {
+                    float *__restrict__ out_d2, const Control *ctl) {
     constexpr int kCap = kKnnMul<kK> * kK;
     __shared__ uint32_t s_stack[128 / 8][kSparseStack];
     __shared__ uint64_t s_keys[128 / 8][kCap];
@@ -437,16 +437,17 @@ __global__ void __launch_bounds__(128)
     uint64_t *keys = s_keys[threadIdx.x >> 3];
     const int lane = threadIdx.x & 31, sl = lane & 7, shift = lane & 24;
     const uint32_t below = (1u << sl) - 1u;
-    const int64_t total = min((int64_t)*redo_count, count);
+    const int64_t total = redo ? min((int64_t)*redo_count, count) : count;
+    const bool built = ctl->build_flags == 0;
     const int64_t stride = ((int64_t)gridDim.x * 128) >> 5;
     for (int64_t g = ((int64_t)blockIdx.x * 128 + threadIdx.x) >> 5; 4 * g < total; g += stride) {
         const bool go = 4 * g + (lane >> 3) < total;
-        const int64_t j = go ? redo[4 * g + (lane >> 3)] : 0;
+        const int64_t j = !go ? 0 : redo ? redo[4 * g + (lane >> 3)] : 4 * g + (lane >> 3);
         const int64_t qi = thread_query(qa, first + j);
         const float3 c =
             make_float3(__ldg(qa.queries + 3 * qi), __ldg(qa.queries + 3 * qi + 1), __ldg(qa.queries + 3 * qi + 2));
         float r2 = radii2[j];
-        int cnt = 0, ns = go ? 1 : 0;
+        int cnt = 0, ns = go && built ? 1 : 0;
         if (sl == 0) stack[0] = 0u;
         __syncwarp();
         while (__any_sync(kFull, ns > 0)) {
@@ -612,8 +613,17 @@ int knn_class(int k) { return k <= 8 ? 8 : k <= 16 ? 16 : 32; }
 
 template <int kP, int kK>
 void knn_chunks(const TreeView &t, const float4 *rec, const uint64_t *codes, const float *bounds, int bits,
-                const QueryArgs &q, bool own, int k, const KnnScratch &sc, uint32_t *out_idx, float *out_d2, Control *ctl,
-                cudaStream_t s) {
+                const QueryArgs &q, bool own, int k, KnnWalk how, const KnnScratch &sc, uint32_t *out_idx, float *out_d2,
+                Control *ctl, cudaStream_t s) {
+    const int64_t redo_grid = (int64_t)device_sm_count() * 12;
+    if (how == kKnnSparse) {  // one chunk: the bounds, then 8 lanes for every query
+        knn_radius_kernel<kP, kK><<<(unsigned)((q.nq + 127) / 128), 128, 0, s>>>(t, codes, bounds, bits, q, k, 0, q.nq, own,
+                                                                                 sc.radii2, ctl);
+        knn_redo_kernel<kP, kK><<<(unsigned)std::min<int64_t>((q.nq + 15) / 16, redo_grid), 128, 0, s>>>(
+            t.leaves, rec, (int)t.n, pack_leaf_start(t.n), q, k, 0, q.nq, sc.radii2, nullptr, nullptr, out_idx, out_d2, ctl);
+        count_launches(2);
+        return;
+    }
     cudaMemsetAsync(sc.redo_counts, 0, (size_t)((q.nq + sc.chunk - 1) / sc.chunk) * 4, s);
     const uint32_t start0 = pack_leaf_start(t.n);
     for (int64_t first = 0; first < q.nq; first += sc.chunk) {
@@ -626,32 +636,43 @@ void knn_chunks(const TreeView &t, const float4 *rec, const uint64_t *codes, con
         uint32_t *redo_count = sc.redo_counts + first / sc.chunk;
         knn_select_kernel<kK><<<blocks, 128, 0, s>>>(q, k, first, count, sc.slots, sc.counts, sc.radii2, sc.redo, redo_count,
                                                      out_idx, out_d2, ctl);
-        knn_redo_kernel<kP, kK><<<(unsigned)std::min<int64_t>((count + 15) / 16, (int64_t)device_sm_count() * 12), 128, 0,
+        knn_redo_kernel<kP, kK><<<(unsigned)std::min<int64_t>((count + 15) / 16, redo_grid), 128, 0,
                                   s>>>(t.leaves, rec, (int)t.n, start0, q, k, first, count, sc.radii2, sc.redo, redo_count,
-                                       out_idx, out_d2);
+                                       out_idx, out_d2, ctl);
         count_launches(4);
     }
 }
 
 }  // namespace
 
-bool knn_in_packets(int64_t nq, int64_t n, int k) {
-    return k >= 5 && k <= kKnnPacketK && n >= 1024 && n <= 4 * nq && nq >= 64 * (int64_t)device_sm_count();
+// 8 lanes per query against the heap (its query order included; us): 100,003
+// uniform points, 10,000 queries, k = 3: 57 / 127, k = 32: 143 / 406;
+// 3.0M points, 30,000 queries, k = 3: 114 / 152, k = 16: 179 / 427; 77,000
+// queries, k = 3: 229 / 193, k = 16: 389 / 519; 150,000, k = 16: about equal.
+// 9,001 points as their own queries (the order is free), k = 1: 31 / 18, k = 3:
+// 47 / 57.
+KnnWalk knn_walk(int64_t nq, int64_t n, int k, bool sorted) {
+    const int64_t sms = device_sm_count();
+    if (k > kKnnPacketK || n < 1024) return kKnnHeap;
+    const bool dense = n <= 4 * nq;
+    if (k >= 5 && dense && nq >= 64 * sms) return kKnnPackets;
+    const int64_t few = k <= 2 && sorted ? 0 : dense ? 64 : k >= 5 ? 512 : 256;
+    return nq <= few * sms ? kKnnSparse : kKnnHeap;
 }
 
 int64_t knn_chunk(int64_t nq) { return std::min<int64_t>(nq, int64_t(1) << 20); }
 size_t knn_slot_bytes(int k) { return (size_t)(k <= 8 ? 8 : 4) * knn_class(k) * sizeof(uint2); }
 
 void launch_knn_packets(const TreeView &t, const float4 *rec, const uint64_t *codes, const float *bounds, int bits,
-                        const QueryArgs &q, bool own, int k, const KnnScratch &sc, uint32_t *out_idx, float *out_d2,
-                        Control *ctl, cudaStream_t s) {
+                        const QueryArgs &q, bool own, int k, KnnWalk how, const KnnScratch &sc, uint32_t *out_idx,
+                        float *out_d2, Control *ctl, cudaStream_t s) {
     if (q.nq <= 0) return;
     auto go = [&](auto kk) {
         constexpr int K = decltype(kk)::value;
         if (t.kind == LBVH_PRIM_POINTS)
-            knn_chunks<LBVH_PRIM_POINTS, K>(t, rec, codes, bounds, bits, q, own, k, sc, out_idx, out_d2, ctl, s);
+            knn_chunks<LBVH_PRIM_POINTS, K>(t, rec, codes, bounds, bits, q, own, k, how, sc, out_idx, out_d2, ctl, s);
         else
-            knn_chunks<LBVH_PRIM_BOXES, K>(t, rec, codes, bounds, bits, q, own, k, sc, out_idx, out_d2, ctl, s);
+            knn_chunks<LBVH_PRIM_BOXES, K>(t, rec, codes, bounds, bits, q, own, k, how, sc, out_idx, out_d2, ctl, s);
     };
     switch (knn_class(k)) {
     case 8: go(std::integral_constant<int, 8>{}); break;

@@ -343,10 +343,15 @@ constexpr int kKnnMaxK = 256;
 void launch_visits(const TreeView &t, const QueryArgs &q, unsigned long long *counts, Control *ctl, cudaStream_t s);
 void launch_knn(const TreeView &t, const uint64_t *codes, const float *bounds, int bits, const QueryArgs &q, int k,
                 uint32_t *out_idx, float *out_d2, Control *ctl, cudaStream_t s);
-// The same in packets (knn.cu): whether they pay for nq queries on n leaves,
-// and the scratch of a call: walked in chunks of `chunk` queries.
+// The same through the leaf blocks (knn.cu): how nq queries on n leaves walk,
+// and the scratch of a call (packets: in chunks of `chunk` queries).
 constexpr int kKnnPacketK = 32;
-bool knn_in_packets(int64_t nq, int64_t n, int k);
+enum KnnWalk : int {
+    kKnnHeap,     // Algorithm 1, a thread per query (launch_knn)
+    kKnnPackets,  // packets of 32 neighbours, which want a query order
+    kKnnSparse    // 8 lanes per query, in any order
+};
+KnnWalk knn_walk(int64_t nq, int64_t n, int k, bool sorted);
 int64_t knn_chunk(int64_t nq);
 size_t knn_slot_bytes(int k);  // per query of a chunk
 struct KnnScratch {
@@ -360,8 +365,8 @@ struct KnnScratch {
 // rec: the tree's leaf blocks; own: walk positions are places in the sorted
 // codes (q.order is the tree's permutation). t.n >= 1024.
 void launch_knn_packets(const TreeView &t, const float4 *rec, const uint64_t *codes, const float *bounds, int bits,
-                        const QueryArgs &q, bool own, int k, const KnnScratch &sc, uint32_t *out_idx, float *out_d2,
-                        Control *ctl, cudaStream_t s);
+                        const QueryArgs &q, bool own, int k, KnnWalk how, const KnnScratch &sc, uint32_t *out_idx,
+                        float *out_d2, Control *ctl, cudaStream_t s);
 // offsets[0..nq] = exclusive scan of counts (offsets[nq] = total =
 // ctl->total).
 int64_t scan_tile_count(int64_t nq);

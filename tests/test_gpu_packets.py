@@ -150,12 +150,16 @@ def test_batch_of_small_and_empty_instances():
 
 
 def knn_both(tree, q, k):
-    """k nearest in packets (all queries at once) and one thread per query (pieces too small for packets)."""
+    """k nearest in packets (all queries at once), by 8 lanes per query (pieces too small for packets) and one
+    thread per query (the first columns of 33 neighbours, more than the others take)."""
     idx, d2 = tree.knn(q, k)
     step = 5000
-    want = [tree.knn(q[a:a + step], k) for a in range(0, len(q), step)]
-    assert torch.equal(idx, torch.cat([w[0] for w in want]))
-    assert torch.equal(d2, torch.cat([w[1] for w in want]))
+    few = [tree.knn(q[a:a + step], k) for a in range(0, len(q), step)]
+    assert torch.equal(idx, torch.cat([w[0] for w in few]))
+    assert torch.equal(d2, torch.cat([w[1] for w in few]))
+    want = tree.knn(q, 33)
+    assert torch.equal(idx, want[0][:, :k])
+    assert torch.equal(d2, want[1][:, :k])
 
 
 @pytest.mark.parametrize("kind", ["points", "boxes"])
