@@ -203,8 +203,8 @@ lbvh_status lbvh_tree_export(lbvh_tree_t tree, uint32_t *h_perm, uint64_t *h_sor
  *              t2 = (hi-o)*inv, tnear = max(tmin, min(t1,t2)), tfar =
  *              min(tmax, max(t1,t2)); hit iff tnear <= tfar. A ray with a
  *              non-finite origin or direction, or a NaN tmin/tmax, hits
- *              nothing. Rays are walked in the order given; spheres and boxes
- *              in the Morton order of their centres.
+ *              nothing. The order in which the queries are walked is the
+ *              library's own and changes no result.
  *   d_radii    float[nq] per-query radius, or NULL to use `radius` for all
  *              (`radius` must then be finite and >= 0).
  *   d_offsets  int64[nq+1]: hits of query q are d_hits[d_offsets[q] ..

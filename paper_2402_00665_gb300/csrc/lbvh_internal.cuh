@@ -241,6 +241,10 @@ __host__ __device__ inline int top_run_shift(int index_bits, int skip) {
 void launch_encode(const float *prims, int64_t n, int kind, int bits, const float *bounds,
                    uint64_t *codes, uint32_t *hist, int hist_passes, int layout, int index_bits, cudaStream_t s,
                    int skip = 0);
+// Words code << 32 | i of ray segments (8-bit codes, see encode_rays_kernel)
+// and their histogram (hist[0..256) zero beforehand).
+void launch_encode_rays(const float *rays, int64_t n, const float *bounds, uint64_t *words, uint32_t *hist,
+                        cudaStream_t s);
 // codes[i] = the Morton code of primitive perm[i].
 void launch_sorted_codes(const float *prims, const uint32_t *perm, int64_t n, int kind, int bits,
                          const float *bounds, uint64_t *codes, cudaStream_t s);

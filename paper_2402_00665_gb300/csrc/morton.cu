@@ -206,6 +206,32 @@ __global__ void __launch_bounds__(kThreads)
     }
 }
 
+// The walk order of ray segments: word (code << 32 | i) per ray, its code the
+// first 8 bits of the Hilbert index of the cell that holds the segment's
+// middle (a segment longer than the scene is cut to the scene's extent, cells
+// outside the scene to its border), and the histogram of the codes.
+__global__ void __launch_bounds__(kThreads)
+    encode_rays_kernel(const float4 *__restrict__ rays, int64_t n, const float *__restrict__ bounds,
+                       uint64_t *__restrict__ words, uint32_t *__restrict__ hist) {
+    __shared__ uint32_t s_hist[kRadix], s_hilbert[kHilbertStates * 8];
+    s_hist[threadIdx.x] = 0;  // kThreads == kRadix
+    if (threadIdx.x < kHilbertStates * 8) s_hilbert[threadIdx.x] = kHilbert.next[threadIdx.x];
+    const Grid3 g = make_grid(bounds, 3);
+    const float extent = fmaxf(g.extent[0], fmaxf(g.extent[1], g.extent[2]));
+    __syncthreads();
+    for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kThreads) {
+        const float4 o = rays[2 * i], d = rays[2 * i + 1];
+        const float speed = fmaxf(fabsf(d.x), fmaxf(fabsf(d.y), fabsf(d.z)));
+        const float t = o.w + 0.5f * fminf(d.w - o.w, extent / speed);
+        const uint64_t c = hilbert(o.x + t * d.x, o.y + t * d.y, o.z + t * d.z, g, 3, s_hilbert) >> 1;
+        words[i] = c << 32 | (uint64_t)(uint32_t)i;
+        atomicAdd(&s_hist[(uint32_t)c], 1u);
+    }
+    __syncthreads();
+    const uint32_t v = s_hist[threadIdx.x];
+    if (v) atomicAdd(&hist[threadIdx.x], v);
+}
+
 // The codes of the primitives in sorted order: codes[i] = the code of
 // primitive perm[i] (a gather through the permutation and the same encoding).
 template <int kKind>
@@ -388,6 +414,13 @@ void launch_encode(const float *prims, int64_t n, int kind, int bits, const floa
          encode_kernel<LBVH_PRIM_BOXES, kCodeTop>, encode_kernel<LBVH_PRIM_BOXES, kCodeHilbert>}};
     table[kind == LBVH_PRIM_POINTS ? 0 : 1][layout]<<<blocks, kThreads, 0, s>>>(prims, n, b, bounds, codes, hist,
                                                                                hist_passes, index_bits, skip);
+    count_launches(1);
+}
+
+void launch_encode_rays(const float *rays, int64_t n, const float *bounds, uint64_t *words, uint32_t *hist,
+                        cudaStream_t s) {
+    encode_rays_kernel<<<bounds_blocks(n), kThreads, 0, s>>>(reinterpret_cast<const float4 *>(rays), n, bounds, words,
+                                                            hist);
     count_launches(1);
 }
 

@@ -166,7 +166,13 @@ __device__ __forceinline__ void collect_walk(const TreeView &t, const QueryArgs 
             ++cnt;
         };
         bool ok;
-        if constexpr (kLanes == 0)
+        if constexpr (kLanes == 0 && kQ == LBVH_Q_RAY) {
+            // one instruction stream for the warp: the general test if any of its rays has a parallel axis
+            if (__any_sync(__activemask(), q.parallel != 0))
+                ok = walk<kP>(t, q, keep);
+            else
+                ok = walk<kP>(t, SlantedRay{q}, keep);
+        } else if constexpr (kLanes == 0)
             ok = walk<kP>(t, q, keep);
         else
             ok = walk_group<kP, kLanes>(t, q, has_query, keep);

@@ -7,6 +7,42 @@
 
 namespace lbvh {
 
+// f32x2: two FP32 operations of one instruction, each rounded as its scalar form
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float min3(float a, float b, float c) {
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
 struct Sphere {
     float3 c;
     float r2;
@@ -56,6 +92,21 @@ __device__ __forceinline__ bool hits(const Ray &r, float3 lo, float3 hi) {
     if (!slab(lo.x, hi.x, r.o.x, r.inv.x, r.parallel & 1u, tn, tf)) return false;
     if (!slab(lo.y, hi.y, r.o.y, r.inv.y, r.parallel & 2u, tn, tf)) return false;
     if (!slab(lo.z, hi.z, r.o.z, r.inv.z, r.parallel & 4u, tn, tf)) return false;
+    return tn <= tf;
+}
+
+// A ray without a parallel axis: the same operations on every axis, x and y
+// in one instruction each and the extremes three at a time (they do not
+// depend on the order; no operand is NaN).
+struct SlantedRay : Ray {};
+__device__ __forceinline__ bool hits(const SlantedRay &r, float3 lo, float3 hi) {
+    const uint64_t minus = pack2(-r.o.x, -r.o.y), inv = pack2(r.inv.x, r.inv.y);
+    float ax, ay, bx, by;
+    unpack2(mul2(add2(pack2(lo.x, lo.y), minus), inv), ax, ay);
+    unpack2(mul2(add2(pack2(hi.x, hi.y), minus), inv), bx, by);
+    const float az = __fmul_rn(__fsub_rn(lo.z, r.o.z), r.inv.z), bz = __fmul_rn(__fsub_rn(hi.z, r.o.z), r.inv.z);
+    const float tn = max3(max3(fminf(ax, bx), fminf(ay, by), fminf(az, bz)), r.tmin, r.tmin);
+    const float tf = min3(min3(fmaxf(ax, bx), fmaxf(ay, by), fmaxf(az, bz)), r.tmax, r.tmax);
     return tn <= tf;
 }
 

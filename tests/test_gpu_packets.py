@@ -200,3 +200,23 @@ def test_knn_packets_in_chunks_without_distances():
     for a in (0, 524_288, n - 3000):
         assert torch.equal(idx[a:a + 3000], t.knn(p[a:a + 3000].contiguous(), 8)[0])
     t.close()
+
+
+@pytest.mark.parametrize("nq", [4095, 4096, 30_001])
+def test_ray_order(nq):
+    """Rays are walked by cells of their middles: pieces too small for an order give the same lists, with parallel
+    axes, reversed, unbounded and non-finite segments among them."""
+    lbvh = L()
+    n = 20_000
+    t = lbvh.Tree().build(boxes_at(inputs.uniform_points(n, seed=1), 0.01), lbvh.BOXES, 63)
+    rays = inputs.random_rays(nq, seed=2, tmax=0.3)
+    rays[3::17, 4], rays[4::17, 5:7], rays[5::31, 4:7] = 0.0, 0.0, 0.0
+    rays[6::29, 7], rays[7::29, 3], rays[8::29, 7] = np.inf, -np.inf, -0.1
+    rays[9::101, 0], rays[10::101, 5], rays[11::101, 7], rays[12::101, 4] = np.nan, np.inf, np.nan, 1e-42
+    off, hits = csr(t, rays, lbvh.RAY)
+    assert off[-1] > nq
+    for a in range(0, nq, 4000):
+        o, h = csr(t, rays[a:a + 4000], lbvh.RAY)
+        assert np.array_equal(off[a:a + len(o)] - off[a], o)
+        assert np.array_equal(hits[off[a]:off[a + len(o) - 1]], h)
+    t.close()
