@@ -864,46 +864,54 @@ lbvh_status build_impl(lbvh_tree_t t, const float *d_prims, int64_t n, int kind,
     t->prof.clear(LBVH_STAGE_SECOND, LBVH_STAGE_SECOND + 1);
     t->prof.clear(LBVH_STAGE_SORTRUNS, LBVH_STAGE_SORTRUNS + 1);
     if (n > 0) {
-        const int passes = sort_passes(morton_bits);
-        LBVH_CUDA(cudaMemsetAsync(t->hist.p, 0, (size_t)kMaxPasses * kRadix * 4, s));
-        t->prof.begin(LBVH_STAGE_BOUNDS, s);
-        launch_bounds(d_prims, n, kind, t->partials.as<float>(), t->bounds.as<float>(), c, s);
-        t->prof.end(LBVH_STAGE_BOUNDS, s);
-        LBVH_LAUNCHED();
-        t->prof.begin(LBVH_STAGE_ENCODE, s);
-        // codes of at most 30 bits are packed with the index from the start
-        // (code << 32 | index); wider codes give their top bits (top << ib |
-        // index) to run_code_sort
-        const bool packed = morton_bits <= 30;
-        const int ib = top_index_bits(n);
-        // the sort choice: tile shape, and whether the top-bits sort covers
-        // one byte fewer (more elements in runs of equal sorted bits)
-        const int choice = t->sort_choice >= 0 ? t->sort_choice : tune_sort_choice(n, morton_bits, kind, 1);
-        const int variant = sort_choice_tile(choice);
-        const int skip = packed ? 0 : sort_choice_skip(choice);
-        launch_encode(d_prims, n, kind, morton_bits, t->bounds.as<float>(), t->keys[0].as<uint64_t>(),
-                      t->hist.as<uint32_t>(), 1, packed ? kCodeLow : kCodeTop, ib, s, skip);
-        t->prof.end(LBVH_STAGE_ENCODE, s);
-        LBVH_LAUNCHED();
-        SortScratch scratch{t->hist.as<uint32_t>(), t->lookback.as<uint32_t>(), sort_tiles_max(n) * kRadix};
-        nvtxRangePushA("sort");
-        cudaEvent_t(*pass_events)[2] = t->prof.on ? &t->prof.ev[LBVH_STAGE_SORT0] : nullptr;
-        // the node records are written by the construct only: until then they
-        // hold run_code_sort's 2n scratch words
-        const uint32_t *perm =
-            packed ? run_index_sort(t->keys[0].as<uint64_t>(), t->keys[1].as<uint64_t>(), t->vals[0].as<uint32_t>(),
-                                    n, morton_bits, scratch, c, s, pass_events, variant)
-                   : run_code_sort(d_prims, kind, morton_bits, t->bounds.as<float>(), n, t->keys[0].as<uint64_t>(),
-                                   t->keys[1].as<uint64_t>(), t->vals[0].as<uint32_t>(), t->vals[1].as<uint32_t>(),
-                                   t->nodes.as<uint32_t>(), scratch, c, s, pass_events,
-                                   t->prof.on ? t->prof.ev[LBVH_STAGE_SORTRUNS] : nullptr, variant, skip);
-        nvtxRangePop();
-        if (t->prof.on) {
-            const int sorted = packed ? passes : kMaxPasses - top_first_byte(ib, skip);
-            for (int p = 0; p < sorted; ++p) t->prof.recorded[LBVH_STAGE_SORT0 + p] = true;
-            if (!packed) t->prof.recorded[LBVH_STAGE_SORTRUNS] = true;
+        const uint32_t *perm = t->vals[0].as<uint32_t>();
+        if (n <= small_sort_max(morton_bits) && t->sort_choice < 0) {
+            t->prof.begin(LBVH_STAGE_SORT0, s);
+            launch_small_sort(d_prims, n, kind, morton_bits, t->bounds.as<float>(), t->vals[0].as<uint32_t>(), c, s);
+            t->prof.end(LBVH_STAGE_SORT0, s);
+            LBVH_LAUNCHED();
+        } else {
+            const int passes = sort_passes(morton_bits);
+            LBVH_CUDA(cudaMemsetAsync(t->hist.p, 0, (size_t)kMaxPasses * kRadix * 4, s));
+            t->prof.begin(LBVH_STAGE_BOUNDS, s);
+            launch_bounds(d_prims, n, kind, t->partials.as<float>(), t->bounds.as<float>(), c, s);
+            t->prof.end(LBVH_STAGE_BOUNDS, s);
+            LBVH_LAUNCHED();
+            t->prof.begin(LBVH_STAGE_ENCODE, s);
+            // codes of at most 30 bits are packed with the index from the start
+            // (code << 32 | index); wider codes give their top bits (top << ib |
+            // index) to run_code_sort
+            const bool packed = morton_bits <= 30;
+            const int ib = top_index_bits(n);
+            // the sort choice: tile shape, and whether the top-bits sort covers
+            // one byte fewer (more elements in runs of equal sorted bits)
+            const int choice = t->sort_choice >= 0 ? t->sort_choice : tune_sort_choice(n, morton_bits, kind, 1);
+            const int variant = sort_choice_tile(choice);
+            const int skip = packed ? 0 : sort_choice_skip(choice);
+            launch_encode(d_prims, n, kind, morton_bits, t->bounds.as<float>(), t->keys[0].as<uint64_t>(),
+                          t->hist.as<uint32_t>(), 1, packed ? kCodeLow : kCodeTop, ib, s, skip);
+            t->prof.end(LBVH_STAGE_ENCODE, s);
+            LBVH_LAUNCHED();
+            SortScratch scratch{t->hist.as<uint32_t>(), t->lookback.as<uint32_t>(), sort_tiles_max(n) * kRadix};
+            nvtxRangePushA("sort");
+            cudaEvent_t(*pass_events)[2] = t->prof.on ? &t->prof.ev[LBVH_STAGE_SORT0] : nullptr;
+            // the node records are written by the construct only: until then they
+            // hold run_code_sort's 2n scratch words
+            perm =
+                packed ? run_index_sort(t->keys[0].as<uint64_t>(), t->keys[1].as<uint64_t>(), t->vals[0].as<uint32_t>(),
+                                        n, morton_bits, scratch, c, s, pass_events, variant)
+                       : run_code_sort(d_prims, kind, morton_bits, t->bounds.as<float>(), n, t->keys[0].as<uint64_t>(),
+                                       t->keys[1].as<uint64_t>(), t->vals[0].as<uint32_t>(), t->vals[1].as<uint32_t>(),
+                                       t->nodes.as<uint32_t>(), scratch, c, s, pass_events,
+                                       t->prof.on ? t->prof.ev[LBVH_STAGE_SORTRUNS] : nullptr, variant, skip);
+            nvtxRangePop();
+            if (t->prof.on) {
+                const int sorted = packed ? passes : kMaxPasses - top_first_byte(ib, skip);
+                for (int p = 0; p < sorted; ++p) t->prof.recorded[LBVH_STAGE_SORT0 + p] = true;
+                if (!packed) t->prof.recorded[LBVH_STAGE_SORTRUNS] = true;
+            }
+            LBVH_LAUNCHED();
         }
-        LBVH_LAUNCHED();
         // the sort leaves the permutation alone; the sorted codes go to keys[0]
         t->perm_in = perm == t->vals[1].as<uint32_t>() ? 1 : 0;
         t->codes_in = 0;

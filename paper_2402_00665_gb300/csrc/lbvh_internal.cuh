@@ -44,7 +44,8 @@ struct Control {
     uint32_t run_sort_count;       //   elements of the fallback sort,
     uint32_t run_heads;            //   runs listed for short_runs_kernel (in this order)
     uint32_t sparse_filled;        // packets left to Algorithm 1
-    uint32_t pad[3];
+    uint32_t scan_ticket;          // tiles of the counts' scan
+    uint32_t pad[2];
 };
 constexpr int kQueryBufferHits = 64;  // hits kept per query by the walk
 
@@ -249,6 +250,16 @@ void launch_encode_rays(const float *rays, int64_t n, const float *bounds, uint6
 void launch_sorted_codes(const float *prims, const uint32_t *perm, int64_t n, int kind, int bits,
                          const float *bounds, uint64_t *codes, cudaStream_t s);
 
+// ---- small trees (small.cu): bounds, codes and sort in one launch. perm: the
+// permutation; kFlagNonfinite is latched as by launch_bounds. 1 <= n <=
+// small_sort_max(bits): whole builds, in one launch / as for large trees (us):
+// 30 bits, 1,024 points 41 / 87, 4,096 57 / 90, 8,192 72 / 91, 12,000 100 / 94;
+// 63 bits, 1,024 45 / 180, 8,192 100 / 189, 16,384 166 / 192.
+constexpr int64_t kSmallSort = 16384;
+inline int64_t small_sort_max(int bits) { return bits > 30 ? kSmallSort : kSmallSort / 2; }
+void launch_small_sort(const float *prims, int64_t n, int kind, int bits, float *bounds, uint32_t *perm, Control *ctl,
+                       cudaStream_t s);
+
 // ---------------------------------------------------------------- construct
 // Algorithm 4 with boxes: writes inodes and leaves (layout above), and uses
 // `store` (n-1 words, all zero on entry; left all zero on exit).
@@ -372,7 +383,8 @@ void launch_knn_packets(const TreeView &t, const float4 *rec, const uint64_t *co
                         const QueryArgs &q, bool own, int k, KnnWalk how, const KnnScratch &sc, uint32_t *out_idx,
                         float *out_d2, Control *ctl, cudaStream_t s);
 // offsets[0..nq] = exclusive scan of counts (offsets[nq] = total =
-// ctl->total).
+// ctl->total). tile_sums: scan_tile_count(nq) words of scratch;
+// ctl->scan_ticket zero beforehand.
 int64_t scan_tile_count(int64_t nq);
 // offsets[0..n) += base (a chunk's CSR offsets moved to its place in the whole)
 void launch_offsets_add(int64_t *offsets, int64_t n, int64_t base, cudaStream_t s);

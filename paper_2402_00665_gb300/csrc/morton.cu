@@ -17,27 +17,6 @@ namespace {
 
 constexpr int kThreads = 256;
 
-struct MinMax {
-    float lo[3], hi[3];
-    bool ok;
-    __device__ void init() {
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = FLT_MAX;
-            hi[a] = -FLT_MAX;
-        }
-        ok = true;
-    }
-    __device__ __forceinline__ void add(float x, float y, float z) {
-        ok = ok && finite3(x, y, z);
-        lo[0] = min_ordered(lo[0], x);
-        lo[1] = min_ordered(lo[1], y);
-        lo[2] = min_ordered(lo[2], z);
-        hi[0] = max_ordered(hi[0], x);
-        hi[1] = max_ordered(hi[1], y);
-        hi[2] = max_ordered(hi[2], z);
-    }
-};
-
 // Visits the centroid of every primitive: f(i, x, y, z). Points go through
 // float4 loads when `prims` is 16-byte aligned (4 points per step).
 template <int kKind, typename F>

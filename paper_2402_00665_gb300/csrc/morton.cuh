@@ -16,6 +16,8 @@
 #include <cfloat>
 #include <cstdint>
 
+#include "lbvh_internal.cuh"
+
 namespace lbvh {
 
 // Mask of the bit positions that input bit k occupies after the spreading
@@ -138,5 +140,27 @@ __device__ __forceinline__ void box_centroid(const float *b, float &x, float &y,
     y = __fmul_rn(__fadd_rn(b[1], b[4]), 0.5f);
     z = __fmul_rn(__fadd_rn(b[2], b[5]), 0.5f);
 }
+
+// Extremes of finite centroids (min_ordered / max_ordered: lbvh_internal.cuh).
+struct MinMax {
+    float lo[3], hi[3];
+    bool ok;
+    __device__ void init() {
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = FLT_MAX;
+            hi[a] = -FLT_MAX;
+        }
+        ok = true;
+    }
+    __device__ __forceinline__ void add(float x, float y, float z) {
+        ok = ok && finite3(x, y, z);
+        lo[0] = min_ordered(lo[0], x);
+        lo[1] = min_ordered(lo[1], y);
+        lo[2] = min_ordered(lo[2], z);
+        hi[0] = max_ordered(hi[0], x);
+        hi[1] = max_ordered(hi[1], y);
+        hi[2] = max_ordered(hi[2], z);
+    }
+};
 
 }  // namespace lbvh

@@ -220,3 +220,55 @@ def test_ray_order(nq):
         assert np.array_equal(off[a:a + len(o)] - off[a], o)
         assert np.array_equal(hits[off[a]:off[a + len(o) - 1]], h)
     t.close()
+
+
+@pytest.mark.parametrize("bits", [3, 30, 33, 63])
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 1023, 1024, 1025, 4096, 4097, 8191, 8192, 8193, 16384, 16385])
+def test_small_builds(n, bits):
+    """Bounds, codes and sort of a small tree in one launch: the tree of the general sort (a chosen sort variant)."""
+    lbvh = L()
+    pts = inputs.uniform_points(n, seed=n)
+    pts[: n // 3] = pts[0]  # equal codes
+    if n > 40:
+        pts[n // 2:, 2] = 0.5
+        pts[7, 0] = -0.0
+    for prims, kind in ((pts, lbvh.POINTS), (boxes_at(pts, 0.01), lbvh.BOXES)):
+        got, want = lbvh.Tree(), lbvh.Tree()
+        want.set_tuning(0, -1)
+        got.build(prims, kind, bits).check()
+        want.build(prims, kind, bits).check()
+        a, b = got.export(), want.export()
+        for key in ("perm", "sorted", "left", "skip_internal", "skip_leaf"):
+            assert np.array_equal(a[key], b[key]), key
+        for key in ("internal_box", "leaf_box", "bounds"):
+            assert np.array_equal(a[key].view(np.uint32), b[key].view(np.uint32)), key
+        got.close()
+        want.close()
+
+
+def test_small_build_refuses_non_finite_points_and_recovers():
+    lbvh = L()
+    pts = inputs.uniform_points(3000, seed=1)
+    bad = pts.copy()
+    bad[2999, 1] = np.inf
+    t = lbvh.Tree().build(bad, lbvh.POINTS, 63)
+    assert t.status() == lbvh.ERR_NONFINITE
+    t.build(pts, lbvh.POINTS, 63).check()
+    t.close()
+
+
+@pytest.mark.parametrize("nq", [1, 4096, 4097, 300_001, 1_245_184, 1_245_185])
+def test_scan_of_counts(nq):
+    """One tile, several by look-back, and the three-pass scan: offsets against the counts' cumulative sum."""
+    lbvh = L()
+    pts = inputs.uniform_points(300, seed=1)
+    t = lbvh.Tree().build(pts, lbvh.POINTS, 30)
+    q = torch.rand((nq, 3), device="cuda")
+    off, hits = t.query(q, lbvh.SPHERE, radius=0.1)
+    p = torch.from_numpy(pts).cuda()
+    counts = torch.cat([((a[:, None] - p[None]).double().square().sum(2) <= 0.01).sum(1) for a in q.split(20_000)])
+    want = torch.cat([torch.zeros(1, dtype=torch.int64, device="cuda"), counts.cumsum(0)])
+    assert int(off[-1]) == hits.numel()
+    assert (off.diff() - counts).abs().sum() <= max(1, nq // 10_000)  # FP64 at the ball's edge
+    assert abs(int(off[-1]) - int(want[-1])) <= max(1, nq // 10_000)
+    t.close()
