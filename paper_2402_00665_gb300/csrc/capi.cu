@@ -530,7 +530,7 @@ struct lbvh_batch_s {
     int passes = 0, qpasses = 0, sort_variant = -1;
     bool self_query = false, sorted_in_b = false;
     DevBuf prim_off, query_off, node_start, store_start, pack_start, chunks, chunk_first, qchunks;
-    DevBuf keys[2], vals[2], nodes, store, lookback, hist, partials, bounds, ctl;
+    DevBuf keys[2], vals[2], nodes, store, pend, lookback, hist, partials, bounds, ctl;
     DevBuf counts, slots, overflow, tile_sums, qkeys[2], qvals[2], qlookback, spill_head, spill, sparse, packed;
     // Segmented-sort tile tables: row r (r < sort_variant_count(): that
     // variant; the last row: the default variant) holds count + 1 entries.
@@ -668,6 +668,7 @@ lbvh_status batch_setup(lbvh_batch_t b, cudaStream_t s) {
     LBVH_CUDA(b->packed.ensure((size_t)records * 32 + 32, s));
     LBVH_CUDA(b->sparse.ensure(((size_t)b->NQ / 32 + 1) * sizeof(uint2), s));
     LBVH_CUDA(b->store.ensure((size_t)words * 8 + 8, s, true));
+    LBVH_CUDA(b->pend.ensure(construct_pend_bytes(b->N), s, true));
     LBVH_CUDA(b->lookback.ensure((size_t)b->max_tiles * kRadix * 8 + 8, s));
     LBVH_CUDA(b->qlookback.ensure((size_t)b->max_qtiles * kRadix * 8 + 8, s));
     LBVH_CUDA(b->hist.ensure((size_t)kMaxPasses * b->count * kRadix * 4 + 4, s));
@@ -707,7 +708,7 @@ lbvh_status batch_enqueue(lbvh_batch_t b, cudaStream_t s) {
                                       b->keys[1].as<uint64_t>(), b->vals[1].as<uint32_t>(), b->N, b->passes,
                                       scratch, c, s, nullptr, b->sort_variant, &seg);
         launch_batch_construct(b->sorted_codes(), b->perm(), g.prims, bt, g.kind, b->nodes.as<float4>(),
-                               b->store.as<unsigned long long>(), &c->build_flags, s);
+                               b->store.as<unsigned long long>(), &c->build_flags, b->pend.p, s);
         LBVH_LAUNCHED();
     }
     if (b->NQ == 0) {
@@ -1532,7 +1533,8 @@ void lbvh_batch_destroy(lbvh_batch_t b) {
                       &b->qchunks, &b->keys[0], &b->keys[1], &b->vals[0], &b->vals[1], &b->nodes, &b->store,
                       &b->lookback, &b->hist, &b->partials, &b->bounds, &b->ctl, &b->counts, &b->slots,
                       &b->overflow, &b->tile_sums, &b->qkeys[0], &b->qkeys[1], &b->qvals[0], &b->qvals[1],
-                      &b->qlookback, &b->tile_first, &b->qtile_first, &b->spill_head, &b->spill, &b->sparse, &b->packed, &b->pack_start})
+                      &b->qlookback, &b->tile_first, &b->qtile_first, &b->spill_head, &b->spill, &b->sparse, &b->packed, &b->pack_start,
+                      &b->pend})
         d->release(s);
     if (s) cudaStreamSynchronize(s);
     pinned_controls().put(b->h_ctl);

@@ -33,13 +33,13 @@
 //   - release/acquire: the exchange is an acq_rel atomic, so a thread's node
 //     is visible before its half of the parent is, and the second thread
 //     reads the sibling's box only after it has seen that half.
-//   - two phases (construct_block_kernel): splits whose two children both
-//     lie inside one group of consecutive leaves (256) meet in
-//     shared memory (block-scope exchange, sibling box from shared memory);
-//     only the nodes spanning a group's edge meet in the device-scope
-//     `store` words (sibling box through L2, ld.global.cg). Batches group
-//     their global sorted positions the same way (a group may hold several
-//     trees; a split only ever joins leaves of one).
+//   - inside a group of 256 consecutive leaves nobody climbs: the nodes whose
+//     range lies in the group are formed from the delta* values side by side
+//     (merge_elements, one warp to 32 leaves, then 32 of what is left); only
+//     the nodes spanning a group's edge meet in the `store` words (sibling
+//     box through L2, ld.global.cg). Batches group their global sorted
+//     positions the same way (a group may hold several trees; a split only
+//     ever joins leaves of one).
 #include <atomic>
 
 #include <cuda/atomic>
@@ -133,22 +133,6 @@ struct Climb {
     float3 lo, hi;
 };
 
-// delta*(i-1), delta*(i), delta*(i+1) around leaf i (255 = +inf at -1 and n-1).
-// Codes out of order (c0 > c1) latch kFlagCorrupt: the input is not sorted.
-__device__ __forceinline__ void leaf_deltas(int i, int n, const uint64_t *__restrict__ codes, uint32_t &dl,
-                                            uint32_t &dr, uint32_t &drn, uint32_t *flags) {
-    const uint64_t c0 = codes[i];
-    dl = i > 0 ? delta_star(codes[i - 1], c0, (uint32_t)(i - 1)) : kInf;
-    dr = kInf;
-    drn = kInf;
-    if (i + 1 < n) {
-        const uint64_t c1 = codes[i + 1];
-        if (c0 > c1) atomicOr(flags, kFlagCorrupt);
-        dr = delta_star(c0, c1, (uint32_t)i);
-        if (i + 2 < n) drn = delta_star(c1, codes[i + 2], (uint32_t)(i + 1));
-    }
-}
-
 // The primitive's box (a point's box is the point).
 template <int kKind>
 __device__ __forceinline__ void gather_box(const float *__restrict__ prims, uint32_t p_id, float3 &lo, float3 &hi) {
@@ -162,45 +146,19 @@ __device__ __forceinline__ void gather_box(const float *__restrict__ prims, uint
     }
 }
 
-// Algorithm 4's leaf step for leaf i of one tree of n leaves, given its
-// delta* values and its primitive (own index p_own, box lo/hi): the leaf's
-// skip and box are written out and the climb state is set.
+// Algorithm 4's leaf lines: leaf i of a tree of n leaves, own index p_own,
+// box lo/hi, with delta*(i) and delta*(i+1).
 template <int kKind>
 __device__ __forceinline__ void leaf_write(int i, int n, uint32_t p_own, float3 lo, float3 hi, float4 *leaves,
-                                           uint32_t dl, uint32_t dr, uint32_t drn, Climb &c) {
-    const int ni = n - 1;
-    const int leaf_skip = i == n - 1 ? kSentinel : (dr < drn ? ni + i + 1 : i + 1);
+                                           uint32_t dr, uint32_t drn) {
     // the leaf's skip is position i+1: one bit says I_{i+1} rather than L_{i+1}
-    const uint32_t word = p_own | (leaf_skip >= 0 && leaf_skip < ni ? kLeafSkipInternal : 0u);
+    const uint32_t word = p_own | (i + 1 < n && dr >= drn ? kLeafSkipInternal : 0u);
     if (kKind == LBVH_PRIM_POINTS) {
         leaves[i] = make_float4(lo.x, lo.y, lo.z, __uint_as_float(word));
     } else {
         leaves[2 * (int64_t)i] = make_float4(lo.x, lo.y, lo.z, __uint_as_float(word));
         leaves[2 * (int64_t)i + 1] = make_float4(hi.x, hi.y, hi.z, 0.0f);
     }
-    c = Climb{(uint32_t)i, (uint32_t)i, dl, dr, drn, lo, hi};
-}
-
-// The leaf step from sorted codes and a permutation. perm holds primitive
-// indices into `prims`, the tree's own indices being perm - perm_base. False
-// (and kFlagCorrupt) if perm is not a permutation of this tree.
-template <int kKind>
-__device__ __forceinline__ bool leaf_step(int i, int n, const uint64_t *__restrict__ codes,
-                                          const uint32_t *__restrict__ perm, uint32_t perm_base,
-                                          const float *__restrict__ prims, float4 *leaves, uint32_t *flags,
-                                          Climb &c) {
-    uint32_t dl, dr, drn;
-    leaf_deltas(i, n, codes, dl, dr, drn, flags);
-    const uint32_t p_id = perm[i];
-    const uint32_t p_own = p_id - perm_base;
-    if (p_own >= (uint32_t)n) {  // not a permutation of this tree: the sort failed
-        atomicOr(flags, kFlagCorrupt);
-        return false;
-    }
-    float3 lo, hi;
-    gather_box<kKind>(prims, p_id, lo, hi);
-    leaf_write<kKind>(i, n, p_own, lo, hi, leaves, dl, dr, drn, c);
-    return true;
 }
 
 // The parent's split p of c's node (range_right for a left child, range_left
@@ -278,167 +236,390 @@ __device__ __forceinline__ void climb_global(Climb c, int n, float4 *inodes, con
     atomicOr(flags, kFlagCorrupt);
 }
 
-// Algorithm 4 with the climb split in two phases. The leaves are cut into
-// groups of kGroup consecutive leaves [a, a + kGroup), one per CTA. A node
-// whose leaf range lies inside a group has both children there, so its split
-// p has a <= p and p + 1 < a + kGroup; such splits meet in a shared-memory
-// word with a block-scope exchange, and the sibling's box is read from shared
-// memory. A thread stops phase 1 at a split on the group's edge, or as the
-// first up at a word. After the group's barrier every node inside the group
-// is finished; a word still holding its first thread's half has a sibling
-// that spans the group's edge, and that thread, like one stopped at the edge,
-// continues with the device-scope exchanges of climb_global. Each node is
-// still written once, by the second thread up at its split, with the same
-// fields: only where the two halves meet changes. Group size, with the
-// climbs that leave a group handed to a second kernel (construct time at 2^25
-// points, 63-bit codes): 64 leaves 1.83 ms (8 hand-off slots 1.67), 128
-// 1.64, 256 1.56 (16 slots; 12: 1.57; 8: 1.55; 32: 1.67), 512 1.57.
-constexpr int kGroup = 256;
+// Nodes inside a group of kGroup consecutive leaves, one group per CTA. A
+// node of split p covers [l, r]: l - 1 and r are the nearest positions on
+// either side whose delta* exceeds delta*(p). So a warp that holds 32
+// consecutive elements (at first the leaves) has all it needs to write the
+// nodes that both ends of which it can see, all at once: which lanes hold a
+// larger gap comes from eight ballots, one to a bit of delta*, and the box of
+// a range of lanes is the union of two entries of a table over runs of 2, 4,
+// 8 and 16 lanes (min and max may count a lane twice). Splits whose range
+// leaves the warp stay open; what lies between two open splits is one
+// finished node (or leaf), an element of the next round. 128 leaves of
+// uniform points leave 22 elements, then 7. What is left goes to the merges
+// above the groups, or climbs with the device-scope exchanges of
+// climb_global. The same nodes are written as by a climb from
+// every leaf, each once.
+//
+// This is bound by instructions issued, not by memory. With a thread per
+// leaf climbing through shared-memory words (block-scope exchanges, half the
+// lanes gone after each level) this pass took 1226 instructions per warp of
+// leaves and 1.57 ms at 2^25 points, 63-bit codes; now 757 and 1.13 (16,384
+// points 32.7 -> 19.0 us, 1.0M 81.9 -> 65.5, 2^23 428 -> 309). Groups of 128 leaves, 12 CTAs to
+// an SM, against 256 with 6: 1.29 and 1.36 ms before the merges above them;
+// 512: 1.48; 10 CTAs: 1.39. More CTAs take the L1's room for shared memory
+// and the gathers miss: 14 CTAs 1.87.
+constexpr int kGroup = 128;
+constexpr int kWarps = kGroup / 32;
+static_assert(kWarps == 4, "GroupSmem::count is one word");
+constexpr int kRounds = 3;
+constexpr int kGroupCtas = 12;  // CTAs of an SM
+constexpr int kRuns = 4;  // runs of 2 .. 2^kRuns lanes in a warp's table
 
-struct GroupSmem {
-    unsigned long long word[kGroup];    // split at global position a + j: word[j]
-    float3 lo[2][kGroup], hi[2][kGroup];  // boxes: [0] leaf, [1] internal node, by global position / index
-    uint64_t code[kGroup + 3];          // sorted codes a-1 .. a+kGroup+1 (construct_encode_kernel)
-    int failed;
-    int pending;                        // climbs handed to climb_pending_kernel
+struct RunTable {
+    float4 a[kRuns][32];  // lo.xyz, hi.x of the run that starts at a lane
+    float2 b[kRuns][32];  // hi.yz
 };
 
-// Climbs that leave a group: the CTA hands up to kPendSlots of them to
-// climb_pending_kernel through its own slots (16 bytes each: l, r, the three
-// delta* values and a valid bit), so that no CTA waits on device-scope
-// exchanges with most of its threads done. On uniform points a group of 128
-// leaves has 7.3 such climbs on average and 13 at most (one more level of
-// the tree per doubling of the group); more than kPendSlots climb in place.
-constexpr int kPendSlots = 12;
-constexpr uint32_t kPendValid = 1u << 31;
+struct ElementList {
+    uint32_t l[kGroup], r[kGroup], gaps[kGroup];
+    float box[6][kGroup];
+    int tree[kGroup];  // batches
+};
 
-// Both phases for thread t, holding leaf i's climb state c (go: the leaf was
-// written and the tree has internal nodes), of a tree of n leaves whose leaf
-// 0 sits at global position o (0 for a single tree; trees of a batch follow
-// each other), in the group whose first global position is a. A split joins
-// two leaves of one tree, so groups may hold several trees. Every thread of
-// the CTA must call this (it holds the group's barrier).
-// pend (nullable): the CTA's kPendSlots slots.
-template <int kKind, bool kJitter = false>
-__device__ __forceinline__ void two_phase(GroupSmem &sm, bool go, Climb c, int n, int64_t o, int64_t a, int t,
-                                          float4 *inodes, const float4 *leaves, unsigned long long *store,
-                                          uint32_t *flags, uint4 *pend, const Jitter &jt = Jitter{}) {
-    const int ni = n - 1;
-    bool pending = false, in_word = false;
-    int word_at = 0;
-    if (go) {
-        sm.lo[0][t] = c.lo;
-        sm.hi[0][t] = c.hi;
-        for (int level = 0; level < 128; ++level) {
-            uint32_t p;
-            unsigned long long mine;
-            const bool is_left = parent_split(c, p, mine);
-            if (p >= (uint32_t)ni) {
-                atomicOr(flags, kFlagCorrupt);
-                break;
-            }
-            const int64_t rel = o + (int64_t)p - a;  // the split's place in the group
-            if (rel < 0 || rel >= kGroup - 1) {       // on the group's edge
-                pending = true;
-                break;
-            }
-            const int at = (int)rel;
-            jitter_wait<kJitter>(jt, (unsigned long long)p << 8 | (unsigned)level);
-            cuda::atomic_ref<unsigned long long, cuda::thread_scope_block> w(sm.word[at]);
-            const unsigned long long other = w.exchange(mine, cuda::memory_order_acq_rel);
-            if (other == 0ull) {  // first up: the sibling may come in this phase, or never
-                pending = in_word = true;
-                word_at = at;
-                break;
-            }
-            w.store(0ull, cuda::memory_order_relaxed);  // taken
-            if ((uint32_t)other >= (uint32_t)n) {
-                atomicOr(flags, kFlagCorrupt);
-                break;
-            }
-            const int sibling = take_half(c, is_left, p, other, ni);
-            const int k = sibling < ni ? 1 : 0;
-            const int sat = (int)(o + (sibling < ni ? sibling : sibling - ni) - a);  // at or at + 1
-            const int q = write_parent(c, p, n, sm.lo[k][sat], sm.hi[k][sat], inodes);
-            if (q == 0) break;  // the root: the whole tree lies in this group
-            const int qat = (int)(o + q - a);  // q is l or r, inside the group
-            sm.lo[1][qat] = c.lo;
-            sm.hi[1][qat] = c.hi;
-        }
-    }
-    __syncthreads();
-    if (!pending) return;
-    if (in_word && sm.word[word_at] == 0ull) return;  // the sibling came and carried on
-    if (pend) {
-        const int slot = atomicAdd(&sm.pending, 1);
-        if (slot < kPendSlots) {
-            pend[slot] = make_uint4(c.l, c.r, kPendValid | c.d_left | c.d_right << 8 | c.d_next << 16, 0u);
-            return;
-        }
-    }
-    // this thread wrote its own node, so its device-scope release covers it
-    climb_global<kKind, kJitter>(c, n, inodes, leaves, store, flags, jt);
+struct GroupSmem {
+    union {
+        uint64_t code[kGroup + 3];  // sorted codes a-1 .. a+kGroup+1
+        RunTable table[kWarps];
+        ElementList list;
+    };
+    uint8_t gap[kGroup + 4];  // delta* at a-1 .. a+kGroup (kInf between two trees)
+    alignas(4) uint8_t count[4];  // elements a warp leaves
+    int instance[2];              // batches: of the first and the last leaf
+    int failed;
+};
+
+// Elements left by a group: the CTA hands them, in order, to
+// merge_pending_kernel through its own kPendSlots slots (16 bytes each: l, r,
+// the three delta* values with a valid bit, the tree). On uniform points a
+// group of 128 leaves has 7.3 of them on average, 1024 leaves 10.3, 7680
+// 13.2; more than 16, 20 and 25 have none of 23,000 groups, none of 2,900 and
+// one of 2,000 (a mixture of tight clusters: one of 1000, 20 and 200). A list
+// longer than its slots climbs in place and marks its first slot
+// kPendClimbed, and then the merge above climbs too.
+constexpr int kPendSlots = 16;
+constexpr int kMergedSlots = 25;  // of a CTA of merge_pending_kernel
+constexpr uint32_t kPendValid = 1u << 31;
+constexpr uint32_t kPendClimbed = 1u << 30;
+
+struct Owner {  // a tree's leaves and memory
+    int n;
+    float4 *inodes;
+    float4 *leaves;
+    unsigned long long *store;
+};
+
+// A finished node or leaf: its leaves [l, r] in its tree, delta*(l-1) |
+// delta*(r) << 8 | delta*(r+1) << 16, its box.
+struct Element {
+    uint32_t l, r, gaps;
+    float3 lo, hi;
+    int tree;
+};
+
+__device__ __forceinline__ float3 min3f(float3 a, float3 b) {
+    return make_float3(min_ordered(a.x, b.x), min_ordered(a.y, b.y), min_ordered(a.z, b.z));
+}
+__device__ __forceinline__ float3 max3f(float3 a, float3 b) {
+    return make_float3(max_ordered(a.x, b.x), max_ordered(a.y, b.y), max_ordered(a.z, b.z));
+}
+__device__ __forceinline__ float3 shfl_down3(float3 v, int by) {
+    return make_float3(__shfl_down_sync(~0u, v.x, by), __shfl_down_sync(~0u, v.y, by), __shfl_down_sync(~0u, v.z, by));
 }
 
-// The climbs handed over by the groups, one thread per slot: the climber's
-// node (range [l, r], written by the first kernel) is read back for its box
-// and the climb goes on with device-scope exchanges. Every valid slot is
-// cleared, so the slots are zero again for the next build.
-template <int kKind, bool kJitter>
-__global__ void __launch_bounds__(256)
-    climb_pending_kernel(uint4 *pend, int64_t slots, int n, float4 *inodes, const float4 *leaves,
-                         unsigned long long *store, uint32_t *flags, Jitter jt) {
-    const int64_t k = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (k >= slots) return;
-    const uint4 e = pend[k];
-    if (!(e.z & kPendValid)) return;
-    pend[k] = make_uint4(0u, 0u, 0u, 0u);
-    if (__ldcg(flags) & (kFlagTimeout | kFlagCorrupt)) return;
-    const int ni = n - 1;
-    Climb c;
-    c.l = e.x;
-    c.r = e.y;
-    c.d_left = e.z & 0xffu;
-    c.d_right = (e.z >> 8) & 0xffu;
-    c.d_next = (e.z >> 16) & 0xffu;
-    if (c.l > c.r || c.r >= (uint32_t)n) {
-        atomicOr(flags, kFlagCorrupt);
+// One warp over its first m lanes' elements (consecutive, m >= 1; all lanes
+// call). Writes the nodes that are complete here; true where the lane's own
+// split stays open: e is then the finished node or leaf that ends there.
+// kPoint: e.lo == e.hi. owner(tree): the Owner.
+template <bool kPoint, typename OwnerOf>
+__device__ __forceinline__ bool merge_elements(RunTable &table, int m, Element &e, const OwnerOf &owner) {
+    const int lane = threadIdx.x & 31;
+    const bool have = lane < m;
+    const uint32_t d = have ? (e.gaps >> 8) & 0xffu : 0u;
+    // lanes with a larger gap, from the highest bit of delta* down
+    uint32_t above = 0u, same = ~0u;
+#pragma unroll
+    for (int bit = 7; bit >= 0; --bit) {
+        const uint32_t set = __ballot_sync(~0u, (d >> bit) & 1u);
+        const uint32_t mine = (uint32_t)((int)(d << (31 - bit)) >> 31);  // all ones if the lane's bit is set
+        above |= same & set & ~mine;
+        same &= ~(set ^ mine);
+    }
+    const uint32_t before = (1u << lane) - 1u;
+    const uint32_t lower = above & before, upper = above & ~before;
+    const uint32_t outer = __shfl_sync(~0u, e.gaps, 0) & 0xffu;
+    const bool complete = have && upper != 0u && (lower != 0u || outer > d);
+    const uint32_t open = __ballot_sync(~0u, have && !complete);
+    const uint32_t stops = complete ? lower : open & before;
+    const int first = 32 - __clz((int)stops);
+    const int last = complete ? __ffs((int)upper) - 1 : lane;
+    const uint32_t p = e.r;
+    const uint32_t l = __shfl_sync(~0u, e.l, first), r = __shfl_sync(~0u, e.r, last);
+    const uint32_t left_gap = __shfl_sync(~0u, e.gaps, first) & 0xffu;
+    const uint32_t right_gaps = __shfl_sync(~0u, e.gaps, last) & ~0xffu;
+    // boxes of runs of 2, 4, 8, 16 lanes
+    float3 lo = e.lo, hi = e.hi;
+#pragma unroll
+    for (int k = 0; k < kRuns; ++k) {
+        const float3 nlo = shfl_down3(lo, 1 << k), nhi = k == 0 && kPoint ? nlo : shfl_down3(hi, 1 << k);
+        lo = min3f(lo, nlo);
+        hi = max3f(hi, nhi);
+        table.a[k][lane] = make_float4(lo.x, lo.y, lo.z, hi.x);
+        table.b[k][lane] = make_float2(hi.y, hi.z);
+    }
+    __syncwarp();
+    const int len = last - first + 1;
+    if (have && len > 1) {
+        const int k = min(31 - __clz(len), kRuns) - 1;
+        const int second = last + 1 - (2 << k);
+        const float4 a0 = table.a[k][first], a1 = table.a[k][second];
+        const float2 b0 = table.b[k][first], b1 = table.b[k][second];
+        e.lo = min3f(make_float3(a0.x, a0.y, a0.z), make_float3(a1.x, a1.y, a1.z));
+        e.hi = max3f(make_float3(a0.w, b0.x, b0.y), make_float3(a1.w, b1.x, b1.y));
+    }
+    e.l = l;
+    e.r = r;
+    e.gaps = left_gap | right_gaps;
+    if (complete) {
+        const Owner o = owner(e.tree);
+        const int ni = o.n - 1;
+        const uint32_t dr = (right_gaps >> 8) & 0xffu;
+        const int q = (int)(dr < left_gap ? r : l);
+        const int left_child = (int)(l == p ? ni + p : p);
+        const int skip = dr == kInf ? kSentinel : (int)(dr < right_gaps >> 16 ? ni + r + 1 : r + 1);
+        o.inodes[2 * (int64_t)q] = make_float4(e.lo.x, e.lo.y, e.lo.z, __int_as_float(left_child));
+        o.inodes[2 * (int64_t)q + 1] = make_float4(e.hi.x, e.hi.y, e.hi.z, __int_as_float(skip));
+    }
+    return have && !complete;
+}
+
+// A CTA's elements, consecutive, one per thread (the first `count`): merges
+// them in rounds; what is left goes to the CTA's slots (pend), or climbs.
+// Every thread of the CTA calls this; the tables' memory is free.
+template <int kKind, bool kPoints, bool kJitter, bool kTrees, typename OwnerOf>
+__device__ __forceinline__ void merge_group(GroupSmem &sm, int count, Element e, const OwnerOf &owner,
+                                            uint32_t *flags, uint4 *pend, int slots, const Jitter &jt) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    bool keep = false;
+    uint32_t kept = 0u;
+    for (int round = 0;; ++round) {
+        const int m = min(count - 32 * warp, 32);
+        keep = false;
+        if (m > 0) {
+            keep = kPoints && round == 0 ? merge_elements<true>(sm.table[warp], m, e, owner)
+                                         : merge_elements<false>(sm.table[warp], m, e, owner);
+            // a whole tree is done (its root is written, or it is one leaf)
+            keep = keep && (e.gaps & 0xffffu) != (kInf | kInf << 8);
+        }
+        kept = __ballot_sync(~0u, keep);
+        if (count <= 32 || round == kRounds - 1) break;
+        if (lane == 0) sm.count[warp] = (uint8_t)__popc(kept);
+        __syncthreads();  // also: every warp is through with its table
+        const uint32_t counts = *reinterpret_cast<const uint32_t *>(sm.count);  // a byte per warp
+        const int at = __popc(kept & ((1u << lane) - 1u)) +
+                       (int)__dp4a(counts & ((1u << (8 * warp)) - 1u), 0x01010101u, 0u);
+        count = (int)__dp4a(counts, 0x01010101u, 0u);
+        if (keep) {
+            sm.list.l[at] = e.l;
+            sm.list.r[at] = e.r;
+            sm.list.gaps[at] = e.gaps;
+            sm.list.box[0][at] = e.lo.x;
+            sm.list.box[1][at] = e.lo.y;
+            sm.list.box[2][at] = e.lo.z;
+            sm.list.box[3][at] = e.hi.x;
+            sm.list.box[4][at] = e.hi.y;
+            sm.list.box[5][at] = e.hi.z;
+            if (kTrees) sm.list.tree[at] = e.tree;
+        }
+        __syncthreads();
+        if ((int)threadIdx.x < count) {
+            const int k = threadIdx.x;
+            e.l = sm.list.l[k];
+            e.r = sm.list.r[k];
+            e.gaps = sm.list.gaps[k];
+            e.lo = make_float3(sm.list.box[0][k], sm.list.box[1][k], sm.list.box[2][k]);
+            e.hi = make_float3(sm.list.box[3][k], sm.list.box[4][k], sm.list.box[5][k]);
+            if (kTrees) e.tree = sm.list.tree[k];
+        }
+        __syncthreads();  // the tables take the list's place
+    }
+    const bool one_warp = count <= 32;  // what is left, and the last round's nodes: the first warp's
+    if (pend && one_warp && __popc(kept) <= slots) {
+        if (keep) pend[__popc(kept & ((1u << lane) - 1u))] = make_uint4(e.l, e.r, kPendValid | e.gaps, (uint32_t)e.tree);
         return;
     }
-    // the node of range [l, r]: leaf l, or internal node r or l (its Karras index)
-    const int id = c.l == c.r ? ni + (int)c.l : (c.d_right < c.d_left ? (int)c.r : (int)c.l);
-    load_node_box<kKind>(inodes, leaves, ni, id, c.lo, c.hi);
-    climb_global<kKind, kJitter>(c, n, inodes, leaves, store, flags, jt);
+    if (pend && threadIdx.x == 0) pend[0] = make_uint4(0u, 0u, kPendClimbed, 0u);
+    // The nodes of this CTA, whichever thread wrote them, are visible to
+    // whoever sees this thread's exchange: the barrier orders them before its
+    // release.
+    if (one_warp) __syncwarp();
+    else __syncthreads();
+    if (!keep) return;
+    const Owner o = owner(e.tree);
+    climb_global<kKind, kJitter>(Climb{e.l, e.r, e.gaps & 0xffu, (e.gaps >> 8) & 0xffu, (e.gaps >> 16) & 0xffu, e.lo, e.hi},
+                                 o.n, o.inodes, o.leaves, o.store, flags, jt);
 }
 
-// Clears the CTA's shared words and reads the build's error flags: true if
-// an earlier stage failed, in which case the whole CTA returns and leaves
-// `store` untouched.
-__device__ __forceinline__ bool group_start(GroupSmem &sm, const uint32_t *flags) {
-    sm.word[threadIdx.x] = 0ull;
-    if (threadIdx.x == 0) {
-        sm.failed = (__ldcg(flags) & (kFlagTimeout | kFlagCorrupt)) != 0;
-        sm.pending = 0;
+// The build's error flags, read once per CTA (they go to sm.failed before the
+// CTA's first barrier): if an earlier stage failed, the whole CTA returns and
+// leaves `store` untouched.
+__device__ __forceinline__ void group_start(GroupSmem &sm, const uint32_t *flags) {
+    if (threadIdx.x == 0) sm.failed = (__ldcg(flags) & (kFlagTimeout | kFlagCorrupt)) != 0;
+}
+
+struct OneTree {
+    Owner o;
+    __device__ __forceinline__ Owner operator()(int) const { return o; }
+};
+
+// The trees of a batch: global sorted position g belongs to the instance b
+// with off[b] <= g < off[b+1]; its tree's records start at node_start[b]
+// (float4 units) and its store words at store_start[b].
+struct ManyTrees {
+    const int64_t *off, *node_start, *store_start;
+    float4 *nodes;
+    unsigned long long *store;
+    __device__ __forceinline__ Owner operator()(int b) const {
+        const int n = (int)(__ldg(off + b + 1) - __ldg(off + b));
+        float4 *inodes = nodes + __ldg(node_start + b);
+        return Owner{n, inodes, inodes + 2 * (int64_t)(n - 1), store + __ldg(store_start + b)};
+    }
+};
+
+// What the groups left, kGroup slots to a CTA, is merged the same way, their
+// nodes read back for their boxes; what is left of that (10 elements to
+// 1024 leaves of uniform points) is merged again or climbs with device-scope exchanges. Every
+// slot is cleared, so the slots are zero again for the next build. With a
+// thread per slot climbing from there the construct of 2^25 points took 1.29
+// ms, so 1.13; 512 batched trees of 36,000 points that climbed inside the
+// groups' kernel 1.13 ms, so 0.65.
+
+template <int kKind, int kSlots, bool kJitter, bool kTrees, typename OwnerOf>
+__global__ void __launch_bounds__(kGroup)
+    merge_pending_kernel(uint4 *pend, int64_t slots, OwnerOf owner, uint32_t *flags, uint4 *out, Jitter jt) {
+    constexpr int kMergeGroups = kGroup / kSlots;
+    __shared__ GroupSmem sm;
+    group_start(sm, flags);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t k = (int64_t)blockIdx.x * (kMergeGroups * kSlots) + threadIdx.x;
+    const bool slot = threadIdx.x < kMergeGroups * kSlots && k < slots;
+    if (out) out += (int64_t)blockIdx.x * kMergedSlots;
+    const uint4 w = slot ? pend[k] : make_uint4(0u, 0u, 0u, 0u);
+    if (w.z) pend[k] = make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t valid = __ballot_sync(~0u, (w.z & kPendValid) != 0u);
+    if (lane == 0) sm.count[warp] = (uint8_t)__popc(valid);
+    Element e{w.x, w.y, w.z & 0xffffffu, make_float3(0.f, 0.f, 0.f), make_float3(0.f, 0.f, 0.f), (int)w.w};
+    bool have = (w.z & kPendValid) != 0u, missing = (w.z & kPendClimbed) != 0u;
+    if (have) {
+        const Owner o = owner(e.tree);
+        if (e.l > e.r || e.r >= (uint32_t)o.n) {
+            atomicOr(flags, kFlagCorrupt);
+            have = false;
+            missing = true;
+        } else {
+            // the node of range [l, r]: leaf l, or internal node r or l (its Karras index)
+            const uint32_t dl = e.gaps & 0xffu, dr = (e.gaps >> 8) & 0xffu;
+            const int id = (int)(e.l == e.r ? (uint32_t)(o.n - 1) + e.l : (dr < dl ? e.r : e.l));
+            load_node_box<kKind>(o.inodes, o.leaves, o.n - 1, id, e.lo, e.hi);
+        }
+    }
+    const bool climbed = __syncthreads_or(missing);
+    if (sm.failed) return;
+    if (climbed) {  // some elements are missing: those that are here climb too
+        if (out && threadIdx.x == 0) out[0] = make_uint4(0u, 0u, kPendClimbed, 0u);
+        if (!have) return;
+        const Owner o = owner(e.tree);
+        climb_global<kKind, kJitter>(
+            Climb{e.l, e.r, e.gaps & 0xffu, (e.gaps >> 8) & 0xffu, (e.gaps >> 16) & 0xffu, e.lo, e.hi}, o.n, o.inodes,
+            o.leaves, o.store, flags, jt);
+        return;
+    }
+    const uint32_t counts = *reinterpret_cast<const uint32_t *>(sm.count);
+    const int at = __popc(valid & ((1u << lane) - 1u)) +
+                   (int)__dp4a(counts & ((1u << (8 * warp)) - 1u), 0x01010101u, 0u);
+    const int count = (int)__dp4a(counts, 0x01010101u, 0u);
+    if (have) {
+        sm.list.l[at] = e.l;
+        sm.list.r[at] = e.r;
+        sm.list.gaps[at] = e.gaps;
+        sm.list.box[0][at] = e.lo.x;
+        sm.list.box[1][at] = e.lo.y;
+        sm.list.box[2][at] = e.lo.z;
+        sm.list.box[3][at] = e.hi.x;
+        sm.list.box[4][at] = e.hi.y;
+        sm.list.box[5][at] = e.hi.z;
+        if (kTrees) sm.list.tree[at] = e.tree;
     }
     __syncthreads();
-    return sm.failed != 0;
+    if ((int)threadIdx.x < count) {
+        const int j = threadIdx.x;
+        e.l = sm.list.l[j];
+        e.r = sm.list.r[j];
+        e.gaps = sm.list.gaps[j];
+        e.lo = make_float3(sm.list.box[0][j], sm.list.box[1][j], sm.list.box[2][j]);
+        e.hi = make_float3(sm.list.box[3][j], sm.list.box[4][j], sm.list.box[5][j]);
+        if (kTrees) e.tree = sm.list.tree[j];
+    }
+    __syncthreads();
+    merge_group<kKind, false, kJitter, kTrees>(sm, count, e, owner, flags, out, kMergedSlots, jt);
+}
+
+// delta* at the CTA's positions, from sm.code. Thread t holds leaf i of a
+// tree of n leaves (i >= n: no leaf). Codes out of order latch kFlagCorrupt:
+// the input is not sorted.
+__device__ __forceinline__ void group_gaps(GroupSmem &sm, int i, int n, uint32_t *flags) {
+    const int t = threadIdx.x;
+    uint32_t dr = kInf;
+    if (i + 1 < n) {
+        const uint64_t c0 = sm.code[t + 1], c1 = sm.code[t + 2];
+        if (c0 > c1) atomicOr(flags, kFlagCorrupt);
+        dr = delta_star(c0, c1, (uint32_t)i);
+    }
+    sm.gap[t + 1] = (uint8_t)dr;
+    if (t == 0) sm.gap[0] = (uint8_t)(i > 0 && i < n ? delta_star(sm.code[0], sm.code[1], (uint32_t)(i - 1)) : kInf);
+    if (t == kGroup - 1)
+        sm.gap[kGroup + 1] =
+            (uint8_t)(i + 2 < n ? delta_star(sm.code[t + 2], sm.code[t + 3], (uint32_t)(i + 1)) : kInf);
+}
+
+// Leaf i's element: its gaps, in place in sm.gap.
+__device__ __forceinline__ uint32_t leaf_gaps(const GroupSmem &sm) {
+    const int t = threadIdx.x;
+    return sm.gap[t] | (uint32_t)sm.gap[t + 1] << 8 | (uint32_t)sm.gap[t + 2] << 16;
 }
 
 // Algorithm 4 from sorted codes and a permutation (lbvh_build_from_sorted,
 // refit, the no-allocation entry point).
 template <int kKind, bool kJitter>
-__global__ void __launch_bounds__(kGroup, 2048 / kGroup)
+__global__ void __launch_bounds__(kGroup, kGroupCtas)
     construct_block_kernel(const uint64_t *__restrict__ codes, const uint32_t *__restrict__ perm,
                            const float *__restrict__ prims, int n, float4 *inodes, float4 *leaves,
                            unsigned long long *store, uint32_t *flags, uint4 *pend, Jitter jt) {
     __shared__ GroupSmem sm;
-    if (group_start(sm, flags)) return;
+    group_start(sm, flags);
     const int t = threadIdx.x;
-    const int i = blockIdx.x * kGroup + t;
-    Climb c;
-    const bool ok = i < n && leaf_step<kKind>(i, n, codes, perm, 0u, prims, leaves, flags, c);
-    two_phase<kKind, kJitter>(sm, ok && n > 1, c, n, 0, (int64_t)blockIdx.x * kGroup, t, inodes, leaves, store,
-                              flags, pend ? pend + (int64_t)blockIdx.x * kPendSlots : nullptr, jt);
+    const int64_t a = (int64_t)blockIdx.x * kGroup;
+    const int i = (int)a + t;
+    const bool mine = i < n;
+    const uint32_t p_id = mine ? perm[i] : 0u;
+    const bool ok = mine && p_id < (uint32_t)n;
+    Element e{(uint32_t)i, (uint32_t)i, 0u, make_float3(0.f, 0.f, 0.f), make_float3(0.f, 0.f, 0.f), 0};
+    if (ok) gather_box<kKind>(prims, p_id, e.lo, e.hi);
+    if (mine) sm.code[t + 1] = codes[i];
+    if (t < 3) {
+        const int64_t h = t == 0 ? a - 1 : a + kGroup + t - 1;
+        if (h >= 0 && h < n) sm.code[t == 0 ? 0 : kGroup + t] = codes[h];
+    }
+    __syncthreads();
+    if (sm.failed) return;
+    if (mine && !ok) atomicOr(flags, kFlagCorrupt);  // not a permutation: the sort failed
+    group_gaps(sm, i, n, flags);
+    __syncthreads();
+    e.gaps = leaf_gaps(sm);
+    if (ok) leaf_write<kKind>(i, n, p_id, e.lo, e.hi, leaves, (e.gaps >> 8) & 0xffu, e.gaps >> 16);
+    merge_group<kKind, kKind == LBVH_PRIM_POINTS, kJitter, false>(
+        sm, (int)min((int64_t)kGroup, n - a), e, OneTree{Owner{n, inodes, leaves, store}}, flags,
+        pend ? pend + (int64_t)blockIdx.x * kPendSlots : nullptr, kPendSlots, jt);
 }
 
 // Algorithm 4 after a sort that kept only the permutation. Each thread
@@ -448,32 +629,25 @@ __global__ void __launch_bounds__(kGroup, 2048 / kGroup)
 // 0-2) meet in shared memory for the delta* values. The sorted codes are
 // written to codes_out (the tree keeps them for export and refit).
 template <int kKind, bool kJitter>
-__global__ void __launch_bounds__(kGroup, 2048 / kGroup)
+__global__ void __launch_bounds__(kGroup, kGroupCtas)
     construct_encode_kernel(const uint32_t *__restrict__ perm, const float *__restrict__ prims,
                             const float *__restrict__ bounds, int b, int n, uint64_t *__restrict__ codes_out,
                             float4 *inodes, float4 *leaves, unsigned long long *store, uint32_t *flags,
                             uint4 *pend, Jitter jt) {
     __shared__ GroupSmem sm;
-    if (group_start(sm, flags)) return;
+    group_start(sm, flags);
     const int t = threadIdx.x;
     const int64_t a = (int64_t)blockIdx.x * kGroup;
     const int i = (int)a + t;
     const Grid3 g = make_grid(bounds, b);
-    bool ok = i < n;
-    uint32_t p_id = 0;
-    float3 lo = make_float3(0.f, 0.f, 0.f), hi = lo;
-    if (ok) {
-        p_id = __ldcs(perm + i);
-        if (p_id >= (uint32_t)n) {  // not a permutation: the sort failed
-            atomicOr(flags, kFlagCorrupt);
-            ok = false;
-        } else {
-            gather_box<kKind>(prims, p_id, lo, hi);
-        }
-    }
+    const bool mine = i < n;
+    const uint32_t p_id = mine ? __ldcs(perm + i) : 0u;
+    const bool ok = mine && p_id < (uint32_t)n;
+    Element e{(uint32_t)i, (uint32_t)i, 0u, make_float3(0.f, 0.f, 0.f), make_float3(0.f, 0.f, 0.f), 0};
+    if (ok) gather_box<kKind>(prims, p_id, e.lo, e.hi);
     // the three neighbours outside the CTA's range
     int64_t hpos = -1;
-    float3 hlo = lo, hhi = hi;
+    float3 hlo = e.lo, hhi = e.hi;
     if (t < 3) {
         hpos = t == 0 ? a - 1 : a + kGroup + t - 1;
         if (hpos >= 0 && hpos < n) {
@@ -484,75 +658,147 @@ __global__ void __launch_bounds__(kGroup, 2048 / kGroup)
             hpos = -1;
         }
     }
-    if (ok) {
-        const uint64_t code = morton(__fmul_rn(__fadd_rn(lo.x, hi.x), 0.5f), __fmul_rn(__fadd_rn(lo.y, hi.y), 0.5f),
-                                     __fmul_rn(__fadd_rn(lo.z, hi.z), 0.5f), g);
+    uint64_t code = 0;
+    if (mine) {
+        code = morton(__fmul_rn(__fadd_rn(e.lo.x, e.hi.x), 0.5f), __fmul_rn(__fadd_rn(e.lo.y, e.hi.y), 0.5f),
+                      __fmul_rn(__fadd_rn(e.lo.z, e.hi.z), 0.5f), g);
         sm.code[t + 1] = code;
-        codes_out[i] = code;
     }
     if (hpos >= 0)
         sm.code[t == 0 ? 0 : kGroup + t] =
             morton(__fmul_rn(__fadd_rn(hlo.x, hhi.x), 0.5f), __fmul_rn(__fadd_rn(hlo.y, hhi.y), 0.5f),
                    __fmul_rn(__fadd_rn(hlo.z, hhi.z), 0.5f), g);
     __syncthreads();
-    Climb c;
-    if (ok) {
-        const uint64_t c0 = sm.code[t + 1];
-        const uint32_t dl = i > 0 ? delta_star(sm.code[t], c0, (uint32_t)(i - 1)) : kInf;
-        uint32_t dr = kInf, drn = kInf;
-        if (i + 1 < n) {
-            const uint64_t c1 = sm.code[t + 2];
-            dr = delta_star(c0, c1, (uint32_t)i);
-            if (i + 2 < n) drn = delta_star(c1, sm.code[t + 3], (uint32_t)(i + 1));
-        }
-        leaf_write<kKind>(i, n, p_id, lo, hi, leaves, dl, dr, drn, c);
-    }
-    two_phase<kKind, kJitter>(sm, ok && n > 1, c, n, 0, a, t, inodes, leaves, store, flags,
-                              pend ? pend + (int64_t)blockIdx.x * kPendSlots : nullptr, jt);
+    if (sm.failed) return;
+    if (ok) codes_out[i] = code;
+    if (mine && !ok) atomicOr(flags, kFlagCorrupt);  // not a permutation: the sort failed
+    group_gaps(sm, i, n, flags);
+    __syncthreads();
+    e.gaps = leaf_gaps(sm);
+    if (ok) leaf_write<kKind>(i, n, p_id, e.lo, e.hi, leaves, (e.gaps >> 8) & 0xffu, e.gaps >> 16);
+    merge_group<kKind, kKind == LBVH_PRIM_POINTS, kJitter, false>(
+        sm, (int)min((int64_t)kGroup, n - a), e, OneTree{Owner{n, inodes, leaves, store}}, flags,
+        pend ? pend + (int64_t)blockIdx.x * kPendSlots : nullptr, kPendSlots, jt);
 }
 
-// Many trees at once, grouped by global sorted position: global position g
-// belongs to the instance b with off[b] <= g < off[b+1]; its tree's records
-// start at node_start[b] (float4 units) and its store words at store_start[b].
+// Many trees at once, grouped by global sorted position.
 template <int kKind>
-__global__ void __launch_bounds__(kGroup, 2048 / kGroup)
+__global__ void __launch_bounds__(kGroup, kGroupCtas)
     batch_construct_block_kernel(const uint64_t *__restrict__ codes, const uint32_t *__restrict__ perm,
                                  const float *__restrict__ prims, const int64_t *__restrict__ off,
                                  const int64_t *__restrict__ node_start, const int64_t *__restrict__ store_start,
                                  int count, int64_t total, float4 *nodes, unsigned long long *store,
-                                 uint32_t *flags) {
+                                 uint32_t *flags, uint4 *pend) {
     __shared__ GroupSmem sm;
-    if (group_start(sm, flags)) return;
+    group_start(sm, flags);
     const int t = threadIdx.x;
-    const int64_t g = (int64_t)blockIdx.x * kGroup + t;
-    const bool active = g < total;
-    const int b = active ? instance_of(off, count, g) : 0;
-    const int64_t o = active ? off[b] : 0;
-    const int n = active ? (int)(off[b + 1] - o) : 1;
-    float4 *inodes = nodes + (active ? node_start[b] : 0);
-    float4 *leaves = inodes + 2 * (int64_t)(n - 1);
-    Climb c;
-    const bool ok = active && leaf_step<kKind>((int)(g - o), n, codes + o, perm + o, (uint32_t)o, prims, leaves,
-                                               flags, c);
-    two_phase<kKind>(sm, ok && n > 1, c, n, o, (int64_t)blockIdx.x * kGroup, t, inodes, leaves,
-                     store + (active ? store_start[b] : 0), flags, nullptr);
+    const int64_t a = (int64_t)blockIdx.x * kGroup, g = a + t;
+    const bool mine = g < total;
+    if (mine) sm.code[t + 1] = codes[g];
+    if (t < 3) {
+        const int64_t h = t == 0 ? a - 1 : a + kGroup + t - 1;
+        if (h >= 0 && h < total) sm.code[t == 0 ? 0 : kGroup + t] = codes[h];
+    }
+    const uint32_t p_id = mine ? perm[g] : 0u;
+    // the instance: most groups lie in one, which the two ends show
+    if (t == 0) sm.instance[0] = instance_of(off, count, a);
+    if (t == 32) sm.instance[1] = instance_of(off, count, min(a + kGroup, total) - 1);
+    __syncthreads();
+    if (sm.failed) return;
+    int b = sm.instance[0];
+    if (mine && b < sm.instance[1]) b += instance_of(off + b, sm.instance[1] - b + 1, g);
+    const ManyTrees owner{off, node_start, store_start, nodes, store};
+    const Owner o = owner(b);
+    const int64_t base = __ldg(off + b);
+    const int i = mine ? (int)(g - base) : o.n;
+    const uint32_t p_own = p_id - (uint32_t)base;
+    const bool ok = mine && p_own < (uint32_t)o.n;
+    Element e{(uint32_t)i, (uint32_t)i, 0u, make_float3(0.f, 0.f, 0.f), make_float3(0.f, 0.f, 0.f), b};
+    if (ok) gather_box<kKind>(prims, p_id, e.lo, e.hi);
+    if (mine && !ok) atomicOr(flags, kFlagCorrupt);  // not a permutation of this tree: the sort failed
+    group_gaps(sm, i, o.n, flags);
+    __syncthreads();
+    e.gaps = leaf_gaps(sm);
+    if (ok) leaf_write<kKind>(i, o.n, p_own, e.lo, e.hi, o.leaves, (e.gaps >> 8) & 0xffu, e.gaps >> 16);
+    merge_group<kKind, kKind == LBVH_PRIM_POINTS, false, true>(sm, (int)min((int64_t)kGroup, total - a), e, owner, flags,
+                                                               pend + (int64_t)blockIdx.x * kPendSlots, kPendSlots,
+                                                               Jitter{});
+}
+
+// How far the merges go before the rest climbs. A merge is a launch of about
+// 6 us that its CTAs' own latency sets, a climb 1-2 us per level of the tree;
+// but an element list longer than its slots, which long lists near the root
+// of a large tree often are, makes every merge above it climb too. Points,
+// 63-bit codes, us, merging to the end / while there are over 4096 CTAs:
+// 20,000 20.4 / 28.6, 100,000 28.6 / 34.8, 300,000 38.8 / 40.9, 1.0M 65.4 /
+// 63.4, 2^23 379 / 307, 2^25 1217 / 1126 (never merging twice: 2^23 334,
+// 2^25 1268; while over 64: 2^23 321, 2^25 1139).
+constexpr int64_t kMergeToEnd = 512;
+constexpr int64_t kMergeAgain = 4096;
+
+// The merges above the groups: kPendSlots slots from each group, kMergedSlots
+// from each CTA of a merge, one region after the other in `pend`.
+int64_t merge_ctas(int64_t from, bool groups) {
+    const int64_t each = groups ? kGroup / kPendSlots : kGroup / kMergedSlots;
+    return (from + each - 1) / each;
+}
+
+template <bool kTrees, typename OwnerOf>
+void launch_merges(int64_t groups, int kind, const OwnerOf &owner, uint32_t *flags, void *pend, const Jitter &jt,
+                   cudaStream_t s) {
+    if (!pend || groups < 2) return;  // one group leaves nothing
+    uint4 *in = static_cast<uint4 *>(pend);
+    int64_t from = groups;
+    int64_t enough = merge_ctas(groups, true) <= kMergeToEnd ? 1 : kMergeAgain;
+    if (jt.max_ns) enough = groups;  // the hook is for climbs: what the first merge leaves climbs
+    const bool pts = kind == LBVH_PRIM_POINTS;
+    for (bool first = true;; first = false) {
+        const int64_t slots = from * (first ? kPendSlots : kMergedSlots), ctas = merge_ctas(from, first);
+        uint4 *out = ctas > enough ? in + slots : nullptr;
+        const auto pick = [&](auto a, auto b, auto c, auto d) { return first ? (pts ? a : b) : (pts ? c : d); };
+        auto k = pick(merge_pending_kernel<LBVH_PRIM_POINTS, kPendSlots, false, kTrees, OwnerOf>,
+                      merge_pending_kernel<LBVH_PRIM_BOXES, kPendSlots, false, kTrees, OwnerOf>,
+                      merge_pending_kernel<LBVH_PRIM_POINTS, kMergedSlots, false, kTrees, OwnerOf>,
+                      merge_pending_kernel<LBVH_PRIM_BOXES, kMergedSlots, false, kTrees, OwnerOf>);
+        if constexpr (!kTrees) {
+            if (jt.max_ns)
+                k = pick(merge_pending_kernel<LBVH_PRIM_POINTS, kPendSlots, true, kTrees, OwnerOf>,
+                         merge_pending_kernel<LBVH_PRIM_BOXES, kPendSlots, true, kTrees, OwnerOf>,
+                         merge_pending_kernel<LBVH_PRIM_POINTS, kMergedSlots, true, kTrees, OwnerOf>,
+                         merge_pending_kernel<LBVH_PRIM_BOXES, kMergedSlots, true, kTrees, OwnerOf>);
+        }
+        k<<<(unsigned)ctas, kGroup, 0, s>>>(in, slots, owner, flags, out, jt);
+        count_launches(1);
+        if (!out) return;
+        in = out;
+        from = ctas;
+    }
 }
 
 }  // namespace
 
+size_t construct_pend_bytes(int64_t n) {
+    int64_t from = (n + kGroup - 1) / kGroup, slots = from * kPendSlots;
+    for (bool first = true; from > 1; first = false) {
+        from = merge_ctas(from, first);
+        slots += from * kMergedSlots;
+    }
+    return (size_t)slots * sizeof(uint4);
+}
+
 void launch_batch_construct(const uint64_t *sorted_codes, const uint32_t *perm, const float *prims,
                             const BatchTables &bt, int kind, float4 *nodes, unsigned long long *store,
-                            uint32_t *flags, cudaStream_t s) {
+                            uint32_t *flags, void *pend, cudaStream_t s) {
     if (bt.total_prims <= 0) return;
     const unsigned blocks = (unsigned)((bt.total_prims + kGroup - 1) / kGroup);
     auto k = kind == LBVH_PRIM_POINTS ? batch_construct_block_kernel<LBVH_PRIM_POINTS>
                                       : batch_construct_block_kernel<LBVH_PRIM_BOXES>;
     k<<<blocks, kGroup, 0, s>>>(sorted_codes, perm, prims, bt.prim_off, bt.node_start, bt.store_start, bt.count,
-                                bt.total_prims, nodes, store, flags);
+                                bt.total_prims, nodes, store, flags, static_cast<uint4 *>(pend));
     count_launches(1);
+    launch_merges<true>(blocks, kind, ManyTrees{bt.prim_off, bt.node_start, bt.store_start, nodes, store}, flags, pend,
+                        Jitter{}, s);
 }
-
-size_t construct_pend_bytes(int64_t n) { return (size_t)((n + kGroup - 1) / kGroup) * kPendSlots * sizeof(uint4); }
 
 namespace {
 
@@ -565,19 +811,6 @@ Jitter jitter_setting() {
     j.seed = g_jitter_seed.load(std::memory_order_relaxed);
     j.max_ns = g_jitter_ns.load(std::memory_order_relaxed);
     return j;
-}
-
-void launch_pending(int64_t n, int kind, float4 *inodes, float4 *leaves, unsigned long long *store,
-                    uint32_t *flags, void *pend, const Jitter &jt, cudaStream_t s) {
-    if (!pend || n < 2) return;
-    const int64_t slots = (n + kGroup - 1) / kGroup * kPendSlots;
-    const unsigned blocks = (unsigned)((slots + 255) / 256);
-    const bool pts = kind == LBVH_PRIM_POINTS;
-    auto k = jt.max_ns ? (pts ? climb_pending_kernel<LBVH_PRIM_POINTS, true> : climb_pending_kernel<LBVH_PRIM_BOXES, true>)
-                       : (pts ? climb_pending_kernel<LBVH_PRIM_POINTS, false>
-                              : climb_pending_kernel<LBVH_PRIM_BOXES, false>);
-    k<<<blocks, 256, 0, s>>>(static_cast<uint4 *>(pend), slots, (int)n, inodes, leaves, store, flags, jt);
-    count_launches(1);
 }
 
 }  // namespace
@@ -596,7 +829,7 @@ void launch_construct(const uint64_t *sorted_codes, const uint32_t *perm, const 
     k<<<blocks, kGroup, 0, s>>>(sorted_codes, perm, prims, (int)n, inodes, leaves, store, flags,
                                 static_cast<uint4 *>(pend), jt);
     count_launches(1);
-    launch_pending(n, kind, inodes, leaves, store, flags, pend, jt, s);
+    launch_merges<false>(blocks, kind, OneTree{Owner{(int)n, inodes, leaves, store}}, flags, pend, jt, s);
 }
 
 void launch_construct_encode(const uint32_t *perm, const float *prims, const float *bounds, int bits, int64_t n,
@@ -613,7 +846,7 @@ void launch_construct_encode(const uint32_t *perm, const float *prims, const flo
     k<<<blocks, kGroup, 0, s>>>(perm, prims, bounds, bits / 3, (int)n, codes_out, inodes, leaves, store, flags,
                                 static_cast<uint4 *>(pend), jt);
     count_launches(1);
-    launch_pending(n, kind, inodes, leaves, store, flags, pend, jt, s);
+    launch_merges<false>(blocks, kind, OneTree{Owner{(int)n, inodes, leaves, store}}, flags, pend, jt, s);
 }
 
 }  // namespace lbvh

@@ -276,9 +276,8 @@ void launch_variant_second(int algorithm, const uint64_t *codes, const uint32_t 
                            int64_t n, int kind, float4 *inodes, float4 *leaves, void *scratch,
                            unsigned long long *store, uint32_t *flags, cudaStream_t s);
 // pend (nullable): construct_pend_bytes(n) of zeroed scratch, left zeroed.
-// With it, the climbs that leave a CTA's group of leaves run in a second
-// kernel with full warps instead of holding their CTA; without it (the
-// no-allocation entry point) they run in place.
+// With it, what a CTA's group of leaves leaves over is merged by a second
+// kernel; without it (the no-allocation entry point) it climbs in place.
 size_t construct_pend_bytes(int64_t n);
 void launch_construct(const uint64_t *sorted_codes, const uint32_t *perm, const float *prims,
                       int64_t n, int kind, float4 *inodes, float4 *leaves,
@@ -487,7 +486,7 @@ void launch_batch_encode(const float *data, int kind, bool queries, const BatchT
                          const float *bounds, uint64_t *keys, uint32_t *hist, cudaStream_t s, bool hilbert = false);
 void launch_batch_construct(const uint64_t *sorted_codes, const uint32_t *perm, const float *prims,
                             const BatchTables &bt, int kind, float4 *nodes, unsigned long long *store,
-                            uint32_t *flags, cudaStream_t s);
+                            uint32_t *flags, void *pend, cudaStream_t s);
 // The collecting walk over all instances' queries (instance of a query found
 // from query_off), and the overflow walk + list sort with device-side counts.
 void launch_batch_collect(const float4 *nodes, int kind, const BatchTables &bt, const QueryArgs &q,
