@@ -419,10 +419,10 @@ lbvh_status query_count(lbvh_tree_t t, lbvh::QueryArgs &qa, int64_t *d_offsets,
     t->prof.clear(LBVH_STAGE_QCOUNT, LBVH_STAGE_QORDER + 1);
     const int choice = t->walk_choice >= 0 ? t->walk_choice : tune_walk_choice(t->n, t->bits, t->kind, qa.qkind, 1);
     qa.walk = walk_choice_kind(choice);
-    // spheres and boxes walk the leaf blocks unless the tuner chose a walk of the nodes
+    // by the leaf blocks unless the tuner chose a walk of the nodes
     RangeWalk how = kRangeNodes;
-    if (qa.walk == kWalkThread && qa.qkind != LBVH_Q_RAY && t->n > 0 && !t->loaded)
-        how = range_walk(qa.nq, t->n, own_order(t, qa));
+    if (qa.walk == kWalkThread && t->n > 0 && !t->loaded)
+        how = range_walk(qa.qkind, qa.nq, t->n, own_order(t, qa));
     // few queries on a large tree whose blocks nobody has packed: the second such call packs them
     // (0.2 ms at 2^25 leaves, about what a call saves), so a tree that is queried once never pays
     if (how == kRangeSparse && !t->packed_ok && t->n > kPackForFew && !t->few_seen) {
@@ -431,7 +431,10 @@ lbvh_status query_count(lbvh_tree_t t, lbvh::QueryArgs &qa, int64_t *d_offsets,
     }
     t->prof.begin(LBVH_STAGE_QORDER, s);
     lbvh_status ost = LBVH_OK;
-    if (how != kRangeSparse || own_order(t, qa))
+    // few rays by 8 lanes: an order pays from about 256 per SM (30,000 on 2^23 boxes 348 us with one, 361
+    // without; 60,000 484, 553; 20,000 on 30,000 68, 49)
+    const bool order_rays = qa.qkind == LBVH_Q_RAY && qa.nq > 256 * (int64_t)device_sm_count();
+    if (how != kRangeSparse || own_order(t, qa) || order_rays)
         ost = query_order(t, qa, s, walk_choice_order_bits(choice), how == kRangePackets ? kCodeHilbert : kCodeLow);
     t->prof.end(LBVH_STAGE_QORDER, s);
     if (ost != LBVH_OK) return ost;

@@ -426,7 +426,7 @@ enum RangeWalk : int {
     kRangeSparse,   // 8 lanes per query through the blocks, in any order
     kRangeNodes     // Algorithm 1, a thread per query
 };
-RangeWalk range_walk(int64_t nq, int64_t n, bool sorted);
+RangeWalk range_walk(int qkind, int64_t nq, int64_t n, bool sorted);
 // Leaves up to which packing them for one call of few queries pays.
 constexpr int64_t kPackForFew = int64_t(1) << 23;
 // The queries of qs.sparse_list.

@@ -363,7 +363,15 @@ __global__ void __launch_bounds__(kSparseThreads)
     typename QueryOf<kQ>::type q{};
     if (has && ok) q = QueryOf<kQ>::load(qa, qi);
     if (has && !ok && (threadIdx.x & 7) == 0) __stcs(qs.counts + qi, 0u);
-    sparse_walk<kQ, kP>(Blocks{leaves, rec, n, start0}, s_stack[threadIdx.x >> 3], q, has && ok, qi, qs, ctl);
+    const Blocks blocks{leaves, rec, n, start0};
+    uint32_t *stack = s_stack[threadIdx.x >> 3];
+    if constexpr (kQ == LBVH_Q_RAY) {  // the general test if any of the warp's rays has a parallel axis
+        if (!__any_sync(kFull, q.parallel != 0)) {
+            sparse_walk<kP>(blocks, stack, SlantedRay{q}, has && ok, qi, qs, ctl);
+            return;
+        }
+    }
+    sparse_walk<kP>(blocks, stack, q, has && ok, qi, qs, ctl);
 }
 
 }  // namespace
@@ -396,7 +404,14 @@ void launch_batch_pack(const float4 *nodes, int kind, const BatchTables &bt, flo
 // apart to share nodes) and enough packets to fill the GPU; below about 1000
 // queries per SM the 8 lanes have the shorter chain of loads, and need no
 // order; in between Algorithm 1 stays.
-RangeWalk range_walk(int64_t nq, int64_t n, bool sorted) {
+// Rays have no packets. 8 lanes per ray against a thread (2^23 mixture boxes,
+// walk and order, us): 30,000 random segments 361 / 791, 60,000 484 / 833,
+// 120,000 758 / 880, 250,000 1407 / 1100, 2^20 5364 / 2656; 20,000 on
+// 30,000 49 / 130, 100,000 on 200,000 249 / 252. Few rays take as long as the
+// longest walk, which is shorter by blocks; many take as long as their
+// instructions.
+RangeWalk range_walk(int qkind, int64_t nq, int64_t n, bool sorted) {
+    if (qkind == LBVH_Q_RAY) return nq <= 640 * (int64_t)device_sm_count() ? kRangeSparse : kRangeNodes;
     const bool dense = n <= 4 * nq;
     const int64_t few = (dense ? (sorted ? 256 : 640) : 1024) * (int64_t)device_sm_count();
     if (nq <= few) return kRangeSparse;
@@ -411,7 +426,11 @@ void dispatch_range_kinds(int qkind, int pkind, F &&f) {
     using Boxes = std::integral_constant<int, LBVH_PRIM_BOXES>;
     using SphereQ = std::integral_constant<int, LBVH_Q_SPHERE>;
     using BoxQ = std::integral_constant<int, LBVH_Q_BOX>;
-    if (qkind == LBVH_Q_SPHERE) {
+    using RayQ = std::integral_constant<int, LBVH_Q_RAY>;
+    if (qkind == LBVH_Q_RAY) {
+        if (pkind == LBVH_PRIM_POINTS) f(RayQ{}, Points{});
+        else f(RayQ{}, Boxes{});
+    } else if (qkind == LBVH_Q_SPHERE) {
         if (pkind == LBVH_PRIM_POINTS) f(SphereQ{}, Points{});
         else f(SphereQ{}, Boxes{});
     } else {
@@ -432,7 +451,7 @@ void launch_query_packets(const TreeView &t, const float4 *rec, const QueryArgs 
         if (how == kRangeSparse) {
             const unsigned blocks = (unsigned)((q.nq + kSparseThreads / 8 - 1) / (kSparseThreads / 8));
             sparse_kernel<Q, P><<<blocks, kSparseThreads, 0, s>>>(t.leaves, rec, n, start0, q, qs, ctl);
-        } else {
+        } else if constexpr (Q != LBVH_Q_RAY) {
             const unsigned blocks = (unsigned)((q.nq + 32 * kPacketWarps - 1) / (32 * kPacketWarps));
             packet_kernel<Q, P><<<blocks, 32 * kPacketWarps, 0, s>>>(t.leaves, rec, n, start0, q, qs, ctl);
         }
@@ -446,8 +465,9 @@ void launch_batch_packets(const float4 *nodes, int kind, const float4 *rec, cons
     if (q.nq <= 0) return;
     const unsigned blocks = (unsigned)((q.nq + 32 * kPacketWarps - 1) / (32 * kPacketWarps));
     dispatch_range_kinds(q.qkind, kind, [&](auto qk, auto pk) {
-        batch_packet_kernel<decltype(qk)::value, decltype(pk)::value><<<blocks, 32 * kPacketWarps, 0, s>>>(nodes, rec, bt,
-                                                                                                           q, qs, ctl);
+        if constexpr (decltype(qk)::value != LBVH_Q_RAY)
+            batch_packet_kernel<decltype(qk)::value, decltype(pk)::value>
+                <<<blocks, 32 * kPacketWarps, 0, s>>>(nodes, rec, bt, q, qs, ctl);
     });
     count_launches(1);
     launch_batch_collect_left(nodes, kind, bt, q, qs, ctl, s);

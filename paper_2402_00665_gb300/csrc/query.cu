@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kThreads)
             const int64_t qi = has ? thread_query(qa, (int64_t)e.x * 32 + at) : 0;
             typename QueryOf<kQ>::type q{};
             if (has) q = QueryOf<kQ>::load(qa, qi);
-            sparse_walk<kQ, kP>(blocks, s_stack[threadIdx.x >> 3], q, has, qi, qs, ctl);
+            sparse_walk<kP>(blocks, s_stack[threadIdx.x >> 3], q, has, qi, qs, ctl);
         }
         return;
     }

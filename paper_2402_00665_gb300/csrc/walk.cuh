@@ -244,9 +244,9 @@ struct Blocks {
 // shared memory per 8 lanes. Warp-wide; `go`: the 8 lanes have a query (qi).
 constexpr int kSparseStack = 80;  // one block per step: 7 entries per height (9 below the root) and 8 at the end
 
-template <int kQ, int kP>
-__device__ __forceinline__ void sparse_walk(const Blocks &t, uint32_t *stack, const typename QueryOf<kQ>::type &q,
-                                            bool go, int64_t qi, const QueryScratch &qs, Control *ctl) {
+template <int kP, typename Q>
+__device__ __forceinline__ void sparse_walk(const Blocks &t, uint32_t *stack, const Q &q, bool go, int64_t qi, const QueryScratch &qs,
+                                            Control *ctl) {
     const int lane = threadIdx.x & 31, sl = lane & 7, shift = lane & 24;
     const uint32_t below = (1u << sl) - 1u;
     uint32_t *slot = qs.slots + qi * kSlot;

@@ -222,6 +222,32 @@ def test_ray_order(nq):
     t.close()
 
 
+@pytest.mark.parametrize("kind", ["points", "boxes"])
+@pytest.mark.parametrize("n", [1, 8, 65, 513, 40000])
+@pytest.mark.parametrize("nq", [1, 33, 5000, 50_000, 110_003])
+def test_rays(n, kind, nq):
+    """8 lanes per ray, with and without an order, and a thread per ray (110,003): rays with parallel axes,
+    unbounded, empty and not finite."""
+    lbvh = L()
+    pts = inputs.uniform_points(n, seed=n)
+    tree = lbvh.Tree()
+    if kind == "points":  # some rays start at points, so they hit them
+        tree.build(pts, lbvh.POINTS, 63)
+    else:
+        tree.build(boxes_at(pts, 0.02), lbvh.BOXES, 63)
+    rng = np.random.default_rng(nq)
+    rays = np.zeros((nq, 8), np.float32)
+    rays[:, :3] = pts[rng.integers(0, n, nq)]
+    rays[:, 4:7] = rng.normal(size=(nq, 3))
+    rays[:, 7] = rng.random(nq)
+    rays[::5, 4] = 0.0
+    rays[::7, 7] = np.inf
+    rays[::11, 7] = -1.0
+    rays[3::97, 5] = np.nan
+    both(tree, torch.from_numpy(rays).cuda(), lbvh.RAY)
+    tree.close()
+
+
 @pytest.mark.parametrize("bits", [3, 30, 33, 63])
 @pytest.mark.parametrize("n", [1, 2, 31, 33, 1023, 1024, 1025, 4096, 4097, 8191, 8192, 8193, 16384, 16385])
 def test_small_builds(n, bits):
