@@ -199,9 +199,9 @@ constexpr uint32_t kNoNeighbours = 0xffffffffu;  // counts[]: a query with a non
 
 template <typename T>
 __device__ __forceinline__ void order2(T &a, T &b) {
-    const T lo = a < b ? a : b, hi = a < b ? b : a;
+    const T lo = a < b ? a : b;
+    b = a ^ b ^ lo;  // a second select instead: 2.8M points, k = 32 4.45 ms, so 4.01; 5.0M, k = 16 3.80, 3.76
     a = lo;
-    b = hi;
 }
 template <>
 __device__ __forceinline__ void order2<float>(float &a, float &b) {
