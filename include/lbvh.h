@@ -259,8 +259,8 @@ lbvh_status lbvh_query(lbvh_tree_t tree, const float *d_queries, int64_t nq, int
                        uint32_t **d_hits, uint64_t *total, lbvh_stream_t stream);
 
 /* Measurement: the number of leaves and internal nodes Algorithm 1 visits
- * for these queries (the collecting walk's work), summed over all queries,
- * walked in the same order as lbvh_query_into; no hits are kept. Arguments
+ * for these queries, one thread per query, summed over all queries; no hits
+ * are kept. lbvh_query_into may answer them by other walks. Arguments
  * as lbvh_query_into. Synchronises `stream`. */
 lbvh_status lbvh_tree_walk_visits(lbvh_tree_t tree, const float *d_queries, int64_t nq, int qkind,
                                   const float *d_radii, float radius, uint64_t *leaf_visits,
@@ -270,9 +270,9 @@ lbvh_status lbvh_tree_walk_visits(lbvh_tree_t tree, const float *d_queries, int6
 #define LBVH_KNN_MAX_K 256
 
 /* The k nearest primitives of each query point: the distance range search of
- * Sec. 1 asked for its k closest answers, walked stacklessly (Algorithm 1)
- * with a ball whose radius is the current k-th best distance, which only
- * shrinks, so the walk never skips a subtree that could hold an answer.
+ * Sec. 1 asked for its k closest answers: a walk with a ball whose radius
+ * bounds the k-th best distance from above, so that it never skips a subtree
+ * that could hold an answer.
  *   d_queries  query points float[nq][3].
  *   k          1 .. LBVH_KNN_MAX_K.
  *   d_idx      uint32[nq][k] out: row q holds the min(k, n) nearest primitive
@@ -539,11 +539,11 @@ enum {
     LBVH_STAGE_ENCODE = 1,     /* Morton codes + sort digit histograms */
     LBVH_STAGE_SORT0 = 2,      /* radix-sort pass k is LBVH_STAGE_SORT0 + k, k < 8 */
     LBVH_STAGE_CONSTRUCT = 10, /* Algorithm 4: nodes, boxes, skips */
-    LBVH_STAGE_QCOUNT = 11,    /* Algorithm 1 walk: counts, short sorted hit lists */
+    LBVH_STAGE_QCOUNT = 11,    /* the collecting walk: counts and hits (and the leaf blocks, when they are due) */
     LBVH_STAGE_QSCAN = 12,     /* exclusive scan of the counts */
     LBVH_STAGE_QFILL = 13,     /* short lists copied to their CSR positions */
-    LBVH_STAGE_QFIXUP = 14,    /* second walk + sort for lists longer than 32 */
-    LBVH_STAGE_QORDER = 15,    /* Morton order of the query centres (encode + sort) */
+    LBVH_STAGE_QFIXUP = 14,    /* copy (or second walk) + sort for lists longer than 64 */
+    LBVH_STAGE_QORDER = 15,    /* order of the query centres along a curve (encode + sort) */
     LBVH_STAGE_SECOND = 16,    /* second pass of lbvh_build_variant's Karras / Apetrei builds */
     LBVH_STAGE_SORTRUNS = 17,  /* codes wider than 30 bits: the sort passes cover the codes' top bits
                                   beside the index; this stage orders the runs of equal top bits */
@@ -579,12 +579,14 @@ uint64_t lbvh_kernel_launches(void);
  *                 byte (one pass) fewer of the codes' top bits, leaving more
  *                 elements in runs of equal sorted bits for the runs stage
  *                 (Sec. 3.1 step 2 either way: the same sorted order);
- *   walk variant  how Algorithm 1's collecting walk runs: 0 one thread per
- *                 query, 1/2/3 groups of 8/16/32 lanes walking the union of
+ *   walk variant  how the collecting walk runs: 0 chosen by the sizes (32
+ *                 queries per warp or 8 lanes per query over blocks of 8
+ *                 leaves, or Algorithm 1 with one thread per query); the
+ *                 others are Algorithm 1: 1/2/3 groups of 8/16/32 lanes walking the union of
  *                 their queries' paths together, 4 one thread per query in
- *                 CTAs of 512 threads instead of 256; 5-9 the same with the
- *                 queries put in the Morton order of 24-bit codes of their
- *                 centres (one sort pass fewer) instead of 30-bit ones
+ *                 CTAs of 512 threads; 5-9 the same with the queries
+ *                 ordered by 24-bit codes of their centres (one sort pass
+ *                 fewer) instead of 30-bit ones
  *                 (lbvh_walk_variant_count() = 10).
  * A process-wide cache holds the choice for each configuration (the GPU's
  * name, ceil(log2 n), Morton bits, primitive kind, query kind, trees built

@@ -329,10 +329,11 @@ lbvh_status read_control(lbvh_tree_t t, cudaStream_t s) {
 
 constexpr int64_t kOrderMinQueries = 2048;  // below this, walk in input order
 constexpr int64_t kOrderMinRays = 4096;
-// Morton bits of the query order: 30 (4 sort passes) by default, or 24 (3
-// passes) as the tuner's choice. 24 bits walk uniform queries as fast as 30,
-// but on clustered queries (a Gaussian mixture) the coarser cells cost more
-// walk time than the pass saves; order changes speed only. Batches use 30.
+// Bits of the query order: 30 (4 sort passes; on the Hilbert curve these
+// hold 32) by default, or 24 (3 passes) as the tuner's choice. 24 bits walk
+// uniform queries as fast as 30, but on clustered queries (a Gaussian mixture)
+// the coarser cells cost more walk time than the pass saves; order changes
+// speed only. Batches use 30.
 constexpr int order_bits() { return 30; }
 
 // The queries are the primitives of the last build (same pointer and count):
@@ -344,8 +345,9 @@ bool own_order(lbvh_tree_t t, const lbvh::QueryArgs &qa) {
 }
 
 // The order in which threads take the queries: the Morton order of the query
-// centres inside the tree's bounds (encode + radix sort of `bits`-bit codes,
-// the build's own kernels). Queries that are the primitives of the last build
+// centres inside the tree's bounds, or the Hilbert order for packets, whose
+// neighbours stay close (encode + radix sort of `bits`-bit codes, the build's
+// own kernels). Queries that are the primitives of the last build
 // (same pointer and count) reuse the build's permutation. Order only changes
 // speed, never results.
 lbvh_status query_order(lbvh_tree_t t, lbvh::QueryArgs &qa, cudaStream_t s, int bits = order_bits(),

@@ -43,7 +43,7 @@ struct Control {
     uint32_t run_fallback;         //   a run too long for one CTA was met,
     uint32_t run_sort_count;       //   elements of the fallback sort,
     uint32_t run_heads;            //   runs listed for short_runs_kernel (in this order)
-    uint32_t sparse_filled;        // packets left to Algorithm 1
+    uint32_t sparse_filled;        // packets left to collect_left_kernel
     uint32_t scan_ticket;          // tiles of the counts' scan
     uint32_t pad[2];
 };
@@ -305,8 +305,10 @@ struct QueryArgs {
     const uint32_t *order;  // null: thread i walks query i; else query order[i]
     int walk = 0;           // kWalk*: how the collecting walk runs
 };
-// The collecting walk: one thread per query (CTAs of 256 threads, or of 512),
-// or groups of 8, 16 or 32 lanes walking together (walk_group in query.cu).
+// The collecting walk: kWalkThread, the default, is range_walk's choice (leaf
+// blocks, or Algorithm 1 with one thread per query in CTAs of 256); the others
+// are Algorithm 1: one thread per query in CTAs of 512, or groups of 8, 16 or
+// 32 lanes walking together (walk_group in query.cu).
 enum : int {
     kWalkThread = 0,
     kWalkGroup8 = 1,
@@ -316,8 +318,8 @@ enum : int {
     kWalkKinds = 5
 };
 // A tree's walk choice c (the tuner's index, lbvh_tree_set_tuning): walk kind
-// c % kWalkKinds, and the Morton bits of the query order: 30 (4 sort passes)
-// for c < kWalkKinds, 24 (3 passes) above.
+// c % kWalkKinds, and the bits of the query order: 30 (4 sort passes; 32 on
+// the packets' Hilbert curve) for c < kWalkKinds, 24 (3 passes) above.
 constexpr int kWalkChoices = 2 * kWalkKinds;
 inline int walk_choice_kind(int c) { return c < 0 ? kWalkThread : c % kWalkKinds; }
 inline int walk_choice_order_bits(int c) { return c >= kWalkKinds ? 24 : 30; }
@@ -342,7 +344,7 @@ struct QueryScratch {
     uint32_t *spill_head;     // nq: first spill chunk of query q
     uint32_t *spill;          // spill_chunks * kSpillChunkWords
     uint32_t spill_chunks;
-    uint2 *sparse_list;       // nq / 32 + 1: packets left to Algorithm 1 (32 walk positions from 32 x, lanes y)
+    uint2 *sparse_list;       // nq / 32 + 1: packets left to collect_left_kernel (32 walk positions from 32 x, lanes y)
 };
 // The collecting walk (counts, short sorted lists, overflow list).
 void launch_query_collect(const TreeView &t, const QueryArgs &q, const QueryScratch &qs, Control *ctl,

@@ -23,9 +23,10 @@
 //      tested by every lane against its own query with the exact predicate,
 //      the candidates' coordinates broadcast from shared memory.
 // sparse_kernel  8 lanes per query: the lanes test the 8 children of one
-//   block at a time with the query's own predicate. For few queries (more
-//   warps in flight, and no query order to compute) and for the packets that
-//   packet_kernel leaves to it: queries too far apart for a common region.
+//   block at a time with the query's own predicate. For few queries and few
+//   rays (more warps in flight, a shorter chain of loads, no query order to
+//   compute). Packets whose queries lie too far apart for a common region are
+//   left to collect_left_kernel (query.cu).
 //
 // Both report exactly the primitives whose own test holds, like Algorithm 1
 // (the hit lists are sorted afterwards, so their order here does not matter).
@@ -41,7 +42,6 @@ namespace lbvh {
 namespace {
 
 // ---------------------------------------------------------------- boxes of the leaf blocks
-
 
 struct Bounds {
     float3 lo, hi;

@@ -317,8 +317,8 @@ __device__ __forceinline__ float3 middle(const Box &b) {
 }
 
 // The lanes of `mine` before its widest step from one query to the next (the
-// order is a Morton curve: it jumps now and then, and a packet that holds a
-// jump is two packets far apart). `mine` is a run of lanes, two at least.
+// order may be a Morton curve, which jumps now and then, or queries may be
+// scarce on their curve: such a packet is two packets far apart). `mine` is a run of lanes, two at least.
 template <typename Q>
 __device__ __forceinline__ uint32_t before_jump(const Q &q, uint32_t mine) {
     const int lane = threadIdx.x & 31;

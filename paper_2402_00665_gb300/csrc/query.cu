@@ -1,6 +1,9 @@
 // query.cu -- stackless range queries (Algorithm 1) and CSR assembly.
 //
-// Each thread walks the tree for one query: start at the root (id 0); when
+// Sphere and box queries take the leaf blocks (packet.cu) unless they are
+// many but far apart, and few rays too; what follows is the walk of the nodes
+// for the others, for trees from checkpoints (it checks their links) and for
+// the tuner's other walk variants. Each thread walks the tree for one query: start at the root (id 0); when
 // the predicate holds on an internal node go to its left child, on a leaf
 // report it and go to its skip; when it fails go to the skip; stop at the
 // sentinel. Every step runs the same code for internal nodes and leaves: a
@@ -18,10 +21,11 @@
 //           because fl(x - y) = -fl(y - x).
 //   box     lo_q <= hi_b and lo_b <= hi_q on every axis.
 //   ray     the slab test of a segment {origin, tmin, direction, tmax}
-//           (see hits(const Ray &...)); rays are walked in input order.
+//           (see hits(const Ray &...)); many rays are walked by the 256
+//           cells of their middles.
 //
 // Threads take the queries in the order given by QueryArgs::order (the
-// queries sorted by the Morton code of their centre, so that a warp's walks
+// queries sorted along a curve through their centres, so that a warp's walks
 // visit the same nodes), and write results at the query's own index.
 //
 // CSR in one walk:
@@ -32,12 +36,13 @@
 //             and the hit count at q. Slot q rather than slot i: the copy
 //             then reads the slots in order (copy 1.86 -> 1.45 ms on 2^25
 //             uniform points; the walk's stores are scattered either way).
-//   scan      exclusive scan of the counts -> offsets, total (host reads it).
+//   scan      exclusive scan of the counts -> offsets, total (host reads
+//             it): one kernel with a bounded look-back, or three for many.
 //   copy      in query order: each thread loads one slot of up to 32 hits
-//             into registers and sorts it with a bitonic network; the warp
-//             writes its 32 lists, adjacent in the CSR, through shared
-//             memory, one coalesced list per step; lists of 33..64 hits are
-//             sorted by the whole warp (two values per lane, shuffles).
+//             into registers and sorts it with an odd-even merge network;
+//             the warp's 32 lists, adjacent in the CSR, leave through shared
+//             memory as one run; lists of 33..64 hits are sorted by the
+//             whole warp (two values per lane, shuffles).
 //   overflow  hits past the slot go on, during the same walk, to chunks of a
 //             shared spill pool; those lists are copied (slot + chunks) to
 //             their CSR ranges; only when the pool runs out does a query walk
