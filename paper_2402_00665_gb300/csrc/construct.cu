@@ -254,15 +254,15 @@ __device__ __forceinline__ void climb_global(Climb c, int n, float4 *inodes, con
 // This is bound by instructions issued, not by memory. With a thread per
 // leaf climbing through shared-memory words (block-scope exchanges, half the
 // lanes gone after each level) this pass took 1226 instructions per warp of
-// leaves and 1.57 ms at 2^25 points, 63-bit codes; now 757 and 1.13 (16,384
-// points 32.7 -> 19.0 us, 1.0M 81.9 -> 65.5, 2^23 428 -> 309). Groups of 128 leaves, 12 CTAs to
+// leaves and 1.57 ms at 2^25 points, 63-bit codes; now 757 and 1.14 (16,500
+// points 31.7 -> 24.5 us, 1.0M 79.8 -> 64.4, 2^23 426 -> 311; a clustered
+// mixture 41.9 -> 26.5, 92.1 -> 75.7, 438 -> 319, 2^25 1589 -> 1149). Groups of 128 leaves, 12 CTAs to
 // an SM, against 256 with 6: 1.29 and 1.36 ms before the merges above them;
 // 512: 1.48; 10 CTAs: 1.39. More CTAs take the L1's room for shared memory
 // and the gathers miss: 14 CTAs 1.87.
 constexpr int kGroup = 128;
 constexpr int kWarps = kGroup / 32;
-static_assert(kWarps == 4, "GroupSmem::count is one word");
-constexpr int kRounds = 3;
+static_assert(kWarps == 4, "MergeSmem::count is one word");
 constexpr int kGroupCtas = 12;  // CTAs of an SM
 constexpr int kRuns = 4;  // runs of 2 .. 2^kRuns lanes in a warp's table
 
@@ -277,30 +277,34 @@ struct ElementList {
     int tree[kGroup];  // batches
 };
 
-struct GroupSmem {
+// A merging CTA; the groups' CTAs also hold codes and gaps.
+struct MergeSmem {
     union {
         uint64_t code[kGroup + 3];  // sorted codes a-1 .. a+kGroup+1
         RunTable table[kWarps];
         ElementList list;
     };
-    uint8_t gap[kGroup + 4];  // delta* at a-1 .. a+kGroup (kInf between two trees)
     alignas(4) uint8_t count[4];  // elements a warp leaves
-    int instance[2];              // batches: of the first and the last leaf
     int failed;
+};
+struct GroupSmem : MergeSmem {
+    uint8_t gap[kGroup + 4];  // delta* at a-1 .. a+kGroup (kInf between two trees)
+    int instance[2];          // batches: of the first and the last leaf
 };
 
 // Elements left by a group: the CTA hands them, in order, to
-// merge_pending_kernel through its own kPendSlots slots (16 bytes each: l, r,
-// the three delta* values with a valid bit, the tree). On uniform points a
-// group of 128 leaves has 7.3 of them on average, 1024 leaves 10.3, 7680
-// 13.2; more than 16, 20 and 25 have none of 23,000 groups, none of 2,900 and
-// one of 2,000 (a mixture of tight clusters: one of 1000, 20 and 200). A list
-// longer than its slots climbs in place and marks its first slot
-// kPendClimbed, and then the merge above climbs too.
-constexpr int kPendSlots = 16;
-constexpr int kMergedSlots = 25;  // of a CTA of merge_pending_kernel
-constexpr uint32_t kPendValid = 1u << 31;
-constexpr uint32_t kPendClimbed = 1u << 30;
+// merge_pending_kernel through its own slots (16 bytes each: l, r, the three
+// delta* values, the tree; the first one also carries how many there are, so
+// only it has to be zero between builds). On uniform points a group of 128
+// leaves has 7.3 of them on average, 1024 leaves 10.3, 7680 13.2, clustered
+// ones 8.1, 12.3 and 15.7 (27 at most of 2,300). What a warp leaves always
+// fits the slots, and 8 groups, or 5 CTAs of a merge, almost always fit a
+// merge's 128 threads (with 256 the construct of 2^25 points took 1.23 ms, not
+// 1.14; with 256 in the second merge alone 1.18). A longer list (chains of leaves with growing gaps) climbs in place and is
+// marked kPendClimbed, and then the merge above climbs too.
+constexpr int kPendSlots = 32;
+constexpr int kPendCount = 24;  // first bit of the count
+constexpr uint32_t kPendClimbed = 1u << 31;
 
 struct Owner {  // a tree's leaves and memory
     int n;
@@ -397,11 +401,12 @@ __device__ __forceinline__ bool merge_elements(RunTable &table, int m, Element &
 // them in rounds; what is left goes to the CTA's slots (pend), or climbs.
 // Every thread of the CTA calls this; the tables' memory is free.
 template <int kKind, bool kPoints, bool kJitter, bool kTrees, typename OwnerOf>
-__device__ __forceinline__ void merge_group(GroupSmem &sm, int count, Element e, const OwnerOf &owner,
-                                            uint32_t *flags, uint4 *pend, int slots, const Jitter &jt) {
+__device__ __forceinline__ void merge_group(MergeSmem &sm, int count, Element e, const OwnerOf &owner,
+                                            uint32_t *flags, uint4 *pend, const Jitter &jt) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     bool keep = false;
     uint32_t kept = 0u;
+    int at = 0, left = 0;  // the element's place among those left, and their number
     for (int round = 0;; ++round) {
         const int m = min(count - 32 * warp, 32);
         keep = false;
@@ -412,13 +417,16 @@ __device__ __forceinline__ void merge_group(GroupSmem &sm, int count, Element e,
             keep = keep && (e.gaps & 0xffffu) != (kInf | kInf << 8);
         }
         kept = __ballot_sync(~0u, keep);
-        if (count <= 32 || round == kRounds - 1) break;
-        if (lane == 0) sm.count[warp] = (uint8_t)__popc(kept);
+        at = __popc(kept & ((1u << lane) - 1u));
+        left = __popc(kept);
+        if (count <= 32) break;  // all of them the first warp's
+        if (lane == 0) sm.count[warp] = (uint8_t)left;
         __syncthreads();  // also: every warp is through with its table
         const uint32_t counts = *reinterpret_cast<const uint32_t *>(sm.count);  // a byte per warp
-        const int at = __popc(kept & ((1u << lane) - 1u)) +
-                       (int)__dp4a(counts & ((1u << (8 * warp)) - 1u), 0x01010101u, 0u);
-        count = (int)__dp4a(counts, 0x01010101u, 0u);
+        at += (int)__dp4a(counts & ((1u << (8 * warp)) - 1u), 0x01010101u, 0u);
+        left = (int)__dp4a(counts, 0x01010101u, 0u);
+        if (left == count) break;  // no warp could merge anything
+        count = left;
         if (keep) {
             sm.list.l[at] = e.l;
             sm.list.r[at] = e.r;
@@ -444,8 +452,9 @@ __device__ __forceinline__ void merge_group(GroupSmem &sm, int count, Element e,
         __syncthreads();  // the tables take the list's place
     }
     const bool one_warp = count <= 32;  // what is left, and the last round's nodes: the first warp's
-    if (pend && one_warp && __popc(kept) <= slots) {
-        if (keep) pend[__popc(kept & ((1u << lane) - 1u))] = make_uint4(e.l, e.r, kPendValid | e.gaps, (uint32_t)e.tree);
+    if (pend && (one_warp ? __popc(kept) : left) <= kPendSlots) {
+        if (keep)
+            pend[at] = make_uint4(e.l, e.r, e.gaps | (at == 0 ? (uint32_t)left << kPendCount : 0u), (uint32_t)e.tree);
         return;
     }
     if (pend && threadIdx.x == 0) pend[0] = make_uint4(0u, 0u, kPendClimbed, 0u);
@@ -463,7 +472,7 @@ __device__ __forceinline__ void merge_group(GroupSmem &sm, int count, Element e,
 // The build's error flags, read once per CTA (they go to sm.failed before the
 // CTA's first barrier): if an earlier stage failed, the whole CTA returns and
 // leaves `store` untouched.
-__device__ __forceinline__ void group_start(GroupSmem &sm, const uint32_t *flags) {
+__device__ __forceinline__ void group_start(MergeSmem &sm, const uint32_t *flags) {
     if (threadIdx.x == 0) sm.failed = (__ldcg(flags) & (kFlagTimeout | kFlagCorrupt)) != 0;
 }
 
@@ -486,82 +495,70 @@ struct ManyTrees {
     }
 };
 
-// What the groups left, kGroup slots to a CTA, is merged the same way, their
-// nodes read back for their boxes; what is left of that (10 elements to
-// 1024 leaves of uniform points) is merged again or climbs with device-scope exchanges. Every
-// slot is cleared, so the slots are zero again for the next build. With a
-// thread per slot climbing from there the construct of 2^25 points took 1.29
-// ms, so 1.13; 512 batched trees of 36,000 points that climbed inside the
-// groups' kernel 1.13 ms, so 0.65.
+// What kMergeGroups groups left (then kMergeCtas CTAs of a merge) is merged the
+// same way, the nodes read back for their boxes. With a thread per element
+// climbing from there the construct of 2^25 points took 1.29 ms, so 1.13; 512
+// batched trees of 36,000 points that climbed inside the groups' kernel 1.13
+// ms, so 0.65.
+constexpr int kMergeGroups = 8;
+constexpr int kMergeCtas = 5;
 
-template <int kKind, int kSlots, bool kJitter, bool kTrees, typename OwnerOf>
+template <int kKind, int kFrom, bool kJitter, bool kTrees, typename OwnerOf>
 __global__ void __launch_bounds__(kGroup)
-    merge_pending_kernel(uint4 *pend, int64_t slots, OwnerOf owner, uint32_t *flags, uint4 *out, Jitter jt) {
-    constexpr int kMergeGroups = kGroup / kSlots;
-    __shared__ GroupSmem sm;
+    merge_pending_kernel(uint4 *pend, int64_t lists, OwnerOf owner, uint32_t *flags, uint4 *out, Jitter jt) {
+    __shared__ MergeSmem sm;
+    __shared__ uint32_t s_lists[kFrom];
     group_start(sm, flags);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t k = (int64_t)blockIdx.x * (kMergeGroups * kSlots) + threadIdx.x;
-    const bool slot = threadIdx.x < kMergeGroups * kSlots && k < slots;
-    if (out) out += (int64_t)blockIdx.x * kMergedSlots;
-    const uint4 w = slot ? pend[k] : make_uint4(0u, 0u, 0u, 0u);
-    if (w.z) pend[k] = make_uint4(0u, 0u, 0u, 0u);
-    const uint32_t valid = __ballot_sync(~0u, (w.z & kPendValid) != 0u);
-    if (lane == 0) sm.count[warp] = (uint8_t)__popc(valid);
-    Element e{w.x, w.y, w.z & 0xffffffu, make_float3(0.f, 0.f, 0.f), make_float3(0.f, 0.f, 0.f), (int)w.w};
-    bool have = (w.z & kPendValid) != 0u, missing = (w.z & kPendClimbed) != 0u;
-    if (have) {
-        const Owner o = owner(e.tree);
-        if (e.l > e.r || e.r >= (uint32_t)o.n) {
-            atomicOr(flags, kFlagCorrupt);
-            have = false;
-            missing = true;
-        } else {
-            // the node of range [l, r]: leaf l, or internal node r or l (its Karras index)
-            const uint32_t dl = e.gaps & 0xffu, dr = (e.gaps >> 8) & 0xffu;
-            const int id = (int)(e.l == e.r ? (uint32_t)(o.n - 1) + e.l : (dr < dl ? e.r : e.l));
-            load_node_box<kKind>(o.inodes, o.leaves, o.n - 1, id, e.lo, e.hi);
+    const int t = threadIdx.x;
+    if (out) out += (int64_t)blockIdx.x * kPendSlots;
+    pend += (int64_t)blockIdx.x * kFrom * kPendSlots;
+    const bool list = t < kFrom && (int64_t)blockIdx.x * kFrom + t < lists;
+    if (t < kFrom) s_lists[t] = list ? pend[t * kPendSlots].z : 0u;
+    __syncthreads();
+    // the thread's element: t, counted through the lists
+    int count = 0, from = 0, at = t;
+    bool missing = false;
+#pragma unroll
+    for (int k = 0; k < kFrom; ++k) {
+        const uint32_t z = s_lists[k];
+        const int c = (int)(z >> kPendCount) & 127;
+        missing = missing || (z & kPendClimbed) != 0u;
+        if (t >= count) {
+            from = k;
+            at = t - count;
         }
+        count += c;
     }
-    const bool climbed = __syncthreads_or(missing);
-    if (sm.failed) return;
-    if (climbed) {  // some elements are missing: those that are here climb too
-        if (out && threadIdx.x == 0) out[0] = make_uint4(0u, 0u, kPendClimbed, 0u);
-        if (!have) return;
+    const auto element = [&](const uint4 &w) {
+        Element e{w.x, w.y, w.z & 0xffffffu, make_float3(0.f, 0.f, 0.f), make_float3(0.f, 0.f, 0.f), (int)w.w};
         const Owner o = owner(e.tree);
-        climb_global<kKind, kJitter>(
-            Climb{e.l, e.r, e.gaps & 0xffu, (e.gaps >> 8) & 0xffu, (e.gaps >> 16) & 0xffu, e.lo, e.hi}, o.n, o.inodes,
-            o.leaves, o.store, flags, jt);
+        // the node of range [l, r]: leaf l, or internal node r or l (its Karras index)
+        const uint32_t dl = e.gaps & 0xffu, dr = (e.gaps >> 8) & 0xffu;
+        const int id = (int)(e.l == e.r ? (uint32_t)(o.n - 1) + e.l : (dr < dl ? e.r : e.l));
+        load_node_box<kKind>(o.inodes, o.leaves, o.n - 1, id, e.lo, e.hi);
+        return e;
+    };
+    if (sm.failed || missing || count > kGroup) {
+        // failed: only the counts are cleared; else (some elements missing, or too many) those that are here climb
+        if (out && t == 0 && !sm.failed) out[0] = make_uint4(0u, 0u, kPendClimbed, 0u);
+        for (int k = 0; k < kFrom && !sm.failed; ++k) {
+            const int c = (int)(s_lists[k] >> kPendCount) & 127;
+            if (t >= c) continue;
+            const Element e = element(pend[k * kPendSlots + t]);
+            const Owner o = owner(e.tree);
+            climb_global<kKind, kJitter>(
+                Climb{e.l, e.r, e.gaps & 0xffu, (e.gaps >> 8) & 0xffu, (e.gaps >> 16) & 0xffu, e.lo, e.hi}, o.n,
+                o.inodes, o.leaves, o.store, flags, jt);
+        }
+        __syncthreads();
+        if (list) pend[t * kPendSlots].z = 0u;
         return;
     }
-    const uint32_t counts = *reinterpret_cast<const uint32_t *>(sm.count);
-    const int at = __popc(valid & ((1u << lane) - 1u)) +
-                   (int)__dp4a(counts & ((1u << (8 * warp)) - 1u), 0x01010101u, 0u);
-    const int count = (int)__dp4a(counts, 0x01010101u, 0u);
-    if (have) {
-        sm.list.l[at] = e.l;
-        sm.list.r[at] = e.r;
-        sm.list.gaps[at] = e.gaps;
-        sm.list.box[0][at] = e.lo.x;
-        sm.list.box[1][at] = e.lo.y;
-        sm.list.box[2][at] = e.lo.z;
-        sm.list.box[3][at] = e.hi.x;
-        sm.list.box[4][at] = e.hi.y;
-        sm.list.box[5][at] = e.hi.z;
-        if (kTrees) sm.list.tree[at] = e.tree;
-    }
+    Element e{};
+    if (t < count) e = element(pend[from * kPendSlots + at]);
     __syncthreads();
-    if ((int)threadIdx.x < count) {
-        const int j = threadIdx.x;
-        e.l = sm.list.l[j];
-        e.r = sm.list.r[j];
-        e.gaps = sm.list.gaps[j];
-        e.lo = make_float3(sm.list.box[0][j], sm.list.box[1][j], sm.list.box[2][j]);
-        e.hi = make_float3(sm.list.box[3][j], sm.list.box[4][j], sm.list.box[5][j]);
-        if (kTrees) e.tree = sm.list.tree[j];
-    }
-    __syncthreads();
-    merge_group<kKind, false, kJitter, kTrees>(sm, count, e, owner, flags, out, kMergedSlots, jt);
+    if (list) pend[t * kPendSlots].z = 0u;
+    merge_group<kKind, false, kJitter, kTrees>(sm, count, e, owner, flags, out, jt);
 }
 
 // delta* at the CTA's positions, from sm.code. Thread t holds leaf i of a
@@ -619,7 +616,7 @@ __global__ void __launch_bounds__(kGroup, kGroupCtas)
     if (ok) leaf_write<kKind>(i, n, p_id, e.lo, e.hi, leaves, (e.gaps >> 8) & 0xffu, e.gaps >> 16);
     merge_group<kKind, kKind == LBVH_PRIM_POINTS, kJitter, false>(
         sm, (int)min((int64_t)kGroup, n - a), e, OneTree{Owner{n, inodes, leaves, store}}, flags,
-        pend ? pend + (int64_t)blockIdx.x * kPendSlots : nullptr, kPendSlots, jt);
+        pend ? pend + (int64_t)blockIdx.x * kPendSlots : nullptr, jt);
 }
 
 // Algorithm 4 after a sort that kept only the permutation. Each thread
@@ -678,7 +675,7 @@ __global__ void __launch_bounds__(kGroup, kGroupCtas)
     if (ok) leaf_write<kKind>(i, n, p_id, e.lo, e.hi, leaves, (e.gaps >> 8) & 0xffu, e.gaps >> 16);
     merge_group<kKind, kKind == LBVH_PRIM_POINTS, kJitter, false>(
         sm, (int)min((int64_t)kGroup, n - a), e, OneTree{Owner{n, inodes, leaves, store}}, flags,
-        pend ? pend + (int64_t)blockIdx.x * kPendSlots : nullptr, kPendSlots, jt);
+        pend ? pend + (int64_t)blockIdx.x * kPendSlots : nullptr, jt);
 }
 
 // Many trees at once, grouped by global sorted position.
@@ -721,26 +718,23 @@ __global__ void __launch_bounds__(kGroup, kGroupCtas)
     e.gaps = leaf_gaps(sm);
     if (ok) leaf_write<kKind>(i, o.n, p_own, e.lo, e.hi, o.leaves, (e.gaps >> 8) & 0xffu, e.gaps >> 16);
     merge_group<kKind, kKind == LBVH_PRIM_POINTS, false, true>(sm, (int)min((int64_t)kGroup, total - a), e, owner, flags,
-                                                               pend + (int64_t)blockIdx.x * kPendSlots, kPendSlots,
-                                                               Jitter{});
+                                                               pend + (int64_t)blockIdx.x * kPendSlots, Jitter{});
 }
 
 // How far the merges go before the rest climbs. A merge is a launch of about
 // 6 us that its CTAs' own latency sets, a climb 1-2 us per level of the tree;
-// but an element list longer than its slots, which long lists near the root
-// of a large tree often are, makes every merge above it climb too. Points,
-// 63-bit codes, us, merging to the end / while there are over 4096 CTAs:
-// 20,000 20.4 / 28.6, 100,000 28.6 / 34.8, 300,000 38.8 / 40.9, 1.0M 65.4 /
-// 63.4, 2^23 379 / 307, 2^25 1217 / 1126 (never merging twice: 2^23 334,
-// 2^25 1268; while over 64: 2^23 321, 2^25 1139).
-constexpr int64_t kMergeToEnd = 512;
+// but where a list is too long, every merge above it waits for its own climbs
+// in turn (64 clusters with points down to 1e-5 of their size, 33,000: 276 us
+// merging to the end, 178 without; 1.0M 309, 108). So only small builds merge
+// to the end: 16,500 points, clustered or not, 24.5 us against 29.6 to 36.8.
+// Merging again while there are over 4096 CTAs (2^25 points): 1.14 ms, never
+// 1.27, to the end (mixture) 1.48.
+constexpr int64_t kMergeToEnd = 24;
 constexpr int64_t kMergeAgain = 4096;
 
-// The merges above the groups: kPendSlots slots from each group, kMergedSlots
-// from each CTA of a merge, one region after the other in `pend`.
-int64_t merge_ctas(int64_t from, bool groups) {
-    const int64_t each = groups ? kGroup / kPendSlots : kGroup / kMergedSlots;
-    return (from + each - 1) / each;
+int64_t merge_ctas(int64_t lists, bool groups) {
+    const int64_t each = groups ? kMergeGroups : kMergeCtas;
+    return (lists + each - 1) / each;
 }
 
 template <bool kTrees, typename OwnerOf>
@@ -753,21 +747,21 @@ void launch_merges(int64_t groups, int kind, const OwnerOf &owner, uint32_t *fla
     if (jt.max_ns) enough = groups;  // the hook is for climbs: what the first merge leaves climbs
     const bool pts = kind == LBVH_PRIM_POINTS;
     for (bool first = true;; first = false) {
-        const int64_t slots = from * (first ? kPendSlots : kMergedSlots), ctas = merge_ctas(from, first);
-        uint4 *out = ctas > enough ? in + slots : nullptr;
+        const int64_t ctas = merge_ctas(from, first);
+        uint4 *out = ctas > enough ? in + from * kPendSlots : nullptr;
         const auto pick = [&](auto a, auto b, auto c, auto d) { return first ? (pts ? a : b) : (pts ? c : d); };
-        auto k = pick(merge_pending_kernel<LBVH_PRIM_POINTS, kPendSlots, false, kTrees, OwnerOf>,
-                      merge_pending_kernel<LBVH_PRIM_BOXES, kPendSlots, false, kTrees, OwnerOf>,
-                      merge_pending_kernel<LBVH_PRIM_POINTS, kMergedSlots, false, kTrees, OwnerOf>,
-                      merge_pending_kernel<LBVH_PRIM_BOXES, kMergedSlots, false, kTrees, OwnerOf>);
+        auto k = pick(merge_pending_kernel<LBVH_PRIM_POINTS, kMergeGroups, false, kTrees, OwnerOf>,
+                      merge_pending_kernel<LBVH_PRIM_BOXES, kMergeGroups, false, kTrees, OwnerOf>,
+                      merge_pending_kernel<LBVH_PRIM_POINTS, kMergeCtas, false, kTrees, OwnerOf>,
+                      merge_pending_kernel<LBVH_PRIM_BOXES, kMergeCtas, false, kTrees, OwnerOf>);
         if constexpr (!kTrees) {
             if (jt.max_ns)
-                k = pick(merge_pending_kernel<LBVH_PRIM_POINTS, kPendSlots, true, kTrees, OwnerOf>,
-                         merge_pending_kernel<LBVH_PRIM_BOXES, kPendSlots, true, kTrees, OwnerOf>,
-                         merge_pending_kernel<LBVH_PRIM_POINTS, kMergedSlots, true, kTrees, OwnerOf>,
-                         merge_pending_kernel<LBVH_PRIM_BOXES, kMergedSlots, true, kTrees, OwnerOf>);
+                k = pick(merge_pending_kernel<LBVH_PRIM_POINTS, kMergeGroups, true, kTrees, OwnerOf>,
+                         merge_pending_kernel<LBVH_PRIM_BOXES, kMergeGroups, true, kTrees, OwnerOf>,
+                         merge_pending_kernel<LBVH_PRIM_POINTS, kMergeCtas, true, kTrees, OwnerOf>,
+                         merge_pending_kernel<LBVH_PRIM_BOXES, kMergeCtas, true, kTrees, OwnerOf>);
         }
-        k<<<(unsigned)ctas, kGroup, 0, s>>>(in, slots, owner, flags, out, jt);
+        k<<<(unsigned)ctas, kGroup, 0, s>>>(in, from, owner, flags, out, jt);
         count_launches(1);
         if (!out) return;
         in = out;
@@ -781,7 +775,7 @@ size_t construct_pend_bytes(int64_t n) {
     int64_t from = (n + kGroup - 1) / kGroup, slots = from * kPendSlots;
     for (bool first = true; from > 1; first = false) {
         from = merge_ctas(from, first);
-        slots += from * kMergedSlots;
+        slots += from * kPendSlots;
     }
     return (size_t)slots * sizeof(uint4);
 }

@@ -399,7 +399,10 @@ void launch_batch_pack(const float4 *nodes, int kind, const BatchTables &bt, flo
 //   2^15 449 / 86 / 295; mixture boxes 2^22 1708 / 7855 / 2324, 2^21 1303 /
 //   3952 / 1299; 2^20 1068 / 2003 / 834; 2^18 731 / 545 / 452.
 //   As many queries as points, in the points' own order: 16384 48 / 32 / 68,
-//   65536 53 / 76 / 80; in another: 2^16 113 / 76 / 139.
+//   65536 53 / 76 / 80; in another: 2^16 113 / 76 / 139. Boxes for boxes, in
+//   their own order: 70,000 121 / 109 / 109, 170,000 150 / 195 / 183; in
+//   another: 119,230 for 310,000 215 / 201 / 216, 130,769 for 170,000 209 /
+//   211 / 216.
 // So packets need a query for at least every fourth leaf (fewer lie too far
 // apart to share nodes) and enough packets to fill the GPU; below about 1000
 // queries per SM the 8 lanes have the shorter chain of loads, and need no
@@ -413,7 +416,8 @@ void launch_batch_pack(const float4 *nodes, int kind, const BatchTables &bt, flo
 RangeWalk range_walk(int qkind, int64_t nq, int64_t n, bool sorted) {
     if (qkind == LBVH_Q_RAY) return nq <= 640 * (int64_t)device_sm_count() ? kRangeSparse : kRangeNodes;
     const bool dense = n <= 4 * nq;
-    const int64_t few = (dense ? (sorted ? 256 : 640) : 1024) * (int64_t)device_sm_count();
+    const bool boxes = qkind == LBVH_Q_BOX;
+    const int64_t few = (dense ? (sorted ? (boxes ? 512 : 256) : (boxes ? 800 : 640)) : 1024) * (int64_t)device_sm_count();
     if (nq <= few) return kRangeSparse;
     return dense ? kRangePackets : kRangeNodes;
 }

@@ -58,7 +58,7 @@ def chain(before, after, seed):
 
 
 @pytest.mark.parametrize("kind", ["points", "boxes"])
-@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 127, 128, 129, 1023, 1025, 5119, 5121, 131073, 524288, 524289, 4500001])
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 127, 128, 129, 1023, 1025, 5119, 5121, 24576, 24577, 131073, 4194304, 4194305])
 def test_group_edges(n, kind):
     lbvh = L()
     pts = inputs.uniform_points(n, seed=n)
