@@ -515,20 +515,23 @@ __global__ void __launch_bounds__(kGroup)
     const bool list = t < kFrom && (int64_t)blockIdx.x * kFrom + t < lists;
     if (t < kFrom) s_lists[t] = list ? pend[t * kPendSlots].z : 0u;
     __syncthreads();
-    // the thread's element: t, counted through the lists
-    int count = 0, from = 0, at = t;
+    int count = 0;
     bool missing = false;
 #pragma unroll
     for (int k = 0; k < kFrom; ++k) {
-        const uint32_t z = s_lists[k];
-        const int c = (int)(z >> kPendCount) & 127;
-        missing = missing || (z & kPendClimbed) != 0u;
-        if (t >= count) {
-            from = k;
-            at = t - count;
-        }
-        count += c;
+        count += (int)(s_lists[k] >> kPendCount) & 127;
+        missing = missing || (s_lists[k] & kPendClimbed) != 0u;
     }
+    // the j-th element, counted through the lists
+    const auto place = [&](int j) {
+        int before = 0, at = j;
+#pragma unroll
+        for (int k = 0; k < kFrom; ++k) {
+            if (j >= before) at = k * kPendSlots + j - before;
+            before += (int)(s_lists[k] >> kPendCount) & 127;
+        }
+        return at;
+    };
     const auto element = [&](const uint4 &w) {
         Element e{w.x, w.y, w.z & 0xffffffu, make_float3(0.f, 0.f, 0.f), make_float3(0.f, 0.f, 0.f), (int)w.w};
         const Owner o = owner(e.tree);
@@ -541,10 +544,8 @@ __global__ void __launch_bounds__(kGroup)
     if (sm.failed || missing || count > kGroup) {
         // failed: only the counts are cleared; else (some elements missing, or too many) those that are here climb
         if (out && t == 0 && !sm.failed) out[0] = make_uint4(0u, 0u, kPendClimbed, 0u);
-        for (int k = 0; k < kFrom && !sm.failed; ++k) {
-            const int c = (int)(s_lists[k] >> kPendCount) & 127;
-            if (t >= c) continue;
-            const Element e = element(pend[k * kPendSlots + t]);
+        for (int k = t; k < count && !sm.failed; k += kGroup) {
+            const Element e = element(pend[place(k)]);
             const Owner o = owner(e.tree);
             climb_global<kKind, kJitter>(
                 Climb{e.l, e.r, e.gaps & 0xffu, (e.gaps >> 8) & 0xffu, (e.gaps >> 16) & 0xffu, e.lo, e.hi}, o.n,
@@ -555,7 +556,7 @@ __global__ void __launch_bounds__(kGroup)
         return;
     }
     Element e{};
-    if (t < count) e = element(pend[from * kPendSlots + at]);
+    if (t < count) e = element(pend[place(t)]);
     __syncthreads();
     if (list) pend[t * kPendSlots].z = 0u;
     merge_group<kKind, false, kJitter, kTrees>(sm, count, e, owner, flags, out, jt);
@@ -724,9 +725,10 @@ __global__ void __launch_bounds__(kGroup, kGroupCtas)
 // How far the merges go before the rest climbs. A merge is a launch of about
 // 6 us that its CTAs' own latency sets, a climb 1-2 us per level of the tree;
 // but where a list is too long, every merge above it waits for its own climbs
-// in turn (64 clusters with points down to 1e-5 of their size, 33,000: 276 us
-// merging to the end, 178 without; 1.0M 309, 108). So only small builds merge
-// to the end: 16,500 points, clustered or not, 24.5 us against 29.6 to 36.8.
+// in turn (64 clusters with points down to 1e-5 of their size, 33,000: 180 us
+// merging to the end, 94 without; 300,000 154, 86). So only small builds merge
+// to the end: 16,500 points, clustered or not, 24.5 us against 29.6 to 36.8
+// (100,000 32.7 against 35 to 43).
 // Merging again while there are over 4096 CTAs (2^25 points): 1.14 ms, never
 // 1.27, to the end (mixture) 1.48.
 constexpr int64_t kMergeToEnd = 24;
