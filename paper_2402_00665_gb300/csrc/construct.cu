@@ -499,7 +499,7 @@ struct ManyTrees {
 // same way, the nodes read back for their boxes. With a thread per element
 // climbing from there the construct of 2^25 points took 1.29 ms, so 1.13; 512
 // batched trees of 36,000 points that climbed inside the groups' kernel 1.13
-// ms, so 0.65.
+// ms, so 0.60.
 constexpr int kMergeGroups = 8;
 constexpr int kMergeCtas = 5;
 
