@@ -157,6 +157,10 @@ __global__ void __launch_bounds__(kThreads)
 // walked in packets).
 __device__ const HilbertTable kHilbert = hilbert_table();
 
+__device__ __forceinline__ void load_hilbert(uint16_t *s) {
+    for (int k = threadIdx.x; k < kHilbertEntries; k += kThreads) s[k] = kHilbert.next[k];
+}
+
 template <int kKind, int kLayout>
 __global__ void __launch_bounds__(kThreads)
     encode_kernel(const float *__restrict__ prims, int64_t n, int b, const float *__restrict__ bounds,
@@ -165,8 +169,8 @@ __global__ void __launch_bounds__(kThreads)
     for (int k = threadIdx.x; k < passes * kRadix; k += kThreads) s_hist[k] = 0;
     const Grid3 g = make_grid(bounds, b);
     const int hist_shift = kLayout == kCodeTop ? kRadixBits * top_first_byte(ib, skip) : 0;
-    __shared__ uint32_t s_hilbert[kLayout == kCodeHilbert ? kHilbertStates * 8 : 1];
-    if (kLayout == kCodeHilbert && threadIdx.x < kHilbertStates * 8) s_hilbert[threadIdx.x] = kHilbert.next[threadIdx.x];
+    __shared__ uint16_t s_hilbert[kLayout == kCodeHilbert ? kHilbertEntries : 1];
+    if (kLayout == kCodeHilbert) load_hilbert(s_hilbert);
     __syncthreads();
     for_each_centroid<kKind>(prims, n, [&](int64_t i, float x, float y, float z) {
         const uint64_t c = kLayout == kCodeHilbert ? hilbert(x, y, z, g, b, s_hilbert) >> ib : morton(x, y, z, g);
@@ -192,9 +196,10 @@ __global__ void __launch_bounds__(kThreads)
 __global__ void __launch_bounds__(kThreads)
     encode_rays_kernel(const float4 *__restrict__ rays, int64_t n, const float *__restrict__ bounds,
                        uint64_t *__restrict__ words, uint32_t *__restrict__ hist) {
-    __shared__ uint32_t s_hist[kRadix], s_hilbert[kHilbertStates * 8];
+    __shared__ uint32_t s_hist[kRadix];
+    __shared__ uint16_t s_hilbert[kHilbertEntries];
     s_hist[threadIdx.x] = 0;  // kThreads == kRadix
-    if (threadIdx.x < kHilbertStates * 8) s_hilbert[threadIdx.x] = kHilbert.next[threadIdx.x];
+    load_hilbert(s_hilbert);
     const Grid3 g = make_grid(bounds, 3);
     const float extent = fmaxf(g.extent[0], fmaxf(g.extent[1], g.extent[2]));
     __syncthreads();
@@ -321,8 +326,8 @@ __global__ void __launch_bounds__(kThreads)
     s_hist[threadIdx.x] = 0;  // kThreads == kRadix
     const BatchChunk c = chunks[blockIdx.x];
     const Grid3 g = make_grid(bounds + 6 * (int64_t)c.inst, b);
-    __shared__ uint32_t s_hilbert[kCurve ? kHilbertStates * 8 : 1];
-    if (kCurve && threadIdx.x < kHilbertStates * 8) s_hilbert[threadIdx.x] = kHilbert.next[threadIdx.x];
+    __shared__ uint16_t s_hilbert[kCurve ? kHilbertEntries : 1];
+    if (kCurve) load_hilbert(s_hilbert);
     __syncthreads();
     for (int64_t i = c.begin + threadIdx.x; i < c.end; i += kThreads) {
         float x, y, z;

