@@ -164,12 +164,16 @@ __device__ __forceinline__ uint32_t test32(const PacketSmem<kP> &sm, int base, c
 }
 
 // A box: q.lo <= hi and lo <= q.hi on every axis, as the signs of hi - q.lo
-// and q.hi - lo (exact under rounding), two candidates per instruction; one
-// sign bit set is a miss.
+// and q.hi - lo, two candidates per instruction; one sign bit set is a miss.
+// Rounding keeps the sign of a difference, and equal values give +0, except
+// zeros: (-0) - (+0) is -0. So the query's bounds come in as 0 - q.lo and
+// q.hi + 0, which are +0 for either zero (2^24 box queries on 2^25 boxes, build
+// and query: 10.73 ms with the bounds as they are, 10.49 with these).
 template <int kP>
 __device__ __forceinline__ uint32_t test32(const PacketSmem<kP> &sm, int base, const Box &q) {
     constexpr int kHi = kP == LBVH_PRIM_POINTS ? 0 : 3;
-    const float ql[3] = {q.lo.x, q.lo.y, q.lo.z}, qh[3] = {q.hi.x, q.hi.y, q.hi.z};
+    const float minus_lo[3] = {__fsub_rn(0.0f, q.lo.x), __fsub_rn(0.0f, q.lo.y), __fsub_rn(0.0f, q.lo.z)};
+    const float plus_hi[3] = {__fadd_rn(q.hi.x, 0.0f), __fadd_rn(q.hi.y, 0.0f), __fadd_rn(q.hi.z, 0.0f)};
     const uint64_t neg = pack2(-1.0f, -1.0f);
     uint32_t miss = 0;
 #pragma unroll
@@ -179,7 +183,7 @@ __device__ __forceinline__ uint32_t test32(const PacketSmem<kP> &sm, int base, c
         for (int d = 0; d < 3; ++d) {
             const ulonglong2 lo = *reinterpret_cast<const ulonglong2 *>(&sm.cand[d][base + j]);
             const ulonglong2 hi = kHi ? *reinterpret_cast<const ulonglong2 *>(&sm.cand[kHi + d][base + j]) : lo;
-            const uint64_t nl = pack2(-ql[d], -ql[d]), h = pack2(qh[d], qh[d]);
+            const uint64_t nl = pack2(minus_lo[d], minus_lo[d]), h = pack2(plus_hi[d], plus_hi[d]);
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 float a, b, c, e;
