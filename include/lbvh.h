@@ -518,6 +518,12 @@ lbvh_status lbvh_construct_static(const uint64_t *d_sorted_codes, const uint32_t
  * after the hook is cleared is correct again. Nothing faults, traps or hangs. */
 lbvh_status lbvh_test_hold_sort_tile(int64_t tile);
 
+/* The same for the scan of a query's hit counts (tiles of 4096 queries, up to
+ * two per SM in one kernel): tile `tile` publishes nothing, the later tiles'
+ * waits run out, the query or batch reports LBVH_ERR_TIMEOUT and no hit is
+ * written. */
+lbvh_status lbvh_test_hold_scan_tile(int64_t tile);
+
 /* Test hook for the order of arrivals in Algorithm 4, off by default
  * (max_ns = 0). While set, every thread of the bottom-up construct waits a
  * pseudo-random time of up to max_ns nanoseconds (drawn from `seed`, the

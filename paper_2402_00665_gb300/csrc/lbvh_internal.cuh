@@ -391,6 +391,9 @@ int64_t scan_tile_count(int64_t nq);
 void launch_offsets_add(int64_t *offsets, int64_t n, int64_t base, cudaStream_t s);
 void launch_exclusive_scan(const uint32_t *counts, int64_t nq, int64_t *offsets,
                            int64_t *tile_sums, Control *ctl, cudaStream_t s);
+// Test hook (lbvh_test_hold_scan_tile): tile `tile` of the one-kernel scan
+// publishes nothing, so later tiles' bounded look-back waits run out; -1: off.
+void scan_set_hold_tile(int64_t tile);
 // Short lists from the scratch buffer to their CSR positions.
 void launch_query_copy(const QueryArgs &q, const QueryScratch &qs, const int64_t *offsets,
                        uint32_t *hits, Control *ctl, cudaStream_t s);
@@ -504,6 +507,7 @@ void launch_batch_collect_left(const float4 *nodes, int kind, const BatchTables 
                                const QueryScratch &qs, Control *ctl, cudaStream_t s);
 // Copy with the capacity check on the device (no host round trip): lists are
 // written only if ctl->total <= capacity; otherwise kFlagCapacity is latched.
+// Nothing is written either once the scan has given up (kFlagTimeout).
 void launch_query_copy_checked(const QueryArgs &q, const QueryScratch &qs, const int64_t *offsets,
                                uint32_t *hits, unsigned long long capacity, Control *ctl, cudaStream_t s);
 

@@ -50,6 +50,7 @@
 //             then sorts every such list, one warp per list (one CTA per list
 //             above 1024 hits).
 #include <algorithm>
+#include <atomic>
 #include <cstdlib>
 #include <type_traits>
 
@@ -355,6 +356,13 @@ __device__ __forceinline__ void sort_short_lists(const uint4 *src, uint32_t c, u
         if (j < (int)c) flat[at + j] = v[j];
 }
 
+// The offsets can be followed and the lists fit the caller's buffer. After a
+// wait of the scan has run out, offsets of later tiles and the total are too
+// small while earlier ones are not: nothing may be written by them.
+__device__ __forceinline__ bool lists_fit(const Control *ctl, unsigned long long capacity) {
+    return ctl->total <= capacity && (ctl->query_flags & kFlagTimeout) == 0;
+}
+
 // Thread q sorts query q's list in registers if it has at most 32 hits; the
 // lists of a warp are adjacent in the CSR, so without a longer one among them
 // they go through shared memory as one run and out 32 words per step (2^25
@@ -369,8 +377,8 @@ __global__ void __launch_bounds__(kThreads, 5)
                 const uint32_t *__restrict__ slots, uint32_t *__restrict__ hits,
                 unsigned long long capacity, Control *ctl) {
     __shared__ uint32_t s_lists[kThreads / 32][32][kRegSort + 1];
-    if (ctl->total > capacity) {  // the caller's buffer is too small: write nothing
-        if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&ctl->query_flags, kFlagCapacity);
+    if (!lists_fit(ctl, capacity)) {  // write nothing
+        if (blockIdx.x == 0 && threadIdx.x == 0 && ctl->total > capacity) atomicOr(&ctl->query_flags, kFlagCapacity);
         return;
     }
     const int64_t q = (int64_t)blockIdx.x * kThreads + threadIdx.x;
@@ -531,7 +539,7 @@ __device__ __forceinline__ int64_t scan_look_back(const unsigned long long *stat
 
 __global__ void __launch_bounds__(kScanThreads)
     scan_kernel(const uint32_t *__restrict__ counts, int64_t nq, unsigned long long *state, int64_t *__restrict__ offsets,
-                Control *ctl) {
+                Control *ctl, int64_t hold_tile) {
     constexpr int kRow = kScanItems + 1;
     __shared__ int64_t s_warp[kScanThreads / 32];
     __shared__ int64_t s_o[kScanThreads * kRow];  // the offsets; first the counts (the scan's barriers
@@ -563,11 +571,12 @@ __global__ void __launch_bounds__(kScanThreads)
     int64_t total;
     int64_t run = block_scan_exclusive(sum, s_warp, total);
     if (threadIdx.x < 32) {
-        if (!alone && threadIdx.x == 0)
+        const bool publish = !alone && threadIdx.x == 0 && tile != hold_tile;
+        if (publish)
             set_scan_word(state + tile, (tile == 0 ? kScanPrefix : kScanSum) | (unsigned long long)total);
         const int64_t before = tile == 0 ? 0 : scan_look_back(state, tile, ctl);
         if (threadIdx.x == 0) {
-            if (tile > 0) set_scan_word(state + tile, kScanPrefix | (unsigned long long)(before + total));
+            if (publish && tile > 0) set_scan_word(state + tile, kScanPrefix | (unsigned long long)(before + total));
             s_before = before;
             if (base + kScanTile >= nq) {  // the last tile
                 offsets[nq] = before + total;
@@ -745,7 +754,7 @@ __global__ void __launch_bounds__(kThreads)
                            const uint32_t *__restrict__ list, uint32_t *__restrict__ big_list, Control *ctl,
                            unsigned long long capacity) {
     __shared__ uint32_t s[kSortWarps][kWarpSortMax];
-    if (ctl->total > capacity) return;
+    if (!lists_fit(ctl, capacity)) return;
     const uint32_t count = ctl->overflow_filled;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t *a = s[warp];
@@ -771,7 +780,7 @@ __global__ void __launch_bounds__(kFixThreads)
                           const uint32_t *__restrict__ big_list, const Control *ctl,
                           unsigned long long capacity) {
     __shared__ uint32_t s[kFixSmem];
-    if (ctl->total > capacity) return;
+    if (!lists_fit(ctl, capacity)) return;
     const uint32_t count = ctl->overflow_big;
     for (uint32_t j = blockIdx.x; j < count; j += gridDim.x) {
         const uint32_t q = big_list[j];
@@ -796,7 +805,7 @@ __global__ void __launch_bounds__(kFixThreads)
 __global__ void __launch_bounds__(kThreads)
     spill_gather_kernel(QueryScratch qs, const int64_t *__restrict__ offsets, uint32_t *__restrict__ hits,
                         const Control *ctl, unsigned long long capacity) {
-    if (ctl->total > capacity) return;
+    if (!lists_fit(ctl, capacity)) return;
     const uint32_t count = ctl->overflow_filled;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int kWarps = kThreads / 32;
@@ -863,7 +872,7 @@ __global__ void __launch_bounds__(kThreads)
                           const uint32_t *__restrict__ list, const Control *ctl,
                           const int64_t *__restrict__ offsets, uint32_t *__restrict__ hits,
                           unsigned long long capacity) {
-    if (ctl->total > capacity) return;  // nothing is written into a buffer that is too small
+    if (!lists_fit(ctl, capacity)) return;
     const uint32_t count = ctl->overflow_filled;
     for (int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x; j < count; j += (int64_t)gridDim.x * kThreads) {
         const uint32_t e = list[j];
@@ -1073,13 +1082,19 @@ void launch_offsets_add(int64_t *offsets, int64_t n, int64_t base, cudaStream_t 
     count_launches(1);
 }
 
+// Test hook (lbvh_test_hold_scan_tile): the tile that publishes nothing.
+static std::atomic<int64_t> g_hold_scan_tile{-1};
+
+void scan_set_hold_tile(int64_t tile) { g_hold_scan_tile.store(tile, std::memory_order_relaxed); }
+
 void launch_exclusive_scan(const uint32_t *counts, int64_t nq, int64_t *offsets,
                            int64_t *tile_sums, Control *ctl, cudaStream_t s) {
     const int64_t tiles = nq > 0 ? scan_tile_count(nq) : 1;
     if (tiles <= kScanOnePass * (int64_t)device_sm_count()) {
         if (tiles > 1) cudaMemsetAsync(tile_sums, 0, (size_t)tiles * 8, s);
         scan_kernel<<<(unsigned)tiles, kScanThreads, 0, s>>>(counts, nq, reinterpret_cast<unsigned long long *>(tile_sums),
-                                                             offsets, ctl);
+                                                             offsets, ctl,
+                                                             g_hold_scan_tile.load(std::memory_order_relaxed));
         count_launches(1);
         return;
     }
