@@ -8,6 +8,7 @@
 // beside codes wider than 30 bits) and the warps' digit counts fill 177 KB.
 #include "lbvh_internal.cuh"
 #include "morton.cuh"
+#include "once_per_device.cuh"
 
 namespace lbvh {
 
@@ -165,11 +166,13 @@ template <int kKind, bool kWide, int kT, int kR>
 void launch(const float *prims, int n, int bits, float *bounds, uint32_t *perm, uint32_t *flags, cudaStream_t s) {
     Kernel k = small_sort_kernel<kKind, kWide, kT, kR>;
     constexpr size_t smem = sizeof(SmallSmem<kWide, kT, kR>);
-    static const bool configured = [] {
-        Kernel f = small_sort_kernel<kKind, kWide, kT, kR>;
-        return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
-    }();
-    (void)configured;
+    static OncePerDevice configured;
+    int dev = 0;
+    // a failure stays the thread's last error, which the caller's launch check reports
+    if (cudaGetDevice(&dev) != cudaSuccess || !configured(dev, [k] {
+            return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
+        }))
+        return;
     k<<<1, kT, smem, s>>>(prims, n, bits, bounds, perm, flags);
 }
 

@@ -38,6 +38,7 @@
 #include <atomic>
 
 #include "lbvh_internal.cuh"
+#include "once_per_device.cuh"
 
 namespace lbvh {
 
@@ -485,19 +486,6 @@ const Variant *variant_table(int *count) {
         make_variant<12, 4, false>(),
         make_variant<16, 3, false>(),
     };
-    // kernel attributes set once, thread-safely (function-local static initialisation)
-    static const bool configured = [] {
-        for (const Variant &v : table)
-            for (int sg = 0; sg < 2; ++sg)
-                for (int kind = 0; kind < kPassKinds; ++kind) {
-                    if (!v.k[sg][kind]) continue;
-                    cudaFuncSetAttribute(v.k[sg][kind], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)pass_smem(v, kind));
-                    cudaFuncSetAttribute(v.k[sg][kind], cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-                }
-        return true;
-    }();
-    (void)configured;
     *count = (int)(sizeof table / sizeof table[0]);
     return table;
 }
@@ -506,6 +494,29 @@ const Variant &variant(int idx = -1) {
     int count = 0;
     const Variant *table = variant_table(&count);
     return table[(idx >= 0 && idx < count) ? idx : 0];
+}
+
+bool allow_smem(PassKernel k, size_t bytes) {
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess &&
+           cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100) == cudaSuccess;
+}
+
+// The kernels' attributes on the current device. A failure stays the thread's
+// last error, which the callers' launch checks report.
+bool variants_configured() {
+    static OncePerDevice configured;
+    int dev = 0;
+    return cudaGetDevice(&dev) == cudaSuccess && configured(dev, [] {
+               int count = 0;
+               const Variant *table = variant_table(&count);
+               for (int v = 0; v < count; ++v)
+                   for (int sg = 0; sg < 2; ++sg)
+                       for (int kind = 0; kind < kPassKinds; ++kind) {
+                           const PassKernel k = table[v].k[sg][kind];
+                           if (k && !allow_smem(k, pass_smem(table[v], kind))) return false;
+                       }
+               return true;
+           });
 }
 
 // count (nullable): only the first *count keys (read on the device) are counted.
@@ -591,7 +602,7 @@ struct Pass {
 void run_pass_list(const Variant &v, const Pass *ps, int passes, int64_t n, const SortScratch &scratch,
                    Control *ctl, cudaStream_t s, cudaEvent_t (*pass_events)[2], const SortSegments *seg) {
     const int64_t tiles = seg ? seg->tiles : (n + (int64_t)kSortThreads * v.items - 1) / ((int64_t)kSortThreads * v.items);
-    if (tiles <= 0) return;
+    if (tiles <= 0 || !variants_configured()) return;
     const SegArgs sa{seg ? seg->off : nullptr, seg ? seg->tile_first : nullptr, seg ? seg->count : 0};
     const int64_t hist_stride = (int64_t)kRadix * (seg ? seg->count : 1);
     cudaMemsetAsync(scratch.lookback, 0, (size_t)tiles * kRadix * sizeof(uint32_t), s);
@@ -690,10 +701,6 @@ const CountedKernels &counted_kernels() {
         k.lo = onesweep_counted_kernel<kInKV, kOutKV, false, kCountedItems, kCountedBlocks, true>;
         k.hi = onesweep_counted_kernel<kInKV, kOutKV, true, kCountedItems, kCountedBlocks, true>;
         k.smem = sizeof(SortSmem<kCountedItems, true, true>);
-        for (PassKernel f : {k.lo, k.hi}) {
-            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
-            cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        }
         return k;
     }();
     return c;
@@ -706,6 +713,11 @@ bool run_counted_sort(uint64_t *keys_a, uint32_t *vals_a, uint64_t *keys_b, uint
                       cudaStream_t s) {
     if (n_max <= 0) return false;
     const CountedKernels &k = counted_kernels();
+    static OncePerDevice configured;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        !configured(dev, [&k] { return allow_smem(k.lo, k.smem) && allow_smem(k.hi, k.smem); }))
+        return false;
     const int passes = sort_passes(key_bits);
     const int64_t tile = (int64_t)kSortThreads * kCountedItems;
     const int64_t tiles_max = (n_max + tile - 1) / tile;
