@@ -197,7 +197,8 @@ struct lbvh_tree_s {
     cudaStream_t xfer = nullptr;
     cudaEvent_t staged[2] = {nullptr, nullptr}, drained[2] = {nullptr, nullptr}, xfer_done = nullptr;
     const float *prims_ptr = nullptr;      // the last build's input (self-queries)
-    int64_t spill_nq = 0;                  // query count the spill pool was sized for
+    uint32_t spill_chunks = 0;             // chunks of the spill pool,
+    uint32_t spill_want = 0;               // and how many a query that ran out of them asks for
     lbvh::Control *h_ctl = nullptr;  // pinned mirror of the control block (from pinned_controls())
     Profiler prof;
 
@@ -398,7 +399,7 @@ lbvh_status query_order(lbvh_tree_t t, lbvh::QueryArgs &qa, cudaStream_t s, int 
 lbvh::QueryScratch query_scratch(lbvh_tree_t t) {
     return lbvh::QueryScratch{t->counts.as<uint32_t>(), t->slots.as<uint32_t>(), t->overflow.as<uint32_t>(),
                               t->spill_head.as<uint32_t>(), t->spill.as<uint32_t>(),
-                              lbvh::spill_chunks_for(t->spill_nq), t->sparse.as<uint2>()};
+                              t->spill_chunks, t->sparse.as<uint2>()};
 }
 
 // The query up to the hit count: order, collecting walk, scan; synchronises `s`.
@@ -410,9 +411,10 @@ lbvh_status query_count(lbvh_tree_t t, lbvh::QueryArgs &qa, int64_t *d_offsets,
     LBVH_CUDA(t->counts.ensure(unq * 4 + 4, s));
     LBVH_CUDA(t->overflow.ensure(unq * 4 + 4, s));
     LBVH_CUDA(t->spill_head.ensure(unq * 4 + 4, s));
-    if (spill_chunks_for(qa.nq) > spill_chunks_for(t->spill_nq) || !t->spill.p) {
-        LBVH_CUDA(t->spill.ensure((size_t)spill_chunks_for(qa.nq) * kSpillChunkWords * 4, s));
-        t->spill_nq = qa.nq;
+    const uint32_t chunks = std::max(spill_chunks_for(qa.nq), t->spill_want);
+    if (chunks > t->spill_chunks || !t->spill.p) {
+        LBVH_CUDA(t->spill.ensure((size_t)chunks * kSpillChunkWords * 4, s));
+        t->spill_chunks = chunks;
     }
     LBVH_CUDA(t->tile_sums.ensure((size_t)scan_tile_count(qa.nq) * 8 + 8, s));
     LBVH_CUDA(t->slots.ensure(unq * kQueryBufferHits * 4 + 16, s));
@@ -463,6 +465,7 @@ lbvh_status query_count(lbvh_tree_t t, lbvh::QueryArgs &qa, int64_t *d_offsets,
     lbvh_status st = read_control(t, s);
     if (st != LBVH_OK) return st;
     if (pack) t->packed_ok = true;  // complete: the stream has been synchronised
+    t->spill_want = std::max(t->spill_want, spill_chunks_after(t->h_ctl->spill_used, t->spill_chunks));
     st = flags_status(t->h_ctl->build_flags);
     if (st == LBVH_OK) st = flags_status(t->h_ctl->query_flags);
     *total = t->h_ctl->total;
@@ -1766,7 +1769,7 @@ void tree_release_query_scratch(lbvh_tree_t t, cudaStream_t s) {
                       &t->qvals[0], &t->qvals[1], &t->qlookback, &t->spill_head, &t->spill, &t->sparse,
                       &t->stage_off[0], &t->stage_off[1], &t->stage_hits[0], &t->stage_hits[1]})
         b->release(s);
-    t->spill_nq = 0;
+    t->spill_chunks = t->spill_want = 0;
 }
 
 }  // namespace lbvh

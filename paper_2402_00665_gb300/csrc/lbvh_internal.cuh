@@ -328,13 +328,25 @@ inline int walk_choice_order_bits(int c) { return c >= kWalkKinds ? 24 : 30; }
 // hold hits). When the pool runs out, the query walks a second time instead.
 constexpr int kSpillChunkWords = 64;
 constexpr uint32_t kSpilledTag = 1u << 31;  // overflow-list entry whose hits are all in slot + chunks
+// The pool's chunks for nq queries: a sixteenth of nq; up to 2^20 queries, an
+// eighth of nq (32 bytes a query, the slots take 256), as long as that is no
+// more than 65,536 (16 MB). A few queries among clustered points want more than
+// a sixteenth (30,011 queries of 20 hits on average 2,169 chunks; with 1,875
+// of them the second walk took 0.42 ms). A tree whose pool ran out all the
+// same has a larger one from the next query on (spill_chunks_after).
+constexpr int64_t kSpillGrowMax = 65536;
 inline uint32_t spill_chunks_for(int64_t nq) {
-    // few queries may all have long lists: 16 chunks each, as long as that is
-    // no more than 16 MB (30,011 queries of 20 hits on average, one in 20 past
-    // its slot: nq / 16 chunks ran out, and the second walk took 0.42 ms)
-    int64_t c = 16 * nq < 65536 ? 16 * nq : 65536;
+    int64_t c = nq / 8 < kSpillGrowMax ? nq / 8 : kSpillGrowMax;
     if (c < nq / 16) c = nq / 16;
     return (uint32_t)(c < 1024 ? 1024 : (c > (1 << 26) ? (1 << 26) : c));
+}
+// What a tree's next pool should hold after a query asked for `used` chunks of
+// a pool of `had` (walks that find it empty stop asking, so `used` may be less
+// than they needed): 0 if it did not run out, else twice, up to kSpillGrowMax.
+inline uint32_t spill_chunks_after(uint32_t used, uint32_t had) {
+    if (used <= had) return 0;
+    const int64_t twice = 2 * (int64_t)(used > had ? used : had);
+    return (uint32_t)(twice < kSpillGrowMax ? twice : kSpillGrowMax);
 }
 
 struct QueryScratch {
