@@ -429,6 +429,11 @@ typedef struct {
 lbvh_status lbvh_server_create(uint64_t hbm_budget_bytes, int slots, int max_batch,
                                lbvh_server_t *out);
 
+/* The working bytes a server's admission counts for a request: its sizes
+ * decide (n, nq, kind, qkind, capacity; no pointer is read). 0 for sizes out
+ * of range. */
+uint64_t lbvh_request_bytes(const lbvh_request *request);
+
 /* Queue a request (copied; returns at once). *ticket identifies it. */
 lbvh_status lbvh_server_submit(lbvh_server_t server, const lbvh_request *request, uint64_t *ticket);
 

@@ -147,14 +147,20 @@ struct Slot {
     std::unique_ptr<Job> job;
 };
 
-// Device bytes one build + query request needs while it runs (inputs staged,
-// sort buffers, nodes, store, query scratch, output): an upper estimate.
+// Device bytes one build + query request needs while it runs: an upper
+// estimate of what grows with it. (Every job holds 256 KB of the pool for
+// long lists and some tables besides.)
 uint64_t estimate_bytes(const lbvh_request &r) {
     const uint64_t n = (uint64_t)r.n, nq = (uint64_t)r.nq;
     const uint64_t prim = r.kind == LBVH_PRIM_POINTS ? 12 : 24;
     const uint64_t qsz = r.qkind == LBVH_Q_SPHERE ? 12 : (r.qkind == LBVH_Q_BOX ? 24 : 32);
-    const uint64_t build = n * (prim + 24 + 24 + 48 + 8 + 16) + (uint64_t)lbvh::pack_records(r.n) * 32;
-    const uint64_t query = nq * (qsz + 4 + 8 + lbvh::kQueryBufferHits * 4 + 4 + 8 + 24 + 8) + r.capacity * 4;
+    // inputs staged, sort buffers, nodes, store; leaf blocks; lists between the construct's merges
+    const uint64_t build = n * (prim + 24 + 24 + 48 + 8 + 16) + (uint64_t)lbvh::pack_records(r.n) * 32 +
+                           (n > 0 ? lbvh::construct_pend_bytes(r.n) : 0);
+    // inputs staged, walk slots, counts and lists, order; the share of the pool for long lists, packets left over
+    const uint64_t pool = lbvh::kSpillChunkWords * 4 / 8;  // bytes per query (spill_chunks_for)
+    const uint64_t query = nq * (qsz + 4 + 8 + lbvh::kQueryBufferHits * 4 + 4 + 8 + 24 + 8 + pool) + nq / 4 + 8 +
+                           r.capacity * 4;
     return std::max<uint64_t>(build + query, 1);  // a running job always counts as in flight
 }
 
@@ -547,6 +553,12 @@ lbvh_status lbvh_server_create(uint64_t hbm_budget_bytes, int slots, int max_bat
     srv->scheduler = std::thread([srv] { srv->schedule_loop(); });
     *out = srv;
     return LBVH_OK;
+}
+
+uint64_t lbvh_request_bytes(const lbvh_request *request) {
+    if (!request || request->n < 0 || request->n > LBVH_MAX_PRIMS || request->nq < 0 || request->nq > LBVH_MAX_PRIMS)
+        return 0;
+    return estimate_bytes(*request);
 }
 
 lbvh_status lbvh_server_submit(lbvh_server_t srv, const lbvh_request *req, uint64_t *ticket) {

@@ -59,6 +59,7 @@ SIGNATURES = {
     "lbvh_batch_export": (_I32, [_P, _I64] + [_P] * 8),
     "lbvh_batch_sort_variant": (_I32, [_P, _P]),
     "lbvh_server_create": (_I32, [_U64, _I32, _I32, _P]),
+    "lbvh_request_bytes": (ctypes.c_uint64, [_P]),
     "lbvh_server_submit": (_I32, [_P, _P, _P]),
     "lbvh_server_wait": (_I32, [_P, _U64, _P]),
     "lbvh_server_stats": (_I32, [_P, _P, _P, _P, _P]),
