@@ -283,6 +283,11 @@ lbvh_status lbvh_tree_walk_visits(lbvh_tree_t tree, const float *d_queries, int6
  *              query with a non-finite coordinate has no neighbours.
  *   d_dist2    float[nq][k] out or NULL: the squared distances, +inf padding.
  * Buffers are the caller's. Synchronises `stream` once (for the status).
+ * Beside the order of the queries (36 bytes each) the tree holds scratch for
+ * 5 <= k <= 32: 512 bytes for each of up to 2^20 queries at a time (1 KB for
+ * k > 16), kept for later queries, and 4.6 bytes per primitive for the boxes
+ * of leaf blocks. Where these cannot be had the call runs without them,
+ * slower.
  * LBVH_ERR_INVALID on bad arguments or an unbuilt tree; the build's error if
  * it failed; LBVH_ERR_CORRUPT if a walk met an id outside the tree. */
 lbvh_status lbvh_knn(lbvh_tree_t tree, const float *d_queries, int64_t nq, int k, uint32_t *d_idx,
@@ -528,6 +533,11 @@ lbvh_status lbvh_test_hold_sort_tile(int64_t tile);
  * waits run out, the query or batch reports LBVH_ERR_TIMEOUT and no hit is
  * written. */
 lbvh_status lbvh_test_hold_scan_tile(int64_t tile);
+
+/* Test hook for memory that cannot be had, off by default (0). While set,
+ * every allocation of more than `max_bytes` of device memory by the library
+ * fails as if the device had none left; nothing is allocated instead. */
+lbvh_status lbvh_test_limit_allocation(uint64_t max_bytes);
 
 /* Test hook for the order of arrivals in Algorithm 4, off by default
  * (max_ns = 0). While set, every thread of the bottom-up construct waits a

@@ -248,7 +248,11 @@ cudaError_t device_pool(cudaMemPool_t *out) {
 }
 }  // namespace
 
+// Test hook (lbvh_test_limit_allocation): larger allocations fail.
+static std::atomic<uint64_t> g_alloc_limit{UINT64_MAX};
+
 cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t s) {
+    if (bytes > g_alloc_limit.load(std::memory_order_relaxed)) return cudaErrorMemoryAllocation;
     cudaMemPool_t pool = nullptr;
     const cudaError_t e = device_pool(&pool);
     if (e != cudaSuccess) return e;
@@ -444,9 +448,18 @@ lbvh_status query_count(lbvh_tree_t t, lbvh::QueryArgs &qa, int64_t *d_offsets,
     if (ost != LBVH_OK) return ost;
     bool pack = false;
     if (how != kRangeNodes) {
-        LBVH_CUDA(t->sparse.ensure((unq / 32 + 1) * sizeof(uint2), s));
         pack = !t->packed_ok;
-        if (pack) LBVH_CUDA(t->packed.ensure((size_t)pack_records(t->n) * 32, s));
+        cudaError_t e = t->sparse.ensure((unq / 32 + 1) * sizeof(uint2), s);
+        if (e == cudaSuccess && pack) e = t->packed.ensure((size_t)pack_records(t->n) * 32, s);
+        if (e == cudaErrorMemoryAllocation) {  // no room for the blocks: Algorithm 1 needs none
+            (void)cudaGetLastError();
+            how = kRangeNodes;
+            pack = false;
+            if (!qa.order) ost = query_order(t, qa, s, walk_choice_order_bits(choice));
+            if (ost != LBVH_OK) return ost;
+        } else {
+            LBVH_CUDA(e);
+        }
     }
     const QueryScratch qs = query_scratch(t);
     t->prof.begin(LBVH_STAGE_QCOUNT, s);
@@ -1373,10 +1386,19 @@ lbvh_status lbvh_knn(lbvh_tree_t t, const float *d_queries, int64_t nq, int k, u
     if (how != kKnnHeap) {
         sc.chunk = knn_chunk(nq);
         const int64_t chunks = (nq + sc.chunk - 1) / sc.chunk;
-        if (how == kKnnPackets) LBVH_CUDA(t->slots.ensure((size_t)sc.chunk * knn_slot_bytes(k), s));
-        LBVH_CUDA(t->counts.ensure((size_t)(3 * sc.chunk + chunks) * 4, s));
         pack = !t->packed_ok;
-        if (pack) LBVH_CUDA(t->packed.ensure((size_t)pack_records(t->n) * 32, s));
+        cudaError_t e = t->counts.ensure((size_t)(3 * sc.chunk + chunks) * 4, s);
+        if (e == cudaSuccess && how == kKnnPackets) e = t->slots.ensure((size_t)sc.chunk * knn_slot_bytes(k), s);
+        if (e == cudaSuccess && pack) e = t->packed.ensure((size_t)pack_records(t->n) * 32, s);
+        if (e == cudaErrorMemoryAllocation) {  // no room for that: the heap keeps its lists in the threads
+            (void)cudaGetLastError();
+            how = kKnnHeap;
+            pack = false;
+            if (!qa.order) st = query_order(t, qa, s);
+            if (st != LBVH_OK) return st;
+        } else {
+            LBVH_CUDA(e);
+        }
         sc.slots = t->slots.as<uint2>();
         sc.counts = t->counts.as<uint32_t>();
         sc.radii2 = t->counts.as<float>() + sc.chunk;
@@ -1446,6 +1468,11 @@ lbvh_status lbvh_test_hold_sort_tile(int64_t tile) {
 lbvh_status lbvh_test_hold_scan_tile(int64_t tile) {
     if (tile < -1) return LBVH_ERR_INVALID;
     lbvh::scan_set_hold_tile(tile);
+    return LBVH_OK;
+}
+
+lbvh_status lbvh_test_limit_allocation(uint64_t max_bytes) {
+    lbvh::g_alloc_limit.store(max_bytes > 0 ? max_bytes : UINT64_MAX, std::memory_order_relaxed);
     return LBVH_OK;
 }
 
@@ -1744,7 +1771,9 @@ lbvh_status tree_from_batch(lbvh_batch_t b, int64_t instance, lbvh_tree_t t, cud
     LBVH_CUDA(t->hist.ensure((size_t)kMaxPasses * kRadix * 4, s));
     LBVH_CUDA(t->bounds.ensure(6 * 4, s));
     const size_t pack_bytes = (size_t)pack_records(n) * 32;
-    LBVH_CUDA(t->packed.ensure(pack_bytes, s));
+    const cudaError_t room = t->packed.ensure(pack_bytes, s);
+    if (room == cudaErrorMemoryAllocation) (void)cudaGetLastError();  // queries of the tree do without
+    else LBVH_CUDA(room);
     t->lean = true;
     t->loaded = false;
     t->n = n;
@@ -1757,7 +1786,7 @@ lbvh_status tree_from_batch(lbvh_batch_t b, int64_t instance, lbvh_tree_t t, cud
     if (units > 0)
         LBVH_CUDA(cudaMemcpyAsync(t->nodes.p, b->nodes.as<float4>() + b->h_node_start[instance], units * 16,
                                   cudaMemcpyDeviceToDevice, s));
-    t->packed_ok = b->packets();  // else the first query packs them
+    t->packed_ok = b->packets() && room == cudaSuccess;  // else the first query packs them
     if (t->packed_ok && pack_bytes > 0)
         LBVH_CUDA(cudaMemcpyAsync(t->packed.p, b->packed.as<float4>() + 2 * b->h_pack_start[instance], pack_bytes,
                                   cudaMemcpyDeviceToDevice, s));
