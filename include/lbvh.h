@@ -612,7 +612,12 @@ uint64_t lbvh_kernel_launches(void);
  * A process-wide cache holds the choice for each configuration (the GPU's
  * name, ceil(log2 n), Morton bits, primitive kind, query kind, trees built
  * together); builds and queries use the cached choice for their
- * configuration, else variant 0. */
+ * configuration, else the default: walk variant 0, and sort variant 0 or, for
+ * trees of up to 8,192 primitives (16,384 with codes wider than 30 bits),
+ * bounds, codes and sort in one launch. A cached choice is used as it is,
+ * whichever version of the library measured it; walk variant 0 and the one
+ * launch came with the walks over leaf blocks, so choices from before are
+ * best measured again. */
 int lbvh_sort_variant_count(void);
 int lbvh_walk_variant_count(void);
 
@@ -622,7 +627,9 @@ int lbvh_walk_variant_count(void);
  * stores the fastest of each in the cache and leaves the tree built with the
  * chosen sort variant.
  * Arguments as lbvh_build and lbvh_query_into; sort_variant / walk_variant
- * (nullable) receive the choices. Synchronises `stream`. */
+ * (nullable) receive the choices (sort variant -1: a small tree's one launch,
+ * which is timed against the variants with their bounds and codes).
+ * Synchronises `stream`. */
 lbvh_status lbvh_tree_autotune(lbvh_tree_t tree, const float *d_prims, int64_t n, int kind, int morton_bits,
                                const float *d_queries, int64_t nq, int query_kind, const float *d_radii,
                                float radius, lbvh_stream_t stream, int *sort_variant, int *walk_variant);

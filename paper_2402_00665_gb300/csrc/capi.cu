@@ -286,6 +286,9 @@ int device_sm_count() {
 
 namespace {
 
+// A tree's sort_choice for the default whatever the tuner's cache says.
+constexpr int kSortDefault = -2;
+
 // Storage for a tree of n primitives; the control block and `store` are
 // zeroed when first allocated and kept clean by the kernels afterwards.
 lbvh_status reserve_tree(lbvh_tree_s *t, int64_t n, int kind, cudaStream_t s) {
@@ -887,7 +890,12 @@ lbvh_status build_impl(lbvh_tree_t t, const float *d_prims, int64_t n, int kind,
     t->prof.clear(LBVH_STAGE_SORTRUNS, LBVH_STAGE_SORTRUNS + 1);
     if (n > 0) {
         const uint32_t *perm = t->vals[0].as<uint32_t>();
-        if (n <= small_sort_max(morton_bits) && t->sort_choice < 0) {
+        // the sort choice: tile shape, and whether the top-bits sort covers
+        // one byte fewer (more elements in runs of equal sorted bits); none
+        // chosen: one launch for small trees, else the default shape
+        int choice = t->sort_choice;
+        if (choice == -1) choice = tune_sort_choice(n, morton_bits, kind, 1);
+        if (n <= small_sort_max(morton_bits) && choice < 0) {
             t->prof.begin(LBVH_STAGE_SORT0, s);
             launch_small_sort(d_prims, n, kind, morton_bits, t->bounds.as<float>(), t->vals[0].as<uint32_t>(), c, s);
             t->prof.end(LBVH_STAGE_SORT0, s);
@@ -905,9 +913,6 @@ lbvh_status build_impl(lbvh_tree_t t, const float *d_prims, int64_t n, int kind,
             // index) to run_code_sort
             const bool packed = morton_bits <= 30;
             const int ib = top_index_bits(n);
-            // the sort choice: tile shape, and whether the top-bits sort covers
-            // one byte fewer (more elements in runs of equal sorted bits)
-            const int choice = t->sort_choice >= 0 ? t->sort_choice : tune_sort_choice(n, morton_bits, kind, 1);
             const int variant = sort_choice_tile(choice);
             const int skip = packed ? 0 : sort_choice_skip(choice);
             launch_encode(d_prims, n, kind, morton_bits, t->bounds.as<float>(), t->keys[0].as<uint64_t>(),
@@ -1865,15 +1870,18 @@ lbvh_status lbvh_tree_autotune(lbvh_tree_t t, const float *d_prims, int64_t n, i
     };
     // the sort: every choice on this build's own keys (tile shapes; for codes
     // wider than 30 bits also one top-bits pass fewer), the best of two runs
-    // each, timed over the passes and the runs stage
+    // each, timed over the passes and the runs stage. A small tree's sort in
+    // one launch covers the bounds and the codes too, so there they count
+    // for all.
+    const bool small = n > 0 && n <= small_sort_max(morton_bits);
     float best_sort = 1e30f;
     int pick_sort = 0;
     const int choices = morton_bits <= 30 ? sort_variant_count() : build_sort_choices();
-    for (int v = 0; v < choices && n > 0; ++v) {
+    for (int v = small ? kSortDefault : 0; v < choices && n > 0; v = v < 0 ? 0 : v + 1) {
         t->sort_choice = v;
         for (int rep = 0; rep < 2; ++rep) {
             if ((st = lbvh_build(t, d_prims, n, kind, morton_bits, stream)) != LBVH_OK) return finish(st);
-            const float mp = stages_ms(t, LBVH_STAGE_SORT0, LBVH_STAGE_SORT0 + kMaxPasses);
+            const float mp = stages_ms(t, small ? LBVH_STAGE_BOUNDS : LBVH_STAGE_SORT0, LBVH_STAGE_SORT0 + kMaxPasses);
             const float mr = stages_ms(t, LBVH_STAGE_SORTRUNS, LBVH_STAGE_SORTRUNS + 1);
             const float ms = mp < 0.0f || mr < 0.0f ? -1.0f : mp + mr;
             if (ms < 0.0f) return finish(LBVH_ERR_CUDA);
@@ -1883,12 +1891,7 @@ lbvh_status lbvh_tree_autotune(lbvh_tree_t t, const float *d_prims, int64_t n, i
             }
         }
     }
-    if (n > 0) {
-        TuneChoice made;
-        made.sort = pick_sort;
-        made.sort_ms = best_sort;
-        tune_put(tune_key(n, morton_bits, kind, -1, 1), made);
-    }
+    if (n > 0) tune_set_sort(tune_key(n, morton_bits, kind, -1, 1), std::max(pick_sort, -1), best_sort);
     t->sort_choice = pick_sort;
     if ((st = lbvh_build(t, d_prims, n, kind, morton_bits, stream)) != LBVH_OK) return finish(st);
     if ((st = lbvh_tree_status(t)) != LBVH_OK) return finish(st);
@@ -1923,7 +1926,7 @@ lbvh_status lbvh_tree_autotune(lbvh_tree_t t, const float *d_prims, int64_t n, i
         made.walk_ms = best_walk;
         tune_put(tune_key(n, morton_bits, kind, qkind, 1), made);
     }
-    if (sort_variant) *sort_variant = pick_sort;
+    if (sort_variant) *sort_variant = std::max(pick_sort, -1);
     if (walk_variant) *walk_variant = pick_walk;
     return finish(LBVH_OK);
 }

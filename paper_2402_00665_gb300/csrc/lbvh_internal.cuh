@@ -551,6 +551,8 @@ TuneKey tune_key(int64_t n, int bits, int kind, int qkind, int64_t instances);
 bool tune_find(const TuneKey &k, TuneChoice *out);
 // Stores the fields of c that are set (>= 0), keeping the others.
 void tune_put(const TuneKey &k, const TuneChoice &c);
+// Sets the entry's sort, also to -1 (the default is the fastest).
+void tune_set_sort(const TuneKey &k, int sort, float ms);
 // The cached choices for a configuration: the sort variant (-1: the default)
 // and the walk (kWalkThread when nothing is cached).
 int tune_sort_choice(int64_t n, int bits, int kind, int64_t instances);

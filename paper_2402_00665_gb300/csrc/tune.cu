@@ -85,6 +85,13 @@ void tune_put(const TuneKey &k, const TuneChoice &c) {
     }
 }
 
+void tune_set_sort(const TuneKey &k, int sort, float ms) {
+    std::lock_guard<std::mutex> lock(g_mu);
+    TuneChoice &e = g_cache[k];
+    e.sort = sort;
+    e.sort_ms = ms;
+}
+
 int tune_sort_choice(int64_t n, int bits, int kind, int64_t instances) {
     TuneChoice c;
     return tune_find(tune_key(n, bits, kind, -1, instances), &c) ? c.sort : -1;
