@@ -204,7 +204,8 @@ __device__ __forceinline__ uint32_t test32(const PacketSmem<kP> &sm, int base, c
 // candidate ring + j). False, with nothing taken: its region is not tight and
 // more than kLeafList - 32 leaf blocks meet it. Warp-wide.
 // Keep::kMaxBlocks (0: none): past this many leaf blocks the walk gives up as
-// well (k.reset() drops what was taken), and a lane is out once k.full().
+// well (k.reset() drops what its own lanes took; the others may hold what an
+// earlier packet gave them), and a lane is out once k.full().
 template <int kQ, int kP, typename Keep>
 __device__ __forceinline__ bool packet_walk(const Blocks &t, PacketSmem<kP> &sm, const typename QueryOf<kQ>::type &q,
                                             bool use, Keep &k) {
@@ -212,6 +213,7 @@ __device__ __forceinline__ bool packet_walk(const Blocks &t, PacketSmem<kP> &sm,
     const int lane = threadIdx.x & 31, sub = lane >> 3;
     const uint32_t below = (1u << lane) - 1u;
     Region<Q> region;
+    const bool mine = use;
     use = use && !Region<Q>::hopeless(q);
     if (!__any_sync(kFull, use)) return true;
     region.gather(q, use);
@@ -256,7 +258,7 @@ __device__ __forceinline__ bool packet_walk(const Blocks &t, PacketSmem<kP> &sm,
         if constexpr (Keep::kMaxBlocks > 0) {
             read += nl;
             if (read > Keep::kMaxBlocks) {
-                k.reset();
+                if (mine) k.reset();
                 return false;
             }
         }
