@@ -45,6 +45,7 @@ template <>
 struct Region<Sphere> {
     float3 lo, hi;  // the box of the centres
     float r2;       // the largest squared radius
+    static constexpr bool kShapes = false;
     // `use`: this lane's query belongs to the packet (warp-wide call)
     __device__ __forceinline__ void gather(const Sphere &s, bool use) {
         const float inf = __int_as_float(0x7f800000);
@@ -94,6 +95,19 @@ struct Region<Box> {
                u.hi.z - u.lo.z <= 3.0f * size.z;
     }
     __device__ __forceinline__ bool meets(float3 blo, float3 bhi) const { return hits(u, blo, bhi); }
+    // The axes along which a query is not much smaller than the largest one
+    // there (bit 0: x). Rods along x beside rods along y share a region that none
+    // of them comes near to filling; those of one shape do not.
+    static constexpr bool kShapes = true;
+    __device__ __forceinline__ uint32_t shape(const Box &q) const {
+        return (8.0f * (q.hi.x - q.lo.x) >= size.x ? 1u : 0u) | (8.0f * (q.hi.y - q.lo.y) >= size.y ? 2u : 0u) |
+               (8.0f * (q.hi.z - q.lo.z) >= size.z ? 4u : 0u);
+    }
+    // Leaf blocks like this one are so small that queries of another shape may pass
+    // them by. (Rods among rods: every block is as long as a rod along all axes.)
+    __device__ __forceinline__ bool passes(float3 blo, float3 bhi) const {
+        return 2.0f * (bhi.x - blo.x) <= size.x && 2.0f * (bhi.y - blo.y) <= size.y && 2.0f * (bhi.z - blo.z) <= size.z;
+    }
 };
 
 // ---------------------------------------------------------------- packets
@@ -201,21 +215,25 @@ __device__ __forceinline__ uint32_t test32(const PacketSmem<kP> &sm, int base, c
 
 // The packet of the lanes with `use` set walks one tree; k.take(m, sm, ring, q)
 // gets every set of candidates with the lane's hits among them (bit 31 - j:
-// candidate ring + j). False, with nothing taken: its region is not tight and
-// more than kLeafList - 32 leaf blocks meet it. Warp-wide.
+// candidate ring + j). Warp-wide. If more than kLeafList - 32 leaf blocks meet
+// its region, a packet that is not tight gives up with nothing taken, and so does a
+// whole one (not yet cut) of several shapes if those blocks are small; `shape` is
+// then the lane's.
 // Keep::kMaxBlocks (0: none): past this many leaf blocks the walk gives up as
 // well (k.reset() drops what its own lanes took; the others may hold what an
 // earlier packet gave them), and a lane is out once k.full().
+enum Walked : int { kWalked, kTooLoose, kUnlike };
+
 template <int kQ, int kP, typename Keep>
-__device__ __forceinline__ bool packet_walk(const Blocks &t, PacketSmem<kP> &sm, const typename QueryOf<kQ>::type &q,
-                                            bool use, Keep &k) {
+__device__ __forceinline__ Walked packet_walk(const Blocks &t, PacketSmem<kP> &sm, const typename QueryOf<kQ>::type &q,
+                                              bool use, bool whole, uint32_t &shape, Keep &k) {
     using Q = typename QueryOf<kQ>::type;
     const int lane = threadIdx.x & 31, sub = lane >> 3;
     const uint32_t below = (1u << lane) - 1u;
     Region<Q> region;
     const bool mine = use;
     use = use && !Region<Q>::hopeless(q);
-    if (!__any_sync(kFull, use)) return true;
+    if (!__any_sync(kFull, use)) return kWalked;
     region.gather(q, use);
     const bool tight = region.tight();
     int ns = 0, nl = 0;      // entries of the stack and of the leaf list
@@ -253,13 +271,26 @@ __device__ __forceinline__ bool packet_walk(const Blocks &t, PacketSmem<kP> &sm,
             nl += __popc(leafs);
             __syncwarp();
         }
-        if (ns > 0 && fresh && !tight) return false;
+        if (ns > 0 && fresh) {
+            if (!tight) return kTooLoose;
+            if constexpr (Region<Q>::kShapes) {
+                if (whole) {
+                    region.gather(q, use);  // (its sizes were not kept in registers)
+                    shape = region.shape(q);
+                    const uint32_t one = __shfl_sync(kFull, shape, __ffs(__ballot_sync(kFull, use)) - 1);
+                    float4 a, b;
+                    ld_node32(t.rec + 2 * (int64_t)sm.list[kStack + lane], a, b);  // one of the leaf blocks
+                    const uint32_t small = __ballot_sync(kFull, region.passes(xyz(a), xyz(b)));
+                    if (__any_sync(kFull, use && shape != one) && __popc(small) >= 16) return kUnlike;
+                }
+            }
+        }
         fresh = false;
         if constexpr (Keep::kMaxBlocks > 0) {
             read += nl;
             if (read > Keep::kMaxBlocks) {
                 if (mine) k.reset();
-                return false;
+                return kTooLoose;
             }
         }
         // ---- leaves
@@ -304,7 +335,7 @@ __device__ __forceinline__ bool packet_walk(const Blocks &t, PacketSmem<kP> &sm,
                     const bool out = use && k.full();
                     if (__any_sync(kFull, out)) {  // the region of the others
                         use = use && !out;
-                        if (!__any_sync(kFull, use)) return true;
+                        if (!__any_sync(kFull, use)) return kWalked;
                         region.gather(q, use);
                     }
                 }
@@ -314,7 +345,7 @@ __device__ __forceinline__ bool packet_walk(const Blocks &t, PacketSmem<kP> &sm,
     }
     if (nc > 0) flush(nc);
     __syncwarp();
-    return true;
+    return kWalked;
 }
 
 __device__ __forceinline__ float3 middle(const Sphere &s) { return s.c; }
@@ -339,28 +370,37 @@ __device__ __forceinline__ uint32_t before_jump(const Q &q, uint32_t mine) {
     return mine & ((1u << cut) - 1u);
 }
 
-// The queries of `mine` (a run of lanes of one tree): as one packet, or as
-// two on either side of the widest jump. Returns the lanes left over, whose
-// queries lie too far apart.
+// The queries of `mine` (a run of lanes of one tree): as one packet, or, where
+// that gave up, as two on either side of the widest jump, or one for each shape
+// (queries on as many points, whole call, as one packet / by shapes: 300,000 rods
+// of 0.2 x 0.002^2 along random axes 750 / 305 us, Algorithm 1 256; 10^6 rods
+// of half the size 1135 / 525, 448; 2 * 10^6 plates of 0.07^2 x 0.001 2262 / 2252,
+// 2771). Returns the lanes left over, whose queries lie too far apart.
 template <int kQ, int kP, typename Keep>
 __device__ __forceinline__ uint32_t packets(const Blocks &t, PacketSmem<kP> &sm, const typename QueryOf<kQ>::type &q,
                                             uint32_t mine, Keep &k) {
     const int lane = threadIdx.x & 31;
-    uint32_t cur = mine, next = 0, left = 0;
-    bool whole = true;
+    uint32_t cur = mine, rest = 0, left = 0, shape = 0;
+    bool whole = true, by_shape = false;
     while (cur) {
-        if (!packet_walk<kQ, kP>(t, sm, q, (cur >> lane) & 1u, k)) {
-            if (whole && __popc(cur) > 1) {
-                const uint32_t first = before_jump(q, cur);
-                next = cur & ~first;
-                cur = first;
-                whole = false;
-                continue;
-            }
+        const Walked w = packet_walk<kQ, kP>(t, sm, q, (cur >> lane) & 1u, whole, shape, k);
+        if (w == kUnlike) {
+            by_shape = true;
+            rest = cur;
+        } else if (w == kTooLoose && whole && __popc(cur) > 1) {
+            const uint32_t first = before_jump(q, cur);
+            rest = cur & ~first;
+            cur = first;
+            whole = false;
+            continue;
+        } else if (w == kTooLoose) {
             left |= cur;
         }
-        cur = next;
-        next = 0;
+        whole = false;
+        cur = rest;
+        if (by_shape && rest)  // the first lane's shape
+            cur &= __ballot_sync(kFull, shape == __shfl_sync(kFull, shape, __ffs(rest) - 1));
+        rest &= ~cur;
     }
     return left;
 }
