@@ -196,8 +196,10 @@ __device__ __forceinline__ void load_node(const float4 *base, int unit, bool lea
 constexpr int kSlot = kQueryBufferHits;  // ids kept per walk (slot size)
 constexpr int kRegSort = 32;             // lists up to this long are sorted in one thread's registers
 
+// The query of walk position i. The order of a sort that gave up a wait holds
+// words it never wrote: whatever they are, no query past the last is indexed.
 __device__ __forceinline__ int64_t thread_query(const QueryArgs &qa, int64_t i) {
-    return qa.order ? (int64_t)__ldcs(qa.order + i) : i;
+    return qa.order ? min((int64_t)__ldcs(qa.order + i), qa.nq - 1) : i;
 }
 
 // Hits past a walk's slot: appended to chunks from the shared pool, the first
