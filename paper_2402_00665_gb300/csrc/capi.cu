@@ -397,9 +397,14 @@ lbvh_status query_order(lbvh_tree_t t, lbvh::QueryArgs &qa, cudaStream_t s, int 
                   t->hist.as<uint32_t>(), 1, curve, whole ? 1 : 0, s);
     LBVH_LAUNCHED();
     SortScratch scratch{t->hist.as<uint32_t>(), t->qlookback.as<uint32_t>(), sort_tiles_max(qa.nq) * kRadix};
-    qa.order = run_index_sort(t->qkeys[0].as<uint64_t>(), t->qkeys[1].as<uint64_t>(), t->qvals[0].as<uint32_t>(),
-                              qa.nq, bits, scratch, t->dctl(), s);
+    uint32_t *order = run_index_sort(t->qkeys[0].as<uint64_t>(), t->qkeys[1].as<uint64_t>(), t->qvals[0].as<uint32_t>(),
+                                     qa.nq, bits, scratch, t->dctl(), s);
     LBVH_LAUNCHED();
+    if (curve == kCodeHilbert) {
+        launch_refine_order(qa, whole ? 11 : bits / 3, t->bounds.as<float>(), order, t->dctl(), s);
+        LBVH_LAUNCHED();
+    }
+    qa.order = order;
     return LBVH_OK;
 }
 

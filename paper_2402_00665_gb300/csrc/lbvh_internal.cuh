@@ -361,6 +361,11 @@ struct QueryScratch {
 // The collecting walk (counts, short sorted lists, overflow list).
 void launch_query_collect(const TreeView &t, const QueryArgs &q, const QueryScratch &qs, Control *ctl,
                           cudaStream_t s);
+// A Hilbert order of q's spheres or boxes (kCodeHilbert words of 2^levels cells
+// per axis), made finer where many of them share a cell; a radius of 0: unknown
+// yet, so small (q.order is not read).
+void launch_refine_order(const QueryArgs &q, int levels, const float *bounds, uint32_t *order, const Control *ctl,
+                         cudaStream_t s);
 // k nearest neighbours of the query points q.queries (float[nq][3], q.order
 // the walk order) into rows of out_idx / out_d2 (uint32 / float [nq][k]);
 // codes: the tree's sorted codes (null: no seeding), bounds and bits of its
