@@ -1397,7 +1397,7 @@ lbvh_status lbvh_knn(lbvh_tree_t t, const float *d_queries, int64_t nq, int k, u
         sc.chunk = knn_chunk(nq);
         const int64_t chunks = (nq + sc.chunk - 1) / sc.chunk;
         pack = !t->packed_ok;
-        cudaError_t e = t->counts.ensure((size_t)(3 * sc.chunk + chunks) * 4, s);
+        cudaError_t e = t->counts.ensure((size_t)(4 * sc.chunk + chunks) * 4, s);
         if (e == cudaSuccess && how == kKnnPackets) e = t->slots.ensure((size_t)sc.chunk * knn_slot_bytes(k), s);
         if (e == cudaSuccess && pack) e = t->packed.ensure((size_t)pack_records(t->n) * 32, s);
         if (e == cudaErrorMemoryAllocation) {  // no room for that: the heap keeps its lists in the threads
@@ -1413,7 +1413,8 @@ lbvh_status lbvh_knn(lbvh_tree_t t, const float *d_queries, int64_t nq, int k, u
         sc.counts = t->counts.as<uint32_t>();
         sc.radii2 = t->counts.as<float>() + sc.chunk;
         sc.redo = sc.counts + 2 * sc.chunk;
-        sc.redo_counts = sc.counts + 3 * sc.chunk;
+        sc.ids = sc.counts + 3 * sc.chunk;
+        sc.redo_counts = sc.counts + 4 * sc.chunk;
     }
     t->prof.begin(LBVH_STAGE_QCOUNT, s);  // the kNN walk is timed as the query walk
     if (how != kKnnHeap) {

@@ -190,6 +190,10 @@ __global__ void __launch_bounds__(128)
 //   4. knn_redo_kernel    queries with fewer hits (their bound was cut too
 //      far) or more than are kept (a bound from leaves far away),
 //      8 lanes each with a bound that shrinks.
+// A bound is a key, not only a distance: of many copies of a point only those up to
+// an index can be among the k (16 nearest of 2 * 10^6 points on 27,000 places 4.91
+// ms with distances alone, so 1.11, the heap 1.19; 100,000 points on 100 places
+// 1.66, 0.72, 0.61).
 // Leaves of the bound's window and hits kept per query, in units of K.
 template <int kK>
 constexpr int kKnnMul = kK <= 8 ? 8 : 4;
@@ -286,12 +290,14 @@ __device__ __forceinline__ float leaf_d2(const float4 *leaves, int64_t pos, floa
 
 // radii2[j]: the bound of the query at walk position first + j, NaN for one
 // with a non-finite coordinate. `own`: the queries are the tree's primitives
-// in sorted order, so a walk position is a place in the codes.
+// in sorted order, so a walk position is a place in the codes. ids[j], only where
+// the bound is 0 (copies of a point, boxes around it): the largest index of k
+// of those leaves that lie at no distance, which ties at the bound need not exceed.
 template <int kP, int kK>
 __global__ void __launch_bounds__(128)
     knn_radius_kernel(TreeView t, const uint64_t *__restrict__ codes, const float *__restrict__ bounds, int bits,
                       QueryArgs qa, int k, int64_t first, int64_t count, bool own, float *__restrict__ radii2,
-                      const Control *ctl) {
+                      uint32_t *__restrict__ ids, const Control *ctl) {
     const int64_t j = (int64_t)blockIdx.x * 128 + threadIdx.x;
     if (j >= count || ctl->build_flags != 0) return;
     const int64_t qi = thread_query(qa, first + j);
@@ -316,6 +322,15 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
         for (int i = 0; i < kK; ++i)
             if (i == k - 1) bound = best[i];
+        if (bound == 0.0f) {
+            uint32_t id = 0;
+            for (int i = s0, left = k; left > 0; ++i)  // k of the window's kMul kK leaves
+                if (leaf_d2<kP>(t.leaves, i, c) == 0.0f) {
+                    id = max(id, __float_as_uint(t.leaves[kP == LBVH_PRIM_BOXES ? 2 * (int64_t)i : i].w) & kLeafIndexMask);
+                    --left;
+                }
+            ids[j] = id;
+        }
     }
     radii2[j] = bound;
 }
@@ -330,12 +345,18 @@ struct KnnKeeper {
     static constexpr int kMaxBlocks = 128 + 4 * kCap;
     uint2 *slot;
     float3 c;
+    uint32_t last;  // the largest index that counts
     uint32_t cnt;
     uint2 held;
     __device__ __forceinline__ bool full() const { return cnt > (uint32_t)kCap; }
     __device__ __forceinline__ void reset() { cnt = 0; }
     template <int kP, typename Q>
     __device__ __forceinline__ void take(uint32_t m, const PacketSmem<kP> &sm, int ring, const Q &) {
+        if (last != ~0u)
+            for (uint32_t r = m; r; r &= r - 1) {
+                const int b = 31 - __clz(r & (0u - r));
+                if (sm.id[ring + 31 - b] > last) m ^= 1u << b;
+            }
         const bool over = cnt + __popc(m) > (uint32_t)kCap;  // the slot is filled up, the rest dropped
         if (over)
             while (m && cnt + __popc(m) > (uint32_t)kCap) m &= m - 1;
@@ -361,7 +382,7 @@ template <int kP, int kK>
 __global__ void __launch_bounds__(32 * kPacketWarps, kPacketCtas<kP>)
     knn_packet_kernel(const float4 *__restrict__ leaves, const float4 *__restrict__ rec, int n, uint32_t start0,
                       QueryArgs qa, int64_t first, int64_t count, const float *__restrict__ radii2,
-                      uint2 *__restrict__ slots, uint32_t *__restrict__ counts, const Control *ctl) {
+                      const uint32_t *__restrict__ ids, uint2 *__restrict__ slots, uint32_t *__restrict__ counts, const Control *ctl) {
     constexpr int kCap = kKnnMul<kK> * kK;
     __shared__ PacketSmem<kP> s_all[kPacketWarps];
     PacketSmem<kP> &sm = s_all[threadIdx.x >> 5];
@@ -387,7 +408,7 @@ __global__ void __launch_bounds__(32 * kPacketWarps, kPacketCtas<kP>)
         if (lane == __ffs(same) - 1) rest = inf;
     }
     if (finite) q.r2 = fminf(q.r2, kKnnCut<kK> * fourth);
-    KnnKeeper<kCap> k{slots + j * kCap, q.c, 0u, make_uint2(0u, 0u)};
+    KnnKeeper<kCap> k{slots + j * kCap, q.c, has && q.r2 == 0.0f ? ids[j] : ~0u, 0u, make_uint2(0u, 0u)};
     const uint32_t left = packets<LBVH_Q_SPHERE, kP>(Blocks{leaves, rec, n, start0}, sm, q, __ballot_sync(kFull, has), k);
     if (!has) return;
     if (k.cnt <= (uint32_t)kCap && (k.cnt & 1u)) k.slot[k.cnt - 1] = k.held;
@@ -428,7 +449,7 @@ template <int kP, int kK>
 __global__ void __launch_bounds__(128)
     knn_redo_kernel(const float4 *__restrict__ leaves, const float4 *__restrict__ rec, int n, uint32_t start0,
                     QueryArgs qa, int k, int64_t first, int64_t count, const float *__restrict__ radii2,
-                    const uint32_t *__restrict__ redo, const uint32_t *redo_count, uint32_t *__restrict__ out_idx,
+                    const uint32_t *__restrict__ ids, const uint32_t *__restrict__ redo, const uint32_t *redo_count, uint32_t *__restrict__ out_idx,
                     float *__restrict__ out_d2, const Control *ctl) {
     constexpr int kCap = kKnnMul<kK> * kK;
     __shared__ uint32_t s_stack[128 / 8][kSparseStack];
@@ -447,6 +468,7 @@ __global__ void __launch_bounds__(128)
         const float3 c =
             make_float3(__ldg(qa.queries + 3 * qi), __ldg(qa.queries + 3 * qi + 1), __ldg(qa.queries + 3 * qi + 2));
         float r2 = radii2[j];
+        uint64_t worst = knn_key(r2, redo || r2 == 0.0f ? ids[j] : ~0u);  // the k smallest keys are no larger
         int cnt = 0, ns = go && built ? 1 : 0;
         if (sl == 0) stack[0] = 0u;
         __syncwarp();
@@ -469,8 +491,8 @@ __global__ void __launch_bounds__(128)
                     if (!leaf) b = __ldg(p + 1);
                 }
                 d2 = box_d2(c, xyz(a), xyz(b));
-                hit = d2 <= r2 && (leaf || __float_as_uint(b.w) == kBlockExists);
                 key = knn_key(d2, __float_as_uint(a.w) & kLeafIndexMask);
+                hit = d2 <= r2 && (leaf ? key <= worst : __float_as_uint(b.w) == kBlockExists);
             }
             const uint32_t bits = (__ballot_sync(kFull, hit) >> shift) & 0xffu;
             if (act) --ns;
@@ -482,7 +504,7 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
                 for (int o = 1; o < kFan; ++o) {
                     const float other = __shfl_xor_sync(kFull, far, o);
-                    farther += other > far || (other == far && (sl ^ o) < sl);
+                    farther += other > far || (other == far && (sl ^ o) > sl);
                 }
                 if (!leaf) before = farther;
             }
@@ -498,7 +520,8 @@ __global__ void __launch_bounds__(128)
                 const int kept = keep_smallest<kCap>(keys, cnt > kCap - 8 ? cnt : 0, k, sl);
                 if (cnt > kCap - 8) {
                     cnt = kept;
-                    r2 = fminf(r2, __uint_as_float((uint32_t)(keys[k - 1] >> 32)));
+                    worst = keys[k - 1];
+                    r2 = fminf(r2, __uint_as_float((uint32_t)(worst >> 32)));
                 }
                 __syncwarp();
             }
@@ -514,12 +537,13 @@ __global__ void __launch_bounds__(128)
     }
 }
 
-// A query with too few or too many hits goes to the list `redo`; radii2 holds
-// its bound (the uncut one, or the k-th smallest of the kCap hits kept).
+// A query with too few or too many hits goes to the list `redo`; radii2 and ids
+// hold its bound (the uncut one, or the k-th smallest of the kCap hits kept).
 template <int kK>
 __global__ void __launch_bounds__(128)
     knn_select_kernel(QueryArgs qa, int k, int64_t first, int64_t count, const uint2 *__restrict__ slots,
-                      const uint32_t *__restrict__ counts, float *__restrict__ radii2, uint32_t *redo,
+                      const uint32_t *__restrict__ counts, float *__restrict__ radii2, uint32_t *__restrict__ ids,
+                      uint32_t *redo,
                       uint32_t *redo_count, uint32_t *__restrict__ out_idx, float *__restrict__ out_d2,
                       const Control *ctl) {
     constexpr int kCap = kKnnMul<kK> * kK;
@@ -530,6 +554,7 @@ __global__ void __launch_bounds__(128)
     const bool none = c == kNoNeighbours;
     if (!none && c < (uint32_t)k) {
         redo[atomicAdd(redo_count, 1u)] = (uint32_t)j;
+        if (radii2[j] != 0.0f) ids[j] = ~0u;
         return;
     }
     const bool over = !none && c > (uint32_t)kCap;
@@ -555,11 +580,12 @@ __global__ void __launch_bounds__(128)
         merge_smallest(best, v);
     }
     if (over) {  // the k-th smallest of some hits bounds the k-th of all
-        uint32_t bound = 0;
+        uint64_t bound = 0;
 #pragma unroll
         for (int i = 0; i < kK; ++i)
-            if (i == k - 1) bound = (uint32_t)(best[i] >> 32);
-        radii2[j] = __uint_as_float(bound);
+            if (i == k - 1) bound = best[i];
+        radii2[j] = __uint_as_float((uint32_t)(bound >> 32));
+        ids[j] = (uint32_t)bound;
         redo[atomicAdd(redo_count, 1u)] = (uint32_t)j;
         return;
     }
@@ -618,9 +644,9 @@ void knn_chunks(const TreeView &t, const float4 *rec, const uint64_t *codes, con
     const int64_t redo_grid = (int64_t)device_sm_count() * 12;
     if (how == kKnnSparse) {  // one chunk: the bounds, then 8 lanes for every query
         knn_radius_kernel<kP, kK><<<(unsigned)((q.nq + 127) / 128), 128, 0, s>>>(t, codes, bounds, bits, q, k, 0, q.nq, own,
-                                                                                 sc.radii2, ctl);
+                                                                                 sc.radii2, sc.ids, ctl);
         knn_redo_kernel<kP, kK><<<(unsigned)std::min<int64_t>((q.nq + 15) / 16, redo_grid), 128, 0, s>>>(
-            t.leaves, rec, (int)t.n, pack_leaf_start(t.n), q, k, 0, q.nq, sc.radii2, nullptr, nullptr, out_idx, out_d2, ctl);
+            t.leaves, rec, (int)t.n, pack_leaf_start(t.n), q, k, 0, q.nq, sc.radii2, sc.ids, nullptr, nullptr, out_idx, out_d2, ctl);
         count_launches(2);
         return;
     }
@@ -629,15 +655,16 @@ void knn_chunks(const TreeView &t, const float4 *rec, const uint64_t *codes, con
     for (int64_t first = 0; first < q.nq; first += sc.chunk) {
         const int64_t count = std::min(sc.chunk, q.nq - first);
         const unsigned blocks = (unsigned)((count + 127) / 128);
-        knn_radius_kernel<kP, kK><<<blocks, 128, 0, s>>>(t, codes, bounds, bits, q, k, first, count, own, sc.radii2, ctl);
+        knn_radius_kernel<kP, kK><<<blocks, 128, 0, s>>>(t, codes, bounds, bits, q, k, first, count, own, sc.radii2, sc.ids,
+                                                      ctl);
         knn_packet_kernel<kP, kK><<<(unsigned)((count + 32 * kPacketWarps - 1) / (32 * kPacketWarps)), 32 * kPacketWarps, 0,
-                                    s>>>(t.leaves, rec, (int)t.n, start0, q, first, count, sc.radii2, sc.slots, sc.counts,
+                                    s>>>(t.leaves, rec, (int)t.n, start0, q, first, count, sc.radii2, sc.ids, sc.slots, sc.counts,
                                          ctl);
         uint32_t *redo_count = sc.redo_counts + first / sc.chunk;
-        knn_select_kernel<kK><<<blocks, 128, 0, s>>>(q, k, first, count, sc.slots, sc.counts, sc.radii2, sc.redo, redo_count,
+        knn_select_kernel<kK><<<blocks, 128, 0, s>>>(q, k, first, count, sc.slots, sc.counts, sc.radii2, sc.ids, sc.redo, redo_count,
                                                      out_idx, out_d2, ctl);
         knn_redo_kernel<kP, kK><<<(unsigned)std::min<int64_t>((count + 15) / 16, redo_grid), 128, 0,
-                                  s>>>(t.leaves, rec, (int)t.n, start0, q, k, first, count, sc.radii2, sc.redo, redo_count,
+                                  s>>>(t.leaves, rec, (int)t.n, start0, q, k, first, count, sc.radii2, sc.ids, sc.redo, redo_count,
                                        out_idx, out_d2, ctl);
         count_launches(4);
     }

@@ -389,7 +389,8 @@ int64_t knn_chunk(int64_t nq);
 size_t knn_slot_bytes(int k);  // per query of a chunk
 struct KnnScratch {
     int64_t chunk;
-    float *radii2;     // chunk
+    float *radii2;     // chunk: bounds of the k-th key, its squared distance
+    uint32_t *ids;     // chunk: and its index
     uint2 *slots;      // chunk * knn_slot_bytes(k)
     uint32_t *counts;  // chunk
     uint32_t *redo;    // chunk: positions for knn_redo_kernel
