@@ -51,7 +51,7 @@ namespace lbvh {
 
 namespace {
 
-constexpr int kThreads = 256;
+
 constexpr uint32_t kInf = 255;  // above every finite delta* (<= 127)
 
 __device__ __forceinline__ uint32_t delta_star(uint64_t a, uint64_t b, uint32_t pos) {
@@ -300,8 +300,14 @@ struct GroupSmem : MergeSmem {
 // ones 8.1, 12.3 and 15.7 (27 at most of 2,300). What a warp leaves always
 // fits the slots, and 8 groups, or 5 CTAs of a merge, almost always fit a
 // merge's 128 threads (with 256 the construct of 2^25 points took 1.23 ms, not
-// 1.14; with 256 in the second merge alone 1.18). A longer list (chains of leaves with growing gaps) climbs in place and is
-// marked kPendClimbed, and then the merge above climbs too.
+// 1.14; with 256 in the second merge alone 1.18). A longer list (chains of leaves
+// with growing gaps) climbs in place and is marked kPendClimbed, and then the
+// merge above climbs too. Where merges go to the end, its elements stay where
+// they are instead: the last launch has a thread for every place of the lists
+// before, and all that is left climbs there at once. (Where each merge waited for
+// its own climbs, 64 clusters with points down to 1e-5 of their size, construct:
+// 20,000 points 158 us, now 90; 24,000 boxes 168, 88; 7,000 points with 30 bits 93,
+// 54. With all climbing from groups of 256: 98, 98, 51.)
 constexpr int kPendSlots = 32;
 constexpr int kPendCount = 24;  // first bit of the count
 constexpr uint32_t kPendClimbed = 1u << 31;
@@ -398,11 +404,12 @@ __device__ __forceinline__ bool merge_elements(RunTable &table, int m, Element &
 }
 
 // A CTA's elements, consecutive, one per thread (the first `count`): merges
-// them in rounds; what is left goes to the CTA's slots (pend), or climbs.
+// them in rounds; what is left goes to the CTA's slots (pend), or, if it is too
+// much for them, to lists at `back` (room for kGroup elements), or climbs.
 // Every thread of the CTA calls this; the tables' memory is free.
 template <int kKind, bool kPoints, bool kJitter, bool kTrees, typename OwnerOf>
 __device__ __forceinline__ void merge_group(MergeSmem &sm, int count, Element e, const OwnerOf &owner,
-                                            uint32_t *flags, uint4 *pend, const Jitter &jt) {
+                                            uint32_t *flags, uint4 *pend, const Jitter &jt, uint4 *back = nullptr) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     bool keep = false;
     uint32_t kept = 0u;
@@ -458,6 +465,11 @@ __device__ __forceinline__ void merge_group(MergeSmem &sm, int count, Element e,
         return;
     }
     if (pend && threadIdx.x == 0) pend[0] = make_uint4(0u, 0u, kPendClimbed, 0u);
+    if (back) {  // (over kPendSlots elements: the barriers above come after the lists there were cleared)
+        const uint32_t listed = at % kPendSlots == 0 ? (uint32_t)min(left - at, kPendSlots) << kPendCount : 0u;
+        if (keep) back[at] = make_uint4(e.l, e.r, e.gaps | listed, (uint32_t)e.tree);
+        return;
+    }
     // The nodes of this CTA, whichever thread wrote them, are visible to
     // whoever sees this thread's exchange: the barrier orders them before its
     // release.
@@ -503,9 +515,23 @@ struct ManyTrees {
 constexpr int kMergeGroups = 8;
 constexpr int kMergeCtas = 5;
 
+// The lists an earlier merge read.
+struct Lists {
+    uint4 *pend;
+    int64_t count;
+    __host__ __device__ int64_t ctas() const { return (count * kPendSlots + kGroup - 1) / kGroup; }
+};
+constexpr int kEarlier = 2;
+struct EarlierMerges {
+    Lists level[kEarlier];
+};
+
+// merging: the CTAs that merge; those beyond (the last launch of several) climb
+// from what the merges before have left. defer: leave what does not fit.
 template <int kKind, int kFrom, bool kJitter, bool kTrees, typename OwnerOf>
 __global__ void __launch_bounds__(kGroup)
-    merge_pending_kernel(uint4 *pend, int64_t lists, OwnerOf owner, uint32_t *flags, uint4 *out, Jitter jt) {
+    merge_pending_kernel(uint4 *pend, int64_t lists, OwnerOf owner, uint32_t *flags, uint4 *out, Jitter jt, bool defer,
+                         unsigned merging, EarlierMerges earlier) {
     __shared__ MergeSmem sm;
     __shared__ uint32_t s_lists[kFrom];
     group_start(sm, flags);
@@ -541,16 +567,32 @@ __global__ void __launch_bounds__(kGroup)
         load_node_box<kKind>(o.inodes, o.leaves, o.n - 1, id, e.lo, e.hi);
         return e;
     };
+    const auto climb = [&](const Element &e) {
+        const Owner o = owner(e.tree);
+        climb_global<kKind, kJitter>(Climb{e.l, e.r, e.gaps & 0xffu, (e.gaps >> 8) & 0xffu, (e.gaps >> 16) & 0xffu, e.lo, e.hi},
+                                     o.n, o.inodes, o.leaves, o.store, flags, jt);
+    };
+    if (blockIdx.x >= merging) {  // a thread for every place of four of the lists before
+        int64_t b = blockIdx.x - merging;
+        int lv = 0;
+        while (lv + 1 < kEarlier && b >= earlier.level[lv].ctas()) b -= earlier.level[lv++].ctas();
+        const Lists left = earlier.level[lv];
+        uint4 *at = left.pend + b * kGroup;
+        const bool there = b * kGroup / kPendSlots + t / kPendSlots < left.count;
+        const uint32_t listed = there ? (at[t / kPendSlots * kPendSlots].z >> kPendCount) & 127u : 0u;
+        if (t % kPendSlots < (int)listed && !sm.failed) climb(element(at[t]));
+        __syncthreads();
+        if (there && t % kPendSlots == 0) at[t].z = 0u;
+        return;
+    }
+    if (defer && !sm.failed && (missing || count > kGroup)) {
+        if (t == 0) out[0] = make_uint4(0u, 0u, kPendClimbed, 0u);
+        return;
+    }
     if (sm.failed || missing || count > kGroup) {
         // failed: only the counts are cleared; else (some elements missing, or too many) those that are here climb
         if (out && t == 0 && !sm.failed) out[0] = make_uint4(0u, 0u, kPendClimbed, 0u);
-        for (int k = t; k < count && !sm.failed; k += kGroup) {
-            const Element e = element(pend[place(k)]);
-            const Owner o = owner(e.tree);
-            climb_global<kKind, kJitter>(
-                Climb{e.l, e.r, e.gaps & 0xffu, (e.gaps >> 8) & 0xffu, (e.gaps >> 16) & 0xffu, e.lo, e.hi}, o.n,
-                o.inodes, o.leaves, o.store, flags, jt);
-        }
+        for (int k = t; k < count && !sm.failed; k += kGroup) climb(element(pend[place(k)]));
         __syncthreads();
         if (list) pend[t * kPendSlots].z = 0u;
         return;
@@ -559,7 +601,7 @@ __global__ void __launch_bounds__(kGroup)
     if (t < count) e = element(pend[place(t)]);
     __syncthreads();
     if (list) pend[t * kPendSlots].z = 0u;
-    merge_group<kKind, false, kJitter, kTrees>(sm, count, e, owner, flags, out, jt);
+    merge_group<kKind, false, kJitter, kTrees>(sm, count, e, owner, flags, out, jt, defer ? pend : nullptr);
 }
 
 // delta* at the CTA's positions, from sm.code. Thread t holds leaf i of a
@@ -724,11 +766,10 @@ __global__ void __launch_bounds__(kGroup, kGroupCtas)
 
 // How far the merges go before the rest climbs. A merge is a launch of about
 // 6 us that its CTAs' own latency sets, a climb 1-2 us per level of the tree;
-// but where a list is too long, every merge above it waits for its own climbs
-// in turn (64 clusters with points down to 1e-5 of their size, 33,000: 180 us
-// merging to the end, 94 without; 300,000 154, 86). So only small builds merge
-// to the end: 16,500 points, clustered or not, 24.5 us against 29.6 to 36.8
-// (100,000 32.7 against 35 to 43).
+// where a list is too long, what waits for it climbs all the same. So only
+// small builds merge to the end: 16,500 points, clustered or not, 24.5 us
+// against 29.6 to 36.8 (100,000 32.7 against 35 to 43, but the last launch's
+// threads for the lists before grow with the build).
 // Merging again while there are over 4096 CTAs (2^25 points): 1.14 ms, never
 // 1.27, to the end (mixture) 1.48.
 constexpr int64_t kMergeToEnd = 24;
@@ -745,8 +786,12 @@ void launch_merges(int64_t groups, int kind, const OwnerOf &owner, uint32_t *fla
     if (!pend || groups < 2) return;  // one group leaves nothing
     uint4 *in = static_cast<uint4 *>(pend);
     int64_t from = groups;
-    int64_t enough = merge_ctas(groups, true) <= kMergeToEnd ? 1 : kMergeAgain;
+    const bool to_end = merge_ctas(groups, true) <= kMergeToEnd && jt.max_ns == 0;
+    int64_t enough = to_end ? 1 : kMergeAgain;
+    EarlierMerges earlier{};
+    int merges = 0;
     if (jt.max_ns) enough = groups;  // the hook is for climbs: what the first merge leaves climbs
+    static_assert(kMergeToEnd <= kMergeCtas * kMergeCtas, "at most kEarlier merges before the last");
     const bool pts = kind == LBVH_PRIM_POINTS;
     for (bool first = true;; first = false) {
         const int64_t ctas = merge_ctas(from, first);
@@ -763,9 +808,13 @@ void launch_merges(int64_t groups, int kind, const OwnerOf &owner, uint32_t *fla
                          merge_pending_kernel<LBVH_PRIM_POINTS, kMergeCtas, true, kTrees, OwnerOf>,
                          merge_pending_kernel<LBVH_PRIM_BOXES, kMergeCtas, true, kTrees, OwnerOf>);
         }
-        k<<<(unsigned)ctas, kGroup, 0, s>>>(in, from, owner, flags, out, jt);
+        int64_t more = 0;  // what the merges to the end leave climbs in the last one
+        if (!out)
+            for (const Lists &l : earlier.level) more += l.ctas();
+        k<<<(unsigned)(ctas + more), kGroup, 0, s>>>(in, from, owner, flags, out, jt, to_end && out, (unsigned)ctas, earlier);
         count_launches(1);
         if (!out) return;
+        if (to_end) earlier.level[merges++] = Lists{in, from};
         in = out;
         from = ctas;
     }
