@@ -45,7 +45,8 @@ struct Control {
     uint32_t run_heads;            //   runs listed for short_runs_kernel (in this order)
     uint32_t sparse_filled;        // packets left to collect_left_kernel
     uint32_t scan_ticket;          // tiles of the counts' scan
-    uint32_t pad[2];
+    uint32_t rays_apart;           // runs of 32 rays, as given, that do not lie together
+    uint32_t pad[1];
 };
 constexpr int kQueryBufferHits = 64;  // hits kept per query by the walk
 
@@ -103,6 +104,9 @@ struct SortScratch {
     uint32_t *hist;          // kMaxPasses * kRadix global digit counts
     uint32_t *lookback;      // 2 regions of tiles * kRadix words
     int64_t lookback_words;  // words per region
+    // the passes do nothing if *unless < unless_min (null: they always run)
+    const uint32_t *unless = nullptr;
+    uint32_t unless_min = 0;
 };
 
 // Global digit histograms of the first `passes` passes (the stand-alone sort
@@ -243,9 +247,10 @@ void launch_encode(const float *prims, int64_t n, int kind, int bits, const floa
                    uint64_t *codes, uint32_t *hist, int hist_passes, int layout, int index_bits, cudaStream_t s,
                    int skip = 0);
 // Words code << 32 | i of ray segments (8-bit codes, see encode_rays_kernel)
-// and their histogram (hist[0..256) zero beforehand).
+// and their histogram (hist[0..256) zero beforehand); *apart (zero beforehand):
+// the runs of 32 rays that do not lie together.
 void launch_encode_rays(const float *rays, int64_t n, const float *bounds, uint64_t *words, uint32_t *hist,
-                        cudaStream_t s);
+                        uint32_t *apart, cudaStream_t s);
 // codes[i] = the Morton code of primitive perm[i].
 void launch_sorted_codes(const float *prims, const uint32_t *perm, int64_t n, int kind, int bits,
                          const float *bounds, uint64_t *codes, cudaStream_t s);
@@ -304,6 +309,9 @@ struct QueryArgs {
     float radius;
     const uint32_t *order;  // null: thread i walks query i; else query order[i]
     int walk = 0;           // kWalk*: how the collecting walk runs
+    // `order` is as given after all if *apart < apart_min (null: never)
+    const uint32_t *apart = nullptr;
+    uint32_t apart_min = 0;
 };
 // The collecting walk: kWalkThread, the default, is range_walk's choice (leaf
 // blocks, or Algorithm 1 with one thread per query in CTAs of 256); the others

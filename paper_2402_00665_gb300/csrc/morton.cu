@@ -192,26 +192,40 @@ __global__ void __launch_bounds__(kThreads)
 // The walk order of ray segments: word (code << 32 | i) per ray, its code the
 // first 8 bits of the Hilbert index of the cell that holds the segment's
 // middle (a segment longer than the scene is cut to the scene's extent, cells
-// outside the scene to its border), and the histogram of the codes.
+// outside the scene to its border), and the histogram of the codes. *apart
+// counts the runs of 32 rays whose middles are not all within an eighth of the
+// scene from the first one's: where they are few, the order as given is kept.
 __global__ void __launch_bounds__(kThreads)
     encode_rays_kernel(const float4 *__restrict__ rays, int64_t n, const float *__restrict__ bounds,
-                       uint64_t *__restrict__ words, uint32_t *__restrict__ hist) {
-    __shared__ uint32_t s_hist[kRadix];
+                       uint64_t *__restrict__ words, uint32_t *__restrict__ hist, uint32_t *apart) {
+    __shared__ uint32_t s_hist[kRadix], s_apart;
     __shared__ uint16_t s_hilbert[kHilbertEntries];
     s_hist[threadIdx.x] = 0;  // kThreads == kRadix
+    if (threadIdx.x == 0) s_apart = 0;
     load_hilbert(s_hilbert);
     const Grid3 g = make_grid(bounds, 3);
     const float extent = fmaxf(g.extent[0], fmaxf(g.extent[1], g.extent[2]));
+    const int lane = threadIdx.x & 31;
     __syncthreads();
-    for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kThreads) {
+    for (int64_t first = (int64_t)blockIdx.x * kThreads + (threadIdx.x & ~31); first < n;
+         first += (int64_t)gridDim.x * kThreads) {
+        const int64_t i = min(first + lane, n - 1);
         const float4 o = rays[2 * i], d = rays[2 * i + 1];
         const float speed = fmaxf(fabsf(d.x), fmaxf(fabsf(d.y), fabsf(d.z)));
         const float t = o.w + 0.5f * fminf(d.w - o.w, extent / speed);
-        const uint64_t c = hilbert(o.x + t * d.x, o.y + t * d.y, o.z + t * d.z, g, 3, s_hilbert) >> 1;
-        words[i] = c << 32 | (uint64_t)(uint32_t)i;
-        atomicAdd(&s_hist[(uint32_t)c], 1u);
+        const float x = o.x + t * d.x, y = o.y + t * d.y, z = o.z + t * d.z;
+        const float away = fmaxf(fabsf(x - __shfl_sync(0xffffffffu, x, 0)),
+                                 fmaxf(fabsf(y - __shfl_sync(0xffffffffu, y, 0)), fabsf(z - __shfl_sync(0xffffffffu, z, 0))));
+        const bool together = __all_sync(0xffffffffu, away <= 0.125f * extent);
+        if (lane == 0 && !together) atomicAdd(&s_apart, 1u);
+        if (first + lane < n) {
+            const uint64_t c = hilbert(x, y, z, g, 3, s_hilbert) >> 1;
+            words[i] = c << 32 | (uint64_t)(uint32_t)i;
+            atomicAdd(&s_hist[(uint32_t)c], 1u);
+        }
     }
     __syncthreads();
+    if (threadIdx.x == 0 && s_apart) atomicAdd(apart, s_apart);
     const uint32_t v = s_hist[threadIdx.x];
     if (v) atomicAdd(&hist[threadIdx.x], v);
 }
@@ -526,9 +540,9 @@ void launch_encode(const float *prims, int64_t n, int kind, int bits, const floa
 }
 
 void launch_encode_rays(const float *rays, int64_t n, const float *bounds, uint64_t *words, uint32_t *hist,
-                        cudaStream_t s) {
+                        uint32_t *apart, cudaStream_t s) {
     encode_rays_kernel<<<bounds_blocks(n), kThreads, 0, s>>>(reinterpret_cast<const float4 *>(rays), n, bounds, words,
-                                                            hist);
+                                                            hist, apart);
     count_launches(1);
 }
 

@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(kSparseThreads)
     __shared__ uint32_t s_stack[kSparseThreads / 8][kSparseStack];
     const int64_t i = ((int64_t)blockIdx.x * kSparseThreads + threadIdx.x) >> 3;
     const bool has = i < qa.nq, ok = ctl->build_flags == 0;
-    const int64_t qi = has ? thread_query(qa, i) : 0;
+    const int64_t qi = has ? query_at<kQ>(qa, i) : 0;
     typename QueryOf<kQ>::type q{};
     if (has && ok) q = QueryOf<kQ>::load(qa, qi);
     if (has && !ok && (threadIdx.x & 7) == 0) __stcs(qs.counts + qi, 0u);

@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(kThreads, 8)
     if (warp_first >= qa.nq) return;  // whole warps leave together
     const bool has = i < qa.nq;
     const bool walk_ok = t.n > 0 && ctl->build_flags == 0;
-    collect_walk<kQ, kP, kP == LBVH_PRIM_POINTS, kLanes>(t, qa, qs, ctl, i, has ? thread_query(qa, i) : 0, walk_ok,
+    collect_walk<kQ, kP, kP == LBVH_PRIM_POINTS, kLanes>(t, qa, qs, ctl, i, has ? query_at<kQ>(qa, i) : 0, walk_ok,
                                                        has);
 }
 
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kT, 2048 / kT)
     const int64_t i = (int64_t)blockIdx.x * kT + threadIdx.x;
     if (i >= qa.nq) return;
     const bool walk_ok = t.n > 0 && ctl->build_flags == 0;
-    collect_walk<kQ, kP, kP == LBVH_PRIM_POINTS>(t, qa, qs, ctl, i, thread_query(qa, i), walk_ok);
+    collect_walk<kQ, kP, kP == LBVH_PRIM_POINTS>(t, qa, qs, ctl, i, query_at<kQ>(qa, i), walk_ok);
 }
 
 // The queries that packet_kernel left (packets of queries too far apart; list
@@ -902,7 +902,7 @@ __global__ void __launch_bounds__(kThreads)
     const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     uint32_t leaves = 0, internal = 0;
     if (i < qa.nq && t.n > 0 && ctl->build_flags == 0) {
-        const auto q = QueryOf<kQ>::load(qa, thread_query(qa, i));
+        const auto q = QueryOf<kQ>::load(qa, query_at<kQ>(qa, i));
         const int ni = (int)t.n - 1;
         const int nodes = 2 * (int)t.n - 1;
         const uint32_t max_steps = 2u * (uint32_t)nodes;

@@ -159,6 +159,8 @@ struct PassArgs {
     SegArgs seg;
     int64_t hold_tile, prefetch_ahead;
     const uint32_t *count;  // persistent passes: the number of keys, on the device
+    const uint32_t *unless;  // nothing is done if *unless < unless_min
+    uint32_t unless_min;
 };
 
 // kIn / kOut: the layouts above; kHi: the digit byte lies in the key's high
@@ -369,6 +371,7 @@ __global__ void __launch_bounds__(kSortThreads, kMinBlocks) onesweep_kernel(cons
     using Smem = SortSmem<kItems, kIn != kInPacked, kTable>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
+    if (a.unless && __ldcg(a.unless) < a.unless_min) return;
     if (threadIdx.x == 0) {
         const uint32_t t = atomicAdd(a.ticket, 1u);
         if (t == a.tiles - 1) *a.ticket = 0;  // last ticket handed out: reset for the next pass
@@ -625,6 +628,8 @@ void run_pass_list(const Variant &v, const Pass *ps, int passes, int64_t n, cons
         a.seg = sa;
         a.hold_tile = p == 0 ? g_hold_tile.load(std::memory_order_relaxed) : -1;
         a.prefetch_ahead = prefetch_tiles();
+        a.unless = scratch.unless;
+        a.unless_min = scratch.unless_min;
         if (pass_events) cudaEventRecord(pass_events[p][0], s);
         v.k[seg ? 1 : 0][q.kind]<<<(unsigned)tiles, kSortThreads, pass_smem(v, q.kind), s>>>(a);
         if (pass_events) cudaEventRecord(pass_events[p][1], s);

@@ -201,6 +201,12 @@ constexpr int kRegSort = 32;             // lists up to this long are sorted in 
 __device__ __forceinline__ int64_t thread_query(const QueryArgs &qa, int64_t i) {
     return qa.order ? min((int64_t)__ldcs(qa.order + i), qa.nq - 1) : i;
 }
+// The same where the queries may be rays, whose order is not always used.
+template <int kQ>
+__device__ __forceinline__ int64_t query_at(const QueryArgs &qa, int64_t i) {
+    if (kQ == LBVH_Q_RAY && qa.apart && *qa.apart < qa.apart_min) return i;
+    return thread_query(qa, i);
+}
 
 // Hits past a walk's slot: appended to chunks from the shared pool, the first
 // chunk recorded in spill_head[q], each chunk's word 0 linking to the next.
