@@ -11,16 +11,22 @@
 //      positions; +inf (255) at -1 and n-1. Only comparisons are made and no
 //      two compared gaps can share a highest bit, so this order is exact.
 //   2. The leaf's skip (Algorithm 4's leaf lines) and box are written.
-//   3. Climb: the parent's split p is range_right (left child: delta_right <
-//      delta_left) or range_left - 1 (right child). The thread swaps its half
-//      of the parent's description into store[p]. The first arrival reads
-//      "empty" and exits; the second receives the other half, so it now knows
-//      the parent's full range [l, r] and delta*(l-1), delta*(r), delta*(r+1).
-//      It computes the Karras index q = r if delta*(r) < delta*(l-1) else l,
-//      the left child (L_p if l == p else I_p: the children of split p are p
-//      and p+1), the skip (sentinel if r == n-1, else L_{r+1} if delta*(r) <
-//      delta*(r+1), else I_{r+1}), and the box, writes node q, and continues
-//      with i = q until q == 0 (I_0 is the root in Karras' ordering).
+//   3. The nodes, without a climb wherever a warp can see both ends of a node's
+//      range (merge_elements): a group of 128 consecutive leaves, in rounds of
+//      32 elements to a warp, leaves about 7 open, which go to the group's
+//      slots; merge_pending_kernel takes what 8 groups, then 5 of its own CTAs,
+//      have left and merges it the same way (launch_merges says how far).
+//   4. The rest climbs as Algorithm 4 does: a node's split p in its parent is
+//      range_right (left child: delta_right < delta_left) or range_left - 1
+//      (right child). The thread swaps its half of the parent's description
+//      into store[p]. The first arrival reads "empty" and exits; the second
+//      receives the other half, so it now knows the parent's full range [l, r]
+//      and delta*(l-1), delta*(r), delta*(r+1). It computes the Karras index q
+//      = r if delta*(r) < delta*(l-1) else l, the left child (L_p if l == p
+//      else I_p: the children of split p are p and p+1), the skip (sentinel if
+//      r == n-1, else L_{r+1} if delta*(r) < delta*(r+1), else I_{r+1}), and the
+//      box, writes node q, and continues with i = q until q == 0 (I_0 is the
+//      root in Karras' ordering).
 //
 // Differences from the listing, with the same result:
 //   - store[p] carries, besides the range end, the delta* values the other
@@ -32,14 +38,10 @@
 //     (it is zeroed once, when allocated).
 //   - release/acquire: the exchange is an acq_rel atomic, so a thread's node
 //     is visible before its half of the parent is, and the second thread
-//     reads the sibling's box only after it has seen that half.
-//   - inside a group of 256 consecutive leaves nobody climbs: the nodes whose
-//     range lies in the group are formed from the delta* values side by side
-//     (merge_elements, one warp to 32 leaves, then 32 of what is left); only
-//     the nodes spanning a group's edge meet in the `store` words (sibling
-//     box through L2, ld.global.cg). Batches group their global sorted
-//     positions the same way (a group may hold several trees; a split only
-//     ever joins leaves of one).
+//     reads the sibling's box (through L2, ld.global.cg) only after it has
+//     seen that half.
+//   - batches group their global sorted positions the same way (a group may
+//     hold several trees; a split only ever joins leaves of one).
 #include <atomic>
 
 #include <cuda/atomic>
@@ -50,7 +52,6 @@
 namespace lbvh {
 
 namespace {
-
 
 constexpr uint32_t kInf = 255;  // above every finite delta* (<= 127)
 

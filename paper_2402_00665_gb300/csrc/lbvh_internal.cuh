@@ -281,8 +281,8 @@ void launch_variant_second(int algorithm, const uint64_t *codes, const uint32_t 
                            int64_t n, int kind, float4 *inodes, float4 *leaves, void *scratch,
                            unsigned long long *store, uint32_t *flags, cudaStream_t s);
 // pend (nullable): construct_pend_bytes(n) of zeroed scratch, left zeroed.
-// With it, what a CTA's group of leaves leaves over is merged by a second
-// kernel; without it (the no-allocation entry point) it climbs in place.
+// With it, what a CTA's group of leaves leaves over is merged by further
+// launches; without it (the no-allocation entry point) it climbs in place.
 size_t construct_pend_bytes(int64_t n);
 void launch_construct(const uint64_t *sorted_codes, const uint32_t *perm, const float *prims,
                       int64_t n, int kind, float4 *inodes, float4 *leaves,
