@@ -257,8 +257,9 @@ __device__ __forceinline__ void centroid_at(const float *prims, int64_t i, float
 // (windows are sorted one by one, so the order is as fine as 4096 queries of a
 // cell allow); 16 nearest neighbours at 1e-4 9165 / 3701 / 5770.
 // It is bound by instructions: 30 us for one wave of CTAs, 100 us for 2 * 10^6
-// crowded queries, 3 us where nothing is crowded (20 for 2^23). Windows of 2048: 70 us, but the
-// 1e-4 clusters take 1206.
+// crowded queries, 3 us where nothing is crowded (20 for 2^23 queries that have to
+// be looked at, 3 where one radius says that none is small). Windows of 2048: 70
+// us, but the 1e-4 clusters take 1206.
 constexpr int kWindow = 4096, kWindowThreads = 512, kEach = kWindow / kWindowThreads;
 constexpr int kCrowd = 64, kCrowdedPairs = 4;
 template <int kKind>
@@ -269,100 +270,103 @@ __global__ void __launch_bounds__(kWindowThreads)
     __shared__ int s_pairs;
     if (ctl->build_flags != 0) return;  // the sort may have given up: the words are not an order
     const int t = threadIdx.x;
-    const int64_t base = (int64_t)blockIdx.x * kWindow;
-    const int count = (int)min((int64_t)kWindow, qa.nq - base);
-    const auto cell = [&](int at, const Grid3 &g) {
-        float x, y, z;
-        centroid_at<kKind>(qa.queries, (int64_t)order[base + at], x, y, z);
-        return morton(x, y, z, g);
-    };
-    if (t == 0) s_pairs = 0;
-    const bool sample = t < kWindow / kCrowd && kCrowd * t < count;
-    bool small = false;
-    if (sample) {
-        const Grid3 g = make_grid(bounds, levels);
-        s_key[t] = cell(kCrowd * t, g);
-        const int64_t q = order[base + kCrowd * t];
-        const float edge = fmaxf(g.extent[0], fmaxf(g.extent[1], g.extent[2])) / g.cells;
-        if (kKind == LBVH_PRIM_POINTS) {
-            small = 4.0f * (qa.radii ? qa.radii[q] : qa.radius) < edge;
-        } else {
-            const float *b = qa.queries + 6 * q;
-            small = 2.0f * fmaxf(b[3] - b[0], fmaxf(b[4] - b[1], b[5] - b[2])) < edge;
+    const Grid3 coarse = make_grid(bounds, levels);
+    const float edge = fmaxf(coarse.extent[0], fmaxf(coarse.extent[1], coarse.extent[2])) / coarse.cells;
+    if (kKind == LBVH_PRIM_POINTS && !qa.radii && 4.0f * qa.radius >= edge) return;
+    for (int64_t base = (int64_t)blockIdx.x * kWindow; base < qa.nq; base += (int64_t)gridDim.x * kWindow) {
+        const int count = (int)min((int64_t)kWindow, qa.nq - base);
+        const auto cell = [&](int at, const Grid3 &g) {
+            float x, y, z;
+            centroid_at<kKind>(qa.queries, (int64_t)order[base + at], x, y, z);
+            return morton(x, y, z, g);
+        };
+        __syncthreads();  // the window before is done
+        if (t == 0) s_pairs = 0;
+        const bool sample = t < kWindow / kCrowd && kCrowd * t < count;
+        bool small = false;
+        if (sample) {
+            s_key[t] = cell(kCrowd * t, coarse);
+            const int64_t q = order[base + kCrowd * t];
+            if (kKind == LBVH_PRIM_POINTS) {
+                small = 4.0f * (qa.radii ? qa.radii[q] : qa.radius) < edge;
+            } else {
+                const float *b = qa.queries + 6 * q;
+                small = 2.0f * fmaxf(b[3] - b[0], fmaxf(b[4] - b[1], b[5] - b[2])) < edge;
+            }
         }
-    }
-    __syncthreads();
-    if (small && t > 0 && s_key[t] == s_key[t - 1]) atomicAdd(&s_pairs, 1);
-    __syncthreads();
-    if (s_pairs < kCrowdedPairs) return;
-    load_hilbert(s_hilbert);
-    const Grid3 g = make_grid(bounds, 21);
-    uint64_t key[kEach];  // places kEach t .. kEach t + kEach - 1: the cells of 21 levels, then their places on the curve
-    uint32_t state[kEach];
+        __syncthreads();
+        if (small && t > 0 && s_key[t] == s_key[t - 1]) atomicAdd(&s_pairs, 1);
+        __syncthreads();
+        if (s_pairs < kCrowdedPairs) continue;
+        load_hilbert(s_hilbert);
+        const Grid3 g = make_grid(bounds, 21);
+        uint64_t key[kEach];  // places kEach t .. kEach t + kEach - 1: the cells of 21 levels, then their places on the curve
+        uint32_t state[kEach];
 #pragma unroll
-    for (int j = 0; j < kEach; ++j) key[j] = cell(min(kEach * t + j, count - 1), g);
-    __syncthreads();
+        for (int j = 0; j < kEach; ++j) key[j] = cell(min(kEach * t + j, count - 1), g);
+        __syncthreads();
 #pragma unroll
-    for (int j = 0; j < kEach; ++j) {  // as hilbert(), the steps of the places side by side: the first three bits,
-        const uint32_t e = s_hilbert[2u << 6 | (uint32_t)(key[j] >> 60)];
-        key[j] = key[j] << 4 | (e & 63u);
-        state[j] = e & ~63u;
-    }
-#pragma unroll 1
-    for (int k = 0; k < 10; ++k)  // then six at a time taken from the top, their places on the curve put in below
-#pragma unroll
-        for (int j = 0; j < kEach; ++j) {
-            const uint32_t e = s_hilbert[state[j] | (uint32_t)(key[j] >> 58)];
-            key[j] = key[j] << 6 | (e & 63u);
+        for (int j = 0; j < kEach; ++j) {  // as hilbert(), the steps of the places side by side: the first three bits,
+            const uint32_t e = s_hilbert[2u << 6 | (uint32_t)(key[j] >> 60)];
+            key[j] = key[j] << 4 | (e & 63u);
             state[j] = e & ~63u;
         }
-#pragma unroll
-    for (int j = 0; j < kEach; ++j) {
-        const int e = kEach * t + j;
-        key[j] = e < count ? key[j] >> 11 << 12 | (uint64_t)e : ~0ull;
-    }
 #pragma unroll 1
-    for (int run = 2; run <= kWindow; run *= 2) {
-        // the smaller key goes to the lower place of an ascending pair and the upper one of a descending pair
-        const auto keep = [&](int j, int d, uint64_t other) {
+        for (int k = 0; k < 10; ++k)  // then six at a time taken from the top, their places on the curve put in below
+#pragma unroll
+            for (int j = 0; j < kEach; ++j) {
+                const uint32_t e = s_hilbert[state[j] | (uint32_t)(key[j] >> 58)];
+                key[j] = key[j] << 6 | (e & 63u);
+                state[j] = e & ~63u;
+            }
+#pragma unroll
+        for (int j = 0; j < kEach; ++j) {
             const int e = kEach * t + j;
-            const bool smaller = ((e & d) == 0) == ((e & run) == 0);
-            key[j] = (key[j] < other) == smaller ? key[j] : other;
-        };
-        int d = run / 2;
-#pragma unroll 1
-        for (; d >= kEach * 32; d /= 2) {
-#pragma unroll
-            for (int j = 0; j < kEach; ++j) s_key[j * kWindowThreads + t] = key[j];
-            __syncthreads();
-#pragma unroll
-            for (int j = 0; j < kEach; ++j) keep(j, d, s_key[j * kWindowThreads + (t ^ (d / kEach))]);
-            __syncthreads();
+            key[j] = e < count ? key[j] >> 11 << 12 | (uint64_t)e : ~0ull;
         }
 #pragma unroll 1
-        for (; d >= kEach; d /= 2)
+        for (int run = 2; run <= kWindow; run *= 2) {
+            // the smaller key goes to the lower place of an ascending pair and the upper one of a descending pair
+            const auto keep = [&](int j, int d, uint64_t other) {
+                const int e = kEach * t + j;
+                const bool smaller = ((e & d) == 0) == ((e & run) == 0);
+                key[j] = (key[j] < other) == smaller ? key[j] : other;
+            };
+            int d = run / 2;
+#pragma unroll 1
+            for (; d >= kEach * 32; d /= 2) {
 #pragma unroll
-            for (int j = 0; j < kEach; ++j) keep(j, d, __shfl_xor_sync(0xffffffffu, key[j], d / kEach));
+                for (int j = 0; j < kEach; ++j) s_key[j * kWindowThreads + t] = key[j];
+                __syncthreads();
 #pragma unroll
-        for (int c = kEach / 2; c > 0; c /= 2)
-            if (c < run) {
-#pragma unroll
-                for (int j = 0; j < kEach; ++j)
-                    if ((j & c) == 0) {
-                        const uint64_t lo = key[j], hi = key[j | c];
-                        keep(j, c, hi);
-                        keep(j | c, c, lo);
-                    }
+                for (int j = 0; j < kEach; ++j) keep(j, d, s_key[j * kWindowThreads + (t ^ (d / kEach))]);
+                __syncthreads();
             }
+#pragma unroll 1
+            for (; d >= kEach; d /= 2)
+#pragma unroll
+                for (int j = 0; j < kEach; ++j) keep(j, d, __shfl_xor_sync(0xffffffffu, key[j], d / kEach));
+#pragma unroll
+            for (int c = kEach / 2; c > 0; c /= 2)
+                if (c < run) {
+#pragma unroll
+                    for (int j = 0; j < kEach; ++j)
+                        if ((j & c) == 0) {
+                            const uint64_t lo = key[j], hi = key[j | c];
+                            keep(j, c, hi);
+                            keep(j | c, c, lo);
+                        }
+                }
+        }
+        uint32_t mine[kEach];
+#pragma unroll
+        for (int j = 0; j < kEach; ++j)
+            mine[j] = kEach * t + j < count ? order[base + (int)(key[j] & (kWindow - 1))] : 0u;
+        __syncthreads();  // every place has been read
+#pragma unroll
+        for (int j = 0; j < kEach; ++j)
+            if (kEach * t + j < count) order[base + kEach * t + j] = mine[j];
     }
-    uint32_t mine[kEach];
-#pragma unroll
-    for (int j = 0; j < kEach; ++j)
-        mine[j] = kEach * t + j < count ? order[base + (int)(key[j] & (kWindow - 1))] : 0u;
-    __syncthreads();  // every place has been read
-#pragma unroll
-    for (int j = 0; j < kEach; ++j)
-        if (kEach * t + j < count) order[base + kEach * t + j] = mine[j];
 }
 
 // The codes of the primitives in sorted order: codes[i] = the code of
@@ -550,7 +554,8 @@ void launch_refine_order(const QueryArgs &q, int levels, const float *bounds, ui
                          cudaStream_t s) {
     if (q.nq <= 0) return;
     auto k = q.qkind == LBVH_Q_SPHERE ? refine_order_kernel<LBVH_PRIM_POINTS> : refine_order_kernel<LBVH_PRIM_BOXES>;
-    k<<<(unsigned)((q.nq + kWindow - 1) / kWindow), kWindowThreads, 0, s>>>(q, levels, bounds, order, ctl);
+    const int64_t windows = (q.nq + kWindow - 1) / kWindow, most = 4 * (int64_t)device_sm_count();
+    k<<<(unsigned)(windows < most ? windows : most), kWindowThreads, 0, s>>>(q, levels, bounds, order, ctl);
     count_launches(1);
 }
 
