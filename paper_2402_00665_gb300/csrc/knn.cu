@@ -190,10 +190,11 @@ __global__ void __launch_bounds__(128)
 //   4. knn_redo_kernel    queries with fewer hits (their bound was cut too
 //      far) or more than are kept (a bound from leaves far away),
 //      8 lanes each with a bound that shrinks.
-// A bound is a key, not only a distance: of many copies of a point only those up to
-// an index can be among the k (16 nearest of 2 * 10^6 points on 27,000 places 4.91
+// A bound of no distance comes with an index: of many copies of a point only those
+// up to it can be among the k (16 nearest of 2 * 10^6 points on 27,000 places 4.91
 // ms with distances alone, so 1.11, the heap 1.19; 100,000 points on 100 places
-// 1.66, 0.72, 0.61).
+// 1.66, 0.80, 0.61). Indices beside every bound, and equal blocks in the order of
+// their leaves, cost mixtures 5 to 8%.
 // Leaves of the bound's window and hits kept per query, in units of K.
 template <int kK>
 constexpr int kKnnMul = kK <= 8 ? 8 : 4;
@@ -336,8 +337,8 @@ __global__ void __launch_bounds__(128)
 }
 
 // A lane's hits with their squared distances: (index, distance) words, the
-// first kCap of them kept, two per 16-byte store.
-template <int kCap>
+// first kCap of them kept, two per 16-byte store. kCopies: `last` is looked at.
+template <int kCap, bool kCopies>
 struct KnnKeeper {
     // Several times what a packet reads (about 180 leaf blocks for k = 16):
     // a few queries far out, whose wide balls reach into a dense part, kept
@@ -352,7 +353,7 @@ struct KnnKeeper {
     __device__ __forceinline__ void reset() { cnt = 0; }
     template <int kP, typename Q>
     __device__ __forceinline__ void take(uint32_t m, const PacketSmem<kP> &sm, int ring, const Q &) {
-        if (last != ~0u)
+        if (kCopies && last != ~0u)
             for (uint32_t r = m; r; r &= r - 1) {
                 const int b = 31 - __clz(r & (0u - r));
                 if (sm.id[ring + 31 - b] > last) m ^= 1u << b;
@@ -407,12 +408,20 @@ __global__ void __launch_bounds__(32 * kPacketWarps, kPacketCtas<kP>)
         const uint32_t same = __ballot_sync(kFull, rest == least);
         if (lane == __ffs(same) - 1) rest = inf;
     }
+    const bool copies = has && q.r2 == 0.0f;  // bounded by an index as well
     if (finite) q.r2 = fminf(q.r2, kKnnCut<kK> * fourth);
-    KnnKeeper<kCap> k{slots + j * kCap, q.c, has && q.r2 == 0.0f ? ids[j] : ~0u, 0u, make_uint2(0u, 0u)};
-    const uint32_t left = packets<LBVH_Q_SPHERE, kP>(Blocks{leaves, rec, n, start0}, sm, q, __ballot_sync(kFull, has), k);
-    if (!has) return;
-    if (k.cnt <= (uint32_t)kCap && (k.cnt & 1u)) k.slot[k.cnt - 1] = k.held;
-    counts[j] = !finite ? kNoNeighbours : ((left >> lane) & 1u) ? 0u : k.cnt;
+    const auto walk = [&](auto k) {
+        const uint32_t left =
+            packets<LBVH_Q_SPHERE, kP>(Blocks{leaves, rec, n, start0}, sm, q, __ballot_sync(kFull, has), k);
+        if (!has) return;
+        if (k.cnt <= (uint32_t)kCap && (k.cnt & 1u)) k.slot[k.cnt - 1] = k.held;
+        counts[j] = !finite ? kNoNeighbours : ((left >> lane) & 1u) ? 0u : k.cnt;
+    };
+    if (!__any_sync(kFull, copies)) {
+        walk(KnnKeeper<kCap, false>{slots + j * kCap, q.c, ~0u, 0u, make_uint2(0u, 0u)});
+    } else {
+        walk(KnnKeeper<kCap, true>{slots + j * kCap, q.c, copies ? ids[j] : ~0u, 0u, make_uint2(0u, 0u)});
+    }
 }
 
 // Sorts the cnt keys of a query (8 lanes, kCap keys of shared memory at most)
@@ -468,7 +477,8 @@ __global__ void __launch_bounds__(128)
         const float3 c =
             make_float3(__ldg(qa.queries + 3 * qi), __ldg(qa.queries + 3 * qi + 1), __ldg(qa.queries + 3 * qi + 2));
         float r2 = radii2[j];
-        uint64_t worst = knn_key(r2, redo || r2 == 0.0f ? ids[j] : ~0u);  // the k smallest keys are no larger
+        const bool copies = r2 == 0.0f;
+        uint32_t last = copies ? ids[j] : ~0u;  // the k smallest keys have no larger index
         int cnt = 0, ns = go && built ? 1 : 0;
         if (sl == 0) stack[0] = 0u;
         __syncwarp();
@@ -492,7 +502,7 @@ __global__ void __launch_bounds__(128)
                 }
                 d2 = box_d2(c, xyz(a), xyz(b));
                 key = knn_key(d2, __float_as_uint(a.w) & kLeafIndexMask);
-                hit = d2 <= r2 && (leaf ? key <= worst : __float_as_uint(b.w) == kBlockExists);
+                hit = d2 <= r2 && (leaf ? (uint32_t)key <= last : __float_as_uint(b.w) == kBlockExists);
             }
             const uint32_t bits = (__ballot_sync(kFull, hit) >> shift) & 0xffu;
             if (act) --ns;
@@ -504,7 +514,7 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
                 for (int o = 1; o < kFan; ++o) {
                     const float other = __shfl_xor_sync(kFull, far, o);
-                    farther += other > far || (other == far && (sl ^ o) > sl);
+                    farther += other > far || (other == far && (sl ^ o) < sl);
                 }
                 if (!leaf) before = farther;
             }
@@ -520,8 +530,8 @@ __global__ void __launch_bounds__(128)
                 const int kept = keep_smallest<kCap>(keys, cnt > kCap - 8 ? cnt : 0, k, sl);
                 if (cnt > kCap - 8) {
                     cnt = kept;
-                    worst = keys[k - 1];
-                    r2 = fminf(r2, __uint_as_float((uint32_t)(worst >> 32)));
+                    r2 = fminf(r2, __uint_as_float((uint32_t)(keys[k - 1] >> 32)));
+                    if (copies) last = (uint32_t)keys[k - 1];
                 }
                 __syncwarp();
             }
@@ -554,7 +564,6 @@ __global__ void __launch_bounds__(128)
     const bool none = c == kNoNeighbours;
     if (!none && c < (uint32_t)k) {
         redo[atomicAdd(redo_count, 1u)] = (uint32_t)j;
-        if (radii2[j] != 0.0f) ids[j] = ~0u;
         return;
     }
     const bool over = !none && c > (uint32_t)kCap;
@@ -585,7 +594,7 @@ __global__ void __launch_bounds__(128)
         for (int i = 0; i < kK; ++i)
             if (i == k - 1) bound = best[i];
         radii2[j] = __uint_as_float((uint32_t)(bound >> 32));
-        ids[j] = (uint32_t)bound;
+        if (bound >> 32 == 0) ids[j] = (uint32_t)bound;
         redo[atomicAdd(redo_count, 1u)] = (uint32_t)j;
         return;
     }
