@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(128)
             make_float3(__ldg(qa.queries + 3 * qi), __ldg(qa.queries + 3 * qi + 1), __ldg(qa.queries + 3 * qi + 2));
         float r2 = radii2[j];
         const bool copies = r2 == 0.0f;
-        uint32_t last = copies ? ids[j] : ~0u;  // the k smallest keys have no larger index
+        const uint32_t last = copies ? ids[j] : ~0u;  // the k smallest keys have no larger index
         int cnt = 0, ns = go && built ? 1 : 0;
         if (sl == 0) stack[0] = 0u;
         __syncwarp();
@@ -501,8 +501,9 @@ __global__ void __launch_bounds__(128)
                     if (!leaf) b = __ldg(p + 1);
                 }
                 d2 = box_d2(c, xyz(a), xyz(b));
+                hit = d2 <= r2 && (leaf || __float_as_uint(b.w) == kBlockExists);
                 key = knn_key(d2, __float_as_uint(a.w) & kLeafIndexMask);
-                hit = d2 <= r2 && (leaf ? (uint32_t)key <= last : __float_as_uint(b.w) == kBlockExists);
+                if (copies && leaf && (uint32_t)key > last) hit = false;
             }
             const uint32_t bits = (__ballot_sync(kFull, hit) >> shift) & 0xffu;
             if (act) --ns;
@@ -531,7 +532,6 @@ __global__ void __launch_bounds__(128)
                 if (cnt > kCap - 8) {
                     cnt = kept;
                     r2 = fminf(r2, __uint_as_float((uint32_t)(keys[k - 1] >> 32)));
-                    if (copies) last = (uint32_t)keys[k - 1];
                 }
                 __syncwarp();
             }
