@@ -283,7 +283,7 @@ lbvh_status lbvh_tree_walk_visits(lbvh_tree_t tree, const float *d_queries, int6
  *              query with a non-finite coordinate has no neighbours.
  *   d_dist2    float[nq][k] out or NULL: the squared distances, +inf padding.
  * Buffers are the caller's. Synchronises `stream` once (for the status).
- * Beside the order of the queries (36 bytes each) the tree holds scratch for
+ * Beside the order of the queries (40 bytes each) the tree holds scratch for
  * 5 <= k <= 32: 512 bytes for each of up to 2^20 queries at a time (1 KB for
  * k > 16), kept for later queries, and 4.6 bytes per primitive for the boxes
  * of leaf blocks. Where these cannot be had the call runs without them,
